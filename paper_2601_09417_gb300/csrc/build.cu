@@ -6,16 +6,20 @@
 // thread per output coefficient (9- and 7-tap filters from constant memory;
 // neighbouring threads read neighbouring inputs, so the taps hit L1/L2).
 //
-// Selection per subband, all on the device except the budget allocation
-// (one copy of the 7J+1 subband energies to the host):
+// Selection, all on the device and over every subband in the same launches:
 //   v = sqrt(((a0 a0 + a1 a1) + a2 a2) + a3 a3) in IEEE float32, rounded op by
 //   op (explicit __fmul_rn/__fadd_rn/__fsqrt_rn, so the order is fixed);
-//   medians and the K-th largest value by radix select on the float bits (v >= 0
-//   so the bits order like the values): four 8-bit histogram passes, no sort;
+//   the medians and the K-th largest value by radix select on the float bits (v >= 0
+//   so the bits order like the values): three passes of 10 or 11 bits, no sort;
 //   sigma = MAD / 0.6745 and T = lambda sigma in float32;
 //   keep = v >= max(T, v_(K')) and v > 0.
-// Kept coefficients are compacted in raster order of each subband by a
-// block scan and mapped to the P[14][capacity] layout.
+// Kept coefficients are marked in a bit mask (raster order of each subband),
+// whose counts are scanned, and mapped chunk by chunk to the P[14][capacity]
+// layout.  The host waits once, for the number kept.  One launch a pass over
+// all bands (10 launches) instead of about 50 a band, and a map over the whole
+// chip instead of one block a band (which took 350 ms on a 512^3 volume):
+// vbm_build of 32^3 / 224 x 160 x 96 / 512^3 volumes 5.5 -> 0.33, 18.8 -> 1.38,
+// 390 -> 36.3 ms, the rest mostly the DWT.
 #include <cmath>
 #include <map>
 #include <vector>
@@ -93,170 +97,378 @@ __global__ void k_dwt_axis(const float *__restrict__ src, float *__restrict__ ds
 
 // ----------------------------------------------------------------- select
 
-struct SubStat {
-    float med, mad, T, thr;
-    float sel_a, sel_b;          // scratch of the two order statistics of a median
-    int64_t count_c;             // |C|
-    int64_t k;                   // rank of the running selection
-    uint32_t prefix, mask;
-    int64_t kept;
+constexpr int kMaxBands = 64;            // 7 J + 1 with J <= 9
+constexpr int kSelThreads = 1024;
+constexpr int kTargets = 3;              // lower median rank, upper median rank, K-th largest
+constexpr int kBins = 2048;              // bins of the widest digit
+constexpr int kChunk = 8192;             // elements of one marking / mapping block
+constexpr int kMarkThreads = 256;
+
+struct Band {
+    int j, o[3], ox, oy, oz, mx, my, mz;
+    int64_t n;
 };
 
-__global__ void k_energy(const float *__restrict__ A, int nx, int ny, int ox, int oy, int oz, int mx, int my, int mz,
-                         double *__restrict__ E)
+// Where the subbands lie: element i (raster order) of band b is word voff[b] +
+// i of the magnitude array (each band padded to whole 32-bit mask words), and
+// pyramid element (oz + z, oy + y, ox + x).  chunk0 and blk0 are the first
+// marking chunk and the first selection block of a band ([nb]: the totals).
+struct BandTab {
+    int nb;
+    int ox[kMaxBands], oy[kMaxBands], oz[kMaxBands], mx[kMaxBands], my[kMaxBands];
+    int64_t n[kMaxBands], voff[kMaxBands];
+    int chunk0[kMaxBands + 1], blk0[kMaxBands + 1];
+};
+
+// Budget of Supp. Sec. 1.1, evaluated on the device from the band energies.
+struct Budget {
+    double alpha_E, beta_N, K_tot;
+    int64_t min_per_band;
+    float lambda;
+};
+
+// Running selections of one band.  rank: what is left of each target's rank
+// inside its prefix; prefix: the digits found so far.
+struct SubState {
+    unsigned long long zeros[2];         // exact zeros among the magnitudes / the deviations
+    long long rank[kTargets];
+    uint32_t prefix[kTargets];
+    uint32_t ticket;                     // blocks of the running pass that are done (wraps to 0)
+    int none;                            // the budget is 0: nothing is kept
+    float med, vk, thr;
+};
+
+__device__ __forceinline__ int band_of(const int *first, int nb, int blk)
 {
-    __shared__ double red[256];
-    const int64_t total = (int64_t)mx * my * mz;
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % mx), y = (int)((i / mx) % my), z = (int)(i / ((int64_t)mx * my));
-        const double a = A[((int64_t)(oz + z) * ny + (oy + y)) * nx + (ox + x)];
-        s += a * a;
-    }
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int off = blockDim.x / 2; off > 0; off >>= 1) {
-        if (threadIdx.x < (unsigned)off) red[threadIdx.x] += red[threadIdx.x + off];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) atomicAdd(E, red[0]);
+    int b = 0;
+    while (b < nb - 1 && blk >= first[b + 1]) b++;
+    return b;
 }
 
-__global__ void k_joint_mag(const float *__restrict__ A, int64_t chan, int nx, int ny, int ox, int oy, int oz, int mx,
-                            int my, int mz, float *__restrict__ v)
+// Pyramid element of band element i.
+__device__ __forceinline__ int64_t pyramid_index(const BandTab &t, int b, int64_t i, int nx, int ny, int &x, int &y,
+                                                 int &z)
 {
-    const int64_t total = (int64_t)mx * my * mz;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % mx), y = (int)((i / mx) % my), z = (int)(i / ((int64_t)mx * my));
-        const int64_t e = ((int64_t)(oz + z) * ny + (oy + y)) * nx + (ox + x);
+    const int64_t row = t.n[b] <= INT_MAX ? (int64_t)((uint32_t)i / (uint32_t)t.mx[b]) : i / t.mx[b];
+    x = (int)(i - row * t.mx[b]);
+    z = t.n[b] <= INT_MAX ? (int)((uint32_t)row / (uint32_t)t.my[b]) : (int)(row / t.my[b]);
+    y = (int)(row - (int64_t)z * t.my[b]);
+    return ((int64_t)(t.oz[b] + z) * ny + (t.oy[b] + y)) * nx + (t.ox[b] + x);
+}
+
+// Joint magnitudes of every band, and the bands' opacity energies in double.
+__global__ void __launch_bounds__(kMarkThreads) k_joint_mag(const float *__restrict__ A, int64_t chan, int nx, int ny,
+                                                            const __grid_constant__ BandTab t, float *__restrict__ v,
+                                                            double *__restrict__ E)
+{
+    const int b = band_of(t.chunk0, t.nb, blockIdx.x);
+    const int64_t i0 = (int64_t)(blockIdx.x - t.chunk0[b]) * kChunk;
+    const int64_t i1 = min(t.n[b], i0 + kChunk);
+    double s = 0.0;
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += kMarkThreads) {
+        int x, y, z;
+        const int64_t e = pyramid_index(t, b, i, nx, ny, x, y, z);
         const float a0 = A[e], a1 = A[chan + e], a2 = A[2 * chan + e], a3 = A[3 * chan + e];
         float acc = __fmul_rn(a0, a0);
         acc = __fadd_rn(acc, __fmul_rn(a1, a1));
         acc = __fadd_rn(acc, __fmul_rn(a2, a2));
         acc = __fadd_rn(acc, __fmul_rn(a3, a3));
-        v[i] = __fsqrt_rn(acc);
+        v[t.voff[b] + i] = __fsqrt_rn(acc);
+        s += (double)a3 * (double)a3;
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    __shared__ double red[kMarkThreads / 32];
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kMarkThreads / 32; w++) s += red[w];
+        atomicAdd(E + b, s);
     }
 }
 
-__global__ void k_abs_dev(const float *__restrict__ v, int64_t n, const SubStat *__restrict__ st,
-                          float *__restrict__ dev)
+// Exclusive block scan of one count per thread; `total` is the block's sum.
+template <int THREADS>
+__device__ __forceinline__ uint32_t block_scan(uint32_t c, uint32_t *warp_sum, uint32_t &total)
 {
-    const float med = st->med;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        dev[i] = fabsf(__fsub_rn(v[i], med));
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t incl = c;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += y;
+    }
+    __syncthreads();                     // the last user of warp_sum is done
+    if (lane == 31) warp_sum[w] = incl;
+    __syncthreads();
+    uint32_t base = 0;
+    total = 0;
+#pragma unroll
+    for (int k = 0; k < THREADS / 32; k++) {
+        const uint32_t ws = warp_sum[k];
+        base += k < w ? ws : 0u;
+        total += ws;
+    }
+    return base + incl - c;
 }
 
-// radix select: histogram of the digit at `shift` among elements matching the prefix
-__global__ void k_sel_hist(const float *__restrict__ v, int64_t n, const SubStat *__restrict__ st, int shift,
-                           uint32_t *__restrict__ hist)
+// The three digits of a selection on the float bits (v >= 0, so the sign bit
+// is 0 and the bits order like the values): bits 30-21, 20-10 and 9-0.
+template <int DIGIT>
+struct Digit {
+    static constexpr int shift = DIGIT == 0 ? 21 : DIGIT == 1 ? 10 : 0;
+    static constexpr int bits = DIGIT == 1 ? 11 : 10;
+};
+
+// One radix-select pass over every band at once: digit DIGIT of the magnitudes
+// (DEV = false: both median ranks and the K-th largest in the same pass) or of
+// their absolute deviations from the median (DEV = true: both median ranks),
+// which are formed on the fly.  A block counts one band's digits in shared
+// memory and adds them to the band's histogram; the band's last block picks
+// the digits, clears the histogram for the next pass and, after the third
+// digit, forms the median (the mean of the two middle values of an even
+// count) or the threshold.
+//
+// Bound by reading the magnitudes (4 bytes an element a pass).  Wide digits
+// keep the passes at three a selection; the first digit (sign-free exponent
+// and two mantissa bits) falls into few bins, so its counts are kept in eight
+// copies, one per lane mod 8, and exact zeros (empty space: often most of a
+// volume) are counted in registers and left out of every histogram.
+template <int DIGIT, bool DEV>
+__global__ void __launch_bounds__(kSelThreads) k_select_pass(const float *__restrict__ v,
+                                                             const __grid_constant__ BandTab t,
+                                                             const __grid_constant__ Budget bud,
+                                                             const double *__restrict__ E, SubState *__restrict__ st,
+                                                             uint32_t *__restrict__ hist)
 {
-    __shared__ uint32_t h[256];
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) h[i] = 0;
+    using D = Digit<DIGIT>;
+    constexpr int NB = 1 << D::bits;
+    constexpr int NT = DIGIT == 0 ? 1 : DEV ? 2 : 3;             // histograms
+    constexpr int COPIES = DIGIT == 0 ? 8 : 1;
+    __shared__ uint32_t h[NT * NB * COPIES];
+    __shared__ uint32_t warp_sum[kSelThreads / 32];
+    __shared__ double share[kMaxBands];
+    __shared__ uint32_t s_last, s_digit;
+    __shared__ long long s_rank;
+    const int tid = threadIdx.x;
+    const int b = band_of(t.blk0, t.nb, blockIdx.x);
+    SubState *sb = st + b;
+    uint32_t *gh = hist + (int64_t)b * kTargets * kBins;
+    for (int i = tid; i < NT * NB * COPIES; i += kSelThreads) h[i] = 0;
     __syncthreads();
-    const uint32_t prefix = st->prefix, mask = st->mask;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t b = __float_as_uint(v[i]);
-        if ((b & mask) == prefix) atomicAdd(&h[(b >> shift) & 255u], 1u);
+    const uint32_t p0 = sb->prefix[0], p1 = sb->prefix[1], p2 = sb->prefix[2];
+    const float med = DEV ? sb->med : 0.f;
+    uint32_t zeros = 0;
+    auto count = [&](float val) {
+        const float x = DEV ? fabsf(__fsub_rn(val, med)) : val;
+        const uint32_t bits = __float_as_uint(x);
+        if (bits == 0) {
+            zeros++;
+            return;
+        }
+        const uint32_t d = (bits >> D::shift) & (NB - 1);
+        if constexpr (DIGIT == 0) {
+            atomicAdd(&h[d * COPIES + (tid & (COPIES - 1))], 1u);
+        } else {
+            const uint32_t p = bits >> (D::shift + D::bits);
+            if (p == p0) atomicAdd(&h[d], 1u);
+            else if (p == p1) atomicAdd(&h[NB + d], 1u);         // where it left the lower rank's prefix
+            if (NT == 3 && p == p2 && p2 != p0 && p2 != p1) atomicAdd(&h[(NT - 1) * NB + d], 1u);
+        }
+    };
+    // this block's share of the band, in whole float4 (bands start on 128-byte boundaries)
+    const int64_t quads = t.n[b] >> 2;
+    const int nblk = t.blk0[b + 1] - t.blk0[b], blk = blockIdx.x - t.blk0[b];
+    const int64_t q0 = quads * blk / nblk, q1 = quads * (blk + 1) / nblk;
+    const float4 *v4 = reinterpret_cast<const float4 *>(v + t.voff[b]);
+    int64_t q = q0 + tid;
+    for (; q + 3 * kSelThreads < q1; q += 4 * kSelThreads) {
+        float4 a[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) a[u] = v4[q + u * kSelThreads];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            count(a[u].x);
+            count(a[u].y);
+            count(a[u].z);
+            count(a[u].w);
+        }
+    }
+    for (; q < q1; q += kSelThreads) {
+        const float4 a = v4[q];
+        count(a.x);
+        count(a.y);
+        count(a.z);
+        count(a.w);
+    }
+    if (blk == nblk - 1 && 4 * quads + tid < t.n[b]) count(v[t.voff[b] + 4 * quads + tid]);
+    if constexpr (DIGIT == 0) {
+        zeros = __reduce_add_sync(0xffffffffu, zeros);
+        if ((tid & 31) == 0 && zeros) atomicAdd(&sb->zeros[DEV], (unsigned long long)zeros);
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < 256; i += blockDim.x)
-        if (h[i]) atomicAdd(&hist[i], h[i]);
-}
-
-__global__ void k_sel_pick(SubStat *st, const uint32_t *__restrict__ hist, int shift)
-{
-    if (threadIdx.x || blockIdx.x) return;
-    int64_t k = st->k;
-    uint32_t d = 0;
-    for (; d < 256; d++) {
-        if (k < (int64_t)hist[d]) break;
-        k -= hist[d];
+    for (int i = tid; i < NT * NB; i += kSelThreads) {
+        uint32_t c = 0;
+#pragma unroll
+        for (int k = 0; k < COPIES; k++) c += h[i * COPIES + k];
+        if (c) atomicAdd(&gh[(i / NB) * kBins + (i & (NB - 1))], c);
     }
-    st->k = k;
-    st->prefix |= d << shift;
-    st->mask |= 255u << shift;
-}
-
-// which: 0 = k fixed (host), 1 = k = n - K' (K-th largest among candidates)
-__global__ void k_sel_begin(SubStat *st, int64_t k, int which, int64_t n, int64_t K)
-{
-    if (threadIdx.x || blockIdx.x) return;
-    if (which == 1) {
-        const int64_t Kp = min(K, st->count_c);
-        k = Kp > 0 ? n - Kp : 0;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicInc(&sb->ticket, (uint32_t)nblk - 1) == (uint32_t)nblk - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // ---- the band's last block: pick the digits
+    const int64_t n = t.n[b];
+    const uint32_t n_zero = (uint32_t)__ldcg(&sb->zeros[DEV]);
+    if (DIGIT == 0 && !DEV) {
+        // K of this band: max(min_per_band, floor(K_tot S / sum S)), S = E^alpha N^beta
+        if (tid < t.nb) share[tid] = pow(__ldcg(E + tid), bud.alpha_E) * pow((double)t.n[tid], bud.beta_N);
+        __syncthreads();
+        if (tid == 0) {
+            double sum = 0.0;
+            for (int k = 0; k < t.nb; k++) sum += share[k];
+            const double mine = sum > 0 ? bud.K_tot * share[b] / sum : 0.0;
+            const int64_t K = max(bud.min_per_band, (int64_t)floor(mine));
+            sb->none = K <= 0;
+            sb->rank[2] = n - min(max(K, (int64_t)1), n);
+        }
     }
-    st->k = k;
-    st->prefix = 0;
-    st->mask = 0;
-}
-
-// where: 0 -> sel_a, 1 -> sel_b
-__global__ void k_sel_store(SubStat *st, int where)
-{
-    if (threadIdx.x || blockIdx.x) return;
-    const float val = __uint_as_float(st->prefix);
-    if (where == 0) st->sel_a = val; else st->sel_b = val;
-}
-
-// role: 0 = median of v -> med, 1 = median of dev -> mad (then sigma, T)
-__global__ void k_median_done(SubStat *st, int even, int role, float lambda)
-{
-    if (threadIdx.x || blockIdx.x) return;
-    const float m = even ? __fmul_rn(__fadd_rn(st->sel_a, st->sel_b), 0.5f) : st->sel_b;
-    if (role == 0) {
-        st->med = m;
-    } else {
-        st->mad = m;
-        const float sigma = __fdiv_rn(m, 0.6745f);
-        st->T = __fmul_rn(lambda, sigma);
+    if (DIGIT == 0 && tid == 0) {
+        sb->rank[0] = (n - 1) / 2;       // the middle value, or the lower one of an even count
+        sb->rank[1] = n / 2;
+        sb->prefix[0] = sb->prefix[1] = 0;
+        if (!DEV) sb->prefix[2] = 0;
+    }
+    __syncthreads();
+    const int n_target = DEV ? 2 : kTargets;
+    uint32_t old[kTargets];
+    for (int k = 0; k < n_target; k++) old[k] = sb->prefix[k];
+    __syncthreads();
+    for (int k = 0; k < n_target; k++) {
+        // the histogram that counted this target's prefix
+        const int src = DIGIT == 0 ? 0 : old[k] == old[0] ? 0 : old[k] == old[1] ? 1 : 2;
+        const long long rank = sb->rank[k];
+        constexpr int PER = (NB + kSelThreads - 1) / kSelThreads;
+        uint32_t c[PER], mine = 0, total;
+#pragma unroll
+        for (int i = 0; i < PER; i++) {
+            const int bin = tid * PER + i;
+            c[i] = __ldcg(&gh[src * kBins + bin]) + (bin == 0 && old[k] == 0 ? n_zero : 0u);
+            mine += c[i];
+        }
+        long long at = rank - (long long)block_scan<kSelThreads>(mine, warp_sum, total);
+        if (at >= 0 && at < (long long)mine) {
+            int i = 0;
+            while (i < PER - 1 && at >= (long long)c[i]) at -= c[i++];
+            s_digit = (uint32_t)(tid * PER + i);
+            s_rank = at;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            sb->rank[k] = s_rank;
+            sb->prefix[k] = (old[k] << D::bits) | s_digit;
+        }
+        __syncthreads();
+    }
+    for (int i = tid; i < kTargets * kBins; i += kSelThreads) gh[i] = 0;
+    if (DIGIT == 2 && tid == 0) {
+        const float a = __uint_as_float(sb->prefix[0]), c = __uint_as_float(sb->prefix[1]);
+        const float m = (n & 1) ? c : __fmul_rn(__fadd_rn(a, c), 0.5f);
+        if (!DEV) {
+            sb->med = m;
+            sb->vk = __uint_as_float(sb->prefix[2]);
+        } else {
+            // keep v >= max(T, v_(K')), K' = min(K, #{v >= T}): where fewer than K
+            // values reach T, v_(K) < T and the maximum is T itself, the same set
+            const float T = __fmul_rn(bud.lambda, __fdiv_rn(m, 0.6745f));
+            sb->thr = sb->none || T != T ? __int_as_float(0x7f800000) : fmaxf(T, sb->vk);
+        }
     }
 }
 
-__global__ void k_count_ge(const float *__restrict__ v, int64_t n, SubStat *st)
-{
-    __shared__ unsigned long long red;
-    if (threadIdx.x == 0) red = 0;
-    __syncthreads();
-    const float T = st->T;
-    unsigned long long c = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        c += v[i] >= T;
-    atomicAdd(&red, c);
-    __syncthreads();
-    if (threadIdx.x == 0) atomicAdd((unsigned long long *)&st->count_c, red);
-}
+// ------------------------------------------------------- marking and map
 
-__global__ void k_threshold(SubStat *st, int64_t K)
+// One bit per band element, set where the coefficient is kept (v >= threshold
+// and v > 0), and each chunk's count; the grid's last block turns the counts
+// into the chunks' first output columns and the total.  keep, if given,
+// receives one byte per pyramid element.
+__global__ void __launch_bounds__(kMarkThreads) k_mark(const float *__restrict__ v, const __grid_constant__ BandTab t,
+                                                       int nx, int ny, const SubState *__restrict__ st,
+                                                       uint32_t *__restrict__ mask, uint32_t *__restrict__ count,
+                                                       int64_t *__restrict__ first, int64_t *__restrict__ total,
+                                                       uint32_t *__restrict__ ticket, uint8_t *__restrict__ keep)
 {
-    if (threadIdx.x || blockIdx.x) return;
-    const int64_t Kp = min(K, st->count_c);
-    st->thr = Kp > 0 ? fmaxf(st->T, __uint_as_float(st->prefix)) : __int_as_float(0x7f800000);
-}
-
-__global__ void k_flags(const float *__restrict__ v, int nx, int ny, int ox, int oy, int oz, int mx, int my, int mz,
-                        SubStat *st, uint8_t *__restrict__ keep)
-{
-    __shared__ unsigned long long red;
-    if (threadIdx.x == 0) red = 0;
+    constexpr int U = 8;                                  // words of a warp, loaded together
+    __shared__ uint32_t s_count, s_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) s_count = 0;
     __syncthreads();
-    const float thr = st->thr;
-    const int64_t total = (int64_t)mx * my * mz;
-    unsigned long long c = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % mx), y = (int)((i / mx) % my), z = (int)(i / ((int64_t)mx * my));
-        const bool k = v[i] >= thr && v[i] > 0.f;
-        keep[((int64_t)(oz + z) * ny + (oy + y)) * nx + (ox + x)] = k;
-        c += k;
+    const int b = band_of(t.chunk0, t.nb, blockIdx.x);
+    const int64_t i0 = (int64_t)(blockIdx.x - t.chunk0[b]) * kChunk, n = t.n[b];
+    const float thr = st[b].thr;
+    const float *vb = v + t.voff[b];
+    uint32_t mine = 0;
+    for (int w0 = warp * U; w0 < kChunk / 32; w0 += kMarkThreads / 32 * U) {
+        float x[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int64_t i = i0 + (w0 + u) * 32 + lane;
+            x[u] = i < n ? vb[i] : 0.f;
+        }
+        uint32_t word = 0;
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const uint32_t bal = __ballot_sync(0xffffffffu, x[u] >= thr && x[u] > 0.f);
+            word = lane == u ? bal : word;
+        }
+        if (lane < U && i0 + (w0 + lane) * 32 < n) {
+            mask[(t.voff[b] + i0) / 32 + w0 + lane] = word;
+            mine += __popc(word);
+        }
+        if (keep) {
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int64_t i = i0 + (w0 + u) * 32 + lane;
+                int cx, cy, cz;
+                if (i < n) keep[pyramid_index(t, b, i, nx, ny, cx, cy, cz)] = x[u] >= thr && x[u] > 0.f;
+            }
+        }
     }
-    atomicAdd(&red, c);
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if (lane == 0) atomicAdd(&s_count, mine);
     __syncthreads();
-    if (threadIdx.x == 0) atomicAdd((unsigned long long *)&st->kept, red);
+    if (tid == 0) {
+        count[blockIdx.x] = s_count;
+        __threadfence();
+        s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    __shared__ uint32_t warp_sum[kMarkThreads / 32];
+    constexpr int PER = 16;
+    int64_t run = 0;
+    for (int c0 = 0; c0 < (int)gridDim.x; c0 += kMarkThreads * PER) {
+        uint32_t c[PER], sum = 0, all;
+#pragma unroll
+        for (int k = 0; k < PER; k++) {
+            const int i = c0 + tid * PER + k;
+            c[k] = i < (int)gridDim.x ? __ldcg(count + i) : 0u;
+            sum += c[k];
+        }
+        int64_t at = run + block_scan<kMarkThreads>(sum, warp_sum, all);
+#pragma unroll
+        for (int k = 0; k < PER; k++) {
+            const int i = c0 + tid * PER + k;
+            if (i < (int)gridDim.x) first[i] = at;
+            at += c[k];
+        }
+        run += all;
+    }
+    if (tid == 0) *total = run;
 }
-
-// ------------------------------------------------------------------ map
 
 struct MapEntry {
     float u[3];
@@ -267,58 +479,55 @@ struct MapEntry {
     int j;
 };
 
-// Single-block ordered compaction of one subband (raster order), then the
-// per-coefficient map of Eq. 22-24.  One block per subband keeps the order
-// without a global scan; blocks walk their subband in chunks of blockDim.
-__global__ void __launch_bounds__(1024) k_map_subband(const float *__restrict__ A, int64_t chan, int nx, int ny,
-                                                      int ox, int oy, int oz, int mx, int my, int mz,
-                                                      const uint8_t *__restrict__ keep, MapEntry me, int64_t out_off,
-                                                      float *__restrict__ P, int64_t stride)
+struct MapTab {
+    MapEntry e[kMaxBands];
+};
+
+// The per-coefficient map (Eq. 22-24) of one chunk's kept coefficients: the
+// mask's set bits are listed in raster order in shared memory, so the threads
+// take consecutive output columns and each of the 14 rows is written in whole
+// lines.  Nothing is written when the total exceeds the capacity.
+__global__ void __launch_bounds__(kMarkThreads) k_map(const float *__restrict__ A, int64_t chan, int nx, int ny,
+                                                      const __grid_constant__ BandTab t,
+                                                      const uint32_t *__restrict__ mask,
+                                                      const uint32_t *__restrict__ count,
+                                                      const int64_t *__restrict__ first,
+                                                      const int64_t *__restrict__ total,
+                                                      const MapTab *__restrict__ tab, float *__restrict__ P,
+                                                      int64_t stride)
 {
-    __shared__ int warp_tot[32];
-    __shared__ int64_t carry;
-    if (threadIdx.x == 0) carry = 0;
+    static_assert(kChunk / 32 == kMarkThreads && kChunk <= 65536, "one mask word per thread, 16-bit positions");
+    __shared__ uint16_t list[kChunk];
+    __shared__ uint32_t warp_sum[kMarkThreads / 32];
+    const uint32_t kept = count[blockIdx.x];
+    if (kept == 0 || *total > stride) return;             // block-uniform
+    const int tid = threadIdx.x;
+    const int b = band_of(t.chunk0, t.nb, blockIdx.x);
+    const int64_t i0 = (int64_t)(blockIdx.x - t.chunk0[b]) * kChunk;
+    uint32_t word = i0 + tid * 32 < t.n[b] ? mask[(t.voff[b] + i0) / 32 + tid] : 0u, all;
+    uint32_t at = block_scan<kMarkThreads>(__popc(word), warp_sum, all);
+    for (; word; word &= word - 1) list[at++] = (uint16_t)(tid * 32 + __ffs(word) - 1);
     __syncthreads();
-    const int64_t total = (int64_t)mx * my * mz;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    for (int64_t base = 0; base < total; base += blockDim.x) {
-        const int64_t i = base + threadIdx.x;
-        int x = 0, y = 0, z = 0;
-        bool k = false;
-        int64_t e = 0;
-        if (i < total) {
-            x = (int)(i % mx); y = (int)((i / mx) % my); z = (int)(i / ((int64_t)mx * my));
-            e = ((int64_t)(oz + z) * ny + (oy + y)) * nx + (ox + x);
-            k = keep[e] != 0;
-        }
-        const uint32_t bal = __ballot_sync(0xffffffffu, k);
-        if (lane == 0) warp_tot[warp] = __popc(bal);
-        __syncthreads();
-        int before = 0, all = 0;
-        for (int w = 0; w < nwarps; w++) {
-            if (w < warp) before += warp_tot[w];
-            all += warp_tot[w];
-        }
-        if (k) {
-            const int64_t pos = out_off + carry + before + __popc(bal & ((1u << lane) - 1u));
-            float amp[4];
-            for (int c = 0; c < 4; c++) amp[c] = me.s * fabsf(A[c * chan + e]) * me.w;
-            const float step = (float)(1 << me.j);
-            P[0 * stride + pos] = me.u[0] + step * x + 0.5f;
-            P[1 * stride + pos] = me.u[1] + step * y + 0.5f;
-            P[2 * stride + pos] = me.u[2] + step * z + 0.5f;
-            for (int d = 0; d < 3; d++) P[(3 + d) * stride + pos] = me.log_scale[d];
-            for (int d = 0; d < 4; d++) P[(6 + d) * stride + pos] = me.quat[d];
-            // floor 2/255: a retained coefficient stays above the 1/255 cut-off
-            const float op = fminf(fmaxf(amp[3], 2.f / 255.f), 0.99f);
-            P[10 * stride + pos] = logf(op / (1.f - op));
-            P[11 * stride + pos] = amp[0];
-            P[12 * stride + pos] = amp[1];
-            P[13 * stride + pos] = amp[2];
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) carry += all;
-        __syncthreads();
+    const MapEntry me = tab->e[b];
+    const int64_t out = first[blockIdx.x];
+    for (uint32_t k = tid; k < kept; k += kMarkThreads) {
+        const int64_t pos = out + k;
+        int x, y, z;
+        const int64_t e = pyramid_index(t, b, i0 + list[k], nx, ny, x, y, z);
+        float amp[4];
+        for (int c = 0; c < 4; c++) amp[c] = me.s * fabsf(A[c * chan + e]) * me.w;
+        const float step = (float)(1 << me.j);
+        P[0 * stride + pos] = me.u[0] + step * x + 0.5f;
+        P[1 * stride + pos] = me.u[1] + step * y + 0.5f;
+        P[2 * stride + pos] = me.u[2] + step * z + 0.5f;
+        for (int d = 0; d < 3; d++) P[(3 + d) * stride + pos] = me.log_scale[d];
+        for (int d = 0; d < 4; d++) P[(6 + d) * stride + pos] = me.quat[d];
+        // floor 2/255: a retained coefficient stays above the 1/255 cut-off
+        const float op = fminf(fmaxf(amp[3], 2.f / 255.f), 0.99f);
+        P[10 * stride + pos] = logf(op / (1.f - op));
+        P[11 * stride + pos] = amp[0];
+        P[12 * stride + pos] = amp[1];
+        P[13 * stride + pos] = amp[2];
     }
 }
 
@@ -381,11 +590,6 @@ vbm_status dwt_channels(float *data, int n_channels, const int dims[3], int leve
     return VBM_OK;
 }
 
-struct Band {
-    int j, o[3], ox, oy, oz, mx, my, mz;
-    int64_t n;
-};
-
 std::vector<Band> bands_of(const int dims[3], int levels)
 {
     std::vector<Band> out;
@@ -403,46 +607,77 @@ std::vector<Band> bands_of(const int dims[3], int levels)
     return out;
 }
 
-// k-th smallest (0-based, k set by k_sel_begin) of v[0..n) into st->prefix
-void radix_select(const float *v, int64_t n, SubStat *st, uint32_t *hist, cudaStream_t s)
+// Element offsets, marking chunks and selection blocks of the bands.  A
+// selection block takes at least 8192 elements of one band; beyond that the
+// blocks are two waves of the chip's resident ones, shared out by band size.
+BandTab band_table(const std::vector<Band> &bands)
 {
-    const int g = grid_for(n);
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        cudaMemsetAsync(hist, 0, 256 * sizeof(uint32_t), s);
-        k_sel_hist<<<g, 256, 0, s>>>(v, n, st, shift, hist);
-        k_sel_pick<<<1, 32, 0, s>>>(st, hist, shift);
+    BandTab t{};
+    t.nb = (int)bands.size();
+    int64_t all = 0, off = 0;
+    for (const Band &B : bands) all += B.n;
+    const int64_t per = std::max<int64_t>(8192, all / (2 * (int64_t)num_sms()) + 1);
+    for (int b = 0; b < t.nb; b++) {
+        const Band &B = bands[b];
+        t.ox[b] = B.ox; t.oy[b] = B.oy; t.oz[b] = B.oz; t.mx[b] = B.mx; t.my[b] = B.my;
+        t.n[b] = B.n;
+        t.voff[b] = off;
+        off += (B.n + 31) / 32 * 32;
+        t.chunk0[b + 1] = t.chunk0[b] + (int)((B.n + kChunk - 1) / kChunk);
+        t.blk0[b + 1] = t.blk0[b] + (int)((B.n + per - 1) / per);
     }
+    return t;
 }
 
-void median_of(const float *v, int64_t n, SubStat *st, uint32_t *hist, int role, float lambda, cudaStream_t s)
+// Device scratch of one build, in order; with ws = NULL only its size.
+struct BuildScratch {
+    float *A, *tmp;
+    uint32_t *mask, *count;
+    int64_t *first;
+    MapTab *map;
+    char *zeroed;            // from here on cleared at the start of a build
+    SubState *st;
+    double *E;
+    uint32_t *hist, *ticket;
+    int64_t *total;
+    size_t bytes, zero_bytes;
+};
+
+BuildScratch build_scratch(void *ws, const int dims[3])
 {
-    const bool even = (n % 2) == 0;
-    if (even) {
-        k_sel_begin<<<1, 32, 0, s>>>(st, n / 2 - 1, 0, n, 0);
-        radix_select(v, n, st, hist, s);
-        k_sel_store<<<1, 32, 0, s>>>(st, 0);
-    }
-    k_sel_begin<<<1, 32, 0, s>>>(st, n / 2, 0, n, 0);
-    radix_select(v, n, st, hist, s);
-    k_sel_store<<<1, 32, 0, s>>>(st, 1);
-    k_median_done<<<1, 32, 0, s>>>(st, even ? 1 : 0, role, lambda);
+    const size_t n = (size_t)dims[0] * dims[1] * dims[2], padded = n + 32 * kMaxBands;
+    BuildScratch s{};
+    size_t at = (256 - (reinterpret_cast<uintptr_t>(ws) & 255)) & 255;     // 256-byte aligned whatever ws is
+    auto take = [&](size_t bytes) {
+        char *p = reinterpret_cast<char *>(ws) + at;
+        at += (bytes + 255) / 256 * 256;
+        return p;
+    };
+    const size_t chunks = n / kChunk + kMaxBands;
+    s.A = (float *)take(4 * n * sizeof(float));                            // RF / pyramid
+    s.tmp = (float *)take(std::max(2 * n, padded) * sizeof(float));        // DWT temporaries, then the magnitudes
+    s.mask = (uint32_t *)take(padded / 32 * sizeof(uint32_t));
+    s.count = (uint32_t *)take(chunks * sizeof(uint32_t));
+    s.first = (int64_t *)take(chunks * sizeof(int64_t));
+    s.map = (MapTab *)take(sizeof(MapTab));
+    const size_t z0 = at;
+    s.zeroed = reinterpret_cast<char *>(ws) + at;
+    s.st = (SubState *)take(kMaxBands * sizeof(SubState));
+    s.E = (double *)take(kMaxBands * sizeof(double));
+    s.ticket = (uint32_t *)take(sizeof(uint32_t));
+    s.total = (int64_t *)take(sizeof(int64_t));
+    s.hist = (uint32_t *)take((size_t)kMaxBands * kTargets * kBins * sizeof(uint32_t));
+    s.zero_bytes = at - z0;
+    s.bytes = at + 256;                                                    // room to align the next ws
+    return s;
 }
 
 }  // namespace
 
 size_t build_workspace_bytes(const int dims[3], int levels)
 {
-    const size_t n = (size_t)dims[0] * dims[1] * dims[2];
-    size_t b = 0;
-    auto add = [&](size_t bytes) { b += (bytes + 255) / 256 * 256; };
-    add(4 * n * sizeof(float));         // RF / pyramid
-    add(2 * n * sizeof(float));         // DWT temporaries (reused as v, dev)
-    add(n);                             // keep flags
-    add(64 * sizeof(SubStat));
-    add(64 * sizeof(double));
-    add(256 * sizeof(uint32_t));
     (void)levels;
-    return b;
+    return build_scratch(nullptr, dims).bytes;
 }
 
 }  // namespace vbm
@@ -494,88 +729,16 @@ vbm_status vbm_build(const float *d_volume, const int dims[3], const vbm_tf *tf,
     VBM_ARG(sel->K_tot > 0 && sel->min_per_band >= 0, "invalid selection parameters");
     cudaStream_t st = (cudaStream_t)stream;
     const int64_t n = (int64_t)dims[0] * dims[1] * dims[2];
-    char *w = (char *)d_ws;
-    auto take = [&](size_t bytes) {
-        char *p = w;
-        w += (bytes + 255) / 256 * 256;
-        return (void *)p;
-    };
-    float *A = (float *)take(4 * n * sizeof(float));
-    float *tmp = (float *)take(2 * n * sizeof(float));
-    uint8_t *keep = (uint8_t *)take(n);
-    SubStat *stats = (SubStat *)take(64 * sizeof(SubStat));
-    double *E = (double *)take(64 * sizeof(double));
-    uint32_t *hist = (uint32_t *)take(256 * sizeof(uint32_t));
-
-    vbm_status s = vbm_tf_apply(d_volume, n, tf, A, stream);
-    if (s != VBM_OK) return s;
-    s = dwt_channels(A, 4, dims, levels, bank->wavelet, tmp, st);
-    if (s != VBM_OK) return s;
+    const BuildScratch w = build_scratch(d_ws, dims);
+    float *A = w.A, *v = w.tmp;
     std::vector<Band> bands = bands_of(dims, levels);
     const int nb = (int)bands.size();
-    VBM_CUDA(cudaMemsetAsync(E, 0, 64 * sizeof(double), st));
-    VBM_CUDA(cudaMemsetAsync(stats, 0, 64 * sizeof(SubStat), st));
-    VBM_CUDA(cudaMemsetAsync(keep, 0, n, st));
-    const float *alpha = A + 3 * n;
-    for (int b = 0; b < nb; b++) {
-        const Band &B = bands[b];
-        k_energy<<<grid_for(B.n), 256, 0, st>>>(alpha, dims[0], dims[1], B.ox, B.oy, B.oz, B.mx, B.my, B.mz, E + b);
-    }
-    VBM_LAUNCH("energy");
-    std::vector<double> hE(nb);
-    VBM_CUDA(cudaMemcpyAsync(hE.data(), E, nb * sizeof(double), cudaMemcpyDeviceToHost, st));
-    VBM_CUDA(cudaStreamSynchronize(st));
-    // budget allocation (Supp. Sec. 1.1), host FP64
-    std::vector<double> S(nb);
-    double sumS = 0.0;
-    for (int b = 0; b < nb; b++) {
-        S[b] = std::pow(hE[b], sel->alpha_E) * std::pow((double)bands[b].n, sel->beta_N);
-        sumS += S[b];
-    }
-    std::vector<int64_t> K(nb);
-    for (int b = 0; b < nb; b++) {
-        double share = sumS > 0 ? (double)sel->K_tot * S[b] / sumS : 0.0;
-        K[b] = std::max<int64_t>(sel->min_per_band, (int64_t)std::floor(share));
-    }
-    float *v = tmp, *dev = tmp + n;
-    const float lam = (float)sel->lambda_mad;
-    for (int b = 0; b < nb; b++) {
-        const Band &B = bands[b];
-        SubStat *stb = stats + b;
-        const int g = grid_for(B.n);
-        k_joint_mag<<<g, 256, 0, st>>>(A, n, dims[0], dims[1], B.ox, B.oy, B.oz, B.mx, B.my, B.mz, v);
-        median_of(v, B.n, stb, hist, 0, lam, st);
-        k_abs_dev<<<g, 256, 0, st>>>(v, B.n, stb, dev);
-        median_of(dev, B.n, stb, hist, 1, lam, st);
-        k_count_ge<<<g, 256, 0, st>>>(v, B.n, stb);
-        k_sel_begin<<<1, 32, 0, st>>>(stb, 0, 1, B.n, K[b]);
-        radix_select(v, B.n, stb, hist, st);
-        k_threshold<<<1, 32, 0, st>>>(stb, K[b]);
-        k_flags<<<g, 256, 0, st>>>(v, dims[0], dims[1], B.ox, B.oy, B.oz, B.mx, B.my, B.mz, stb, keep);
-        VBM_LAUNCH("select");
-    }
-    std::vector<SubStat> hs(nb);
-    VBM_CUDA(cudaMemcpyAsync(hs.data(), stats, nb * sizeof(SubStat), cudaMemcpyDeviceToHost, st));
-    VBM_CUDA(cudaStreamSynchronize(st));
-    int64_t total = 0;
-    std::vector<int64_t> off(nb);
-    for (int b = 0; b < nb; b++) {
-        off[b] = total;
-        total += hs[b].kept;
-    }
-    *n_out = total;
-    if (d_coef) VBM_CUDA(cudaMemcpyAsync(d_coef, A, 4 * n * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    if (d_keep) VBM_CUDA(cudaMemcpyAsync(d_keep, keep, n, cudaMemcpyDeviceToDevice, st));
-    if (total > capacity) {
-        VBM_CUDA(cudaStreamSynchronize(st));
-        set_error("vbm_build: " + std::to_string(total) + " Gaussians kept, capacity " + std::to_string(capacity));
-        return VBM_ERR_CAPACITY;
-    }
+    MapTab map{};
     for (int b = 0; b < nb; b++) {
         const Band &B = bands[b];
         const vbm_bank_entry &e = bank->sub[b];
         VBM_ARG(e.j == B.j && e.o[0] == B.o[0] && e.o[1] == B.o[1] && e.o[2] == B.o[2], "bank order mismatch");
-        MapEntry me;
+        MapEntry &me = map.e[b];
         for (int d = 0; d < 3; d++) {
             me.u[d] = (float)e.u[d];
             me.log_scale[d] = e.log_scale[d];
@@ -584,12 +747,42 @@ vbm_status vbm_build(const float *d_volume, const int dims[3], const vbm_tf *tf,
         me.w = (float)e.w;
         me.j = B.j;
         me.s = sel->energy_comp ? (float)std::pow(2.0, -1.5 * B.j) : 1.f;
-        if (hs[b].kept == 0) continue;
-        k_map_subband<<<1, 1024, 0, st>>>(A, n, dims[0], dims[1], B.ox, B.oy, B.oz, B.mx, B.my, B.mz, keep, me,
-                                          off[b], d_params, capacity);
-        VBM_LAUNCH("map_subband");
     }
+    const BandTab t = band_table(bands);
+    const Budget bud{sel->alpha_E, sel->beta_N, (double)sel->K_tot, sel->min_per_band, (float)sel->lambda_mad};
+
+    VBM_CUDA(cudaMemcpyAsync(w.map, &map, sizeof(map), cudaMemcpyHostToDevice, st));
+    VBM_CUDA(cudaMemsetAsync(w.zeroed, 0, w.zero_bytes, st));
+    vbm_status s = vbm_tf_apply(d_volume, n, tf, A, stream);
+    if (s != VBM_OK) return s;
+    s = dwt_channels(A, 4, dims, levels, bank->wavelet, w.tmp, st);
+    if (s != VBM_OK) return s;
+    const int chunks = t.chunk0[nb], blocks = t.blk0[nb];
+    k_joint_mag<<<chunks, kMarkThreads, 0, st>>>(A, n, dims[0], dims[1], t, v, w.E);
+    k_select_pass<0, false><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
+    k_select_pass<1, false><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
+    k_select_pass<2, false><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
+    k_select_pass<0, true><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
+    k_select_pass<1, true><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
+    k_select_pass<2, true><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
+    VBM_LAUNCH("select");
+    k_mark<<<chunks, kMarkThreads, 0, st>>>(v, t, dims[0], dims[1], w.st, w.mask, w.count, w.first, w.total, w.ticket,
+                                            d_keep);
+    VBM_LAUNCH("mark");
+    int64_t total = 0;
+    VBM_CUDA(cudaMemcpyAsync(&total, w.total, sizeof(total), cudaMemcpyDeviceToHost, st));
+    if (capacity > 0) {
+        k_map<<<chunks, kMarkThreads, 0, st>>>(A, n, dims[0], dims[1], t, w.mask, w.count, w.first, w.total, w.map,
+                                               d_params, capacity);
+        VBM_LAUNCH("map");
+    }
+    if (d_coef) VBM_CUDA(cudaMemcpyAsync(d_coef, A, 4 * n * sizeof(float), cudaMemcpyDeviceToDevice, st));
     VBM_CUDA(cudaStreamSynchronize(st));
+    *n_out = total;
+    if (total > capacity) {
+        set_error("vbm_build: " + std::to_string(total) + " Gaussians kept, capacity " + std::to_string(capacity));
+        return VBM_ERR_CAPACITY;
+    }
     return VBM_OK;
 }
 
