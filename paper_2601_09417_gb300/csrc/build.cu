@@ -1,10 +1,6 @@
-// Volume -> Gaussians (Sec. 4.1-4.3): transfer function, periodised 3D DWT,
-// adaptive coefficient filtering (Supp. Sec. 1) and the per-coefficient map
-// (Eq. 22-24).  A setup step, run once per volume and TF.
-//
-// DWT: one level = three axis passes (x, y, z), each a gather kernel with one
-// thread per output coefficient (9- and 7-tap filters from constant memory;
-// neighbouring threads read neighbouring inputs, so the taps hit L1/L2).
+// Volume -> Gaussians (Sec. 4.1-4.3): transfer function and periodised 3D DWT
+// (dwt.cu), adaptive coefficient filtering (Supp. Sec. 1) and the
+// per-coefficient map (Eq. 22-24).  A setup step, run once per volume and TF.
 //
 // Selection, all on the device and over every subband in the same launches:
 //   v = sqrt(((a0 a0 + a1 a1) + a2 a2) + a3 a3) in IEEE float32, rounded op by
@@ -29,71 +25,6 @@
 namespace vbm {
 
 namespace {
-
-struct DevFilters {
-    int lo_n0, lo_len, hi_n0, hi_len;
-    float lo[16], hi[16];
-};
-__constant__ DevFilters c_filt;
-
-struct TFDev {
-    int n;
-    float x[16];
-    float rgba[16][4];
-};
-
-__global__ void k_tf_apply(const float *__restrict__ F, int64_t n, TFDev tf, float *__restrict__ RF)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        float f = fminf(fmaxf(F[i], 0.f), 1.f);
-        float out[4];
-        if (f <= tf.x[0]) {
-            for (int c = 0; c < 4; c++) out[c] = tf.rgba[0][c];
-        } else if (f >= tf.x[tf.n - 1]) {
-            for (int c = 0; c < 4; c++) out[c] = tf.rgba[tf.n - 1][c];
-        } else {
-            int k = 0;
-            while (k < tf.n - 2 && tf.x[k + 1] <= f) k++;
-            const float t = (f - tf.x[k]) / (tf.x[k + 1] - tf.x[k]);
-            for (int c = 0; c < 4; c++) out[c] = (1.f - t) * tf.rgba[k][c] + t * tf.rgba[k + 1][c];
-        }
-        for (int c = 0; c < 4; c++) RF[c * n + i] = out[c];
-    }
-}
-
-// One periodised analysis pass along `axis` over the region [0,s0)x[0,s1)x[0,s2)
-// of arrays with row strides (nx, nx*ny): output index k < L/2 is the
-// low-pass a[k], k >= L/2 the high-pass d[k - L/2].
-__global__ void k_dwt_axis(const float *__restrict__ src, float *__restrict__ dst, int nx, int ny, int sx, int sy,
-                           int sz, int axis)
-{
-    const int64_t total = (int64_t)sx * sy * sz;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % sx);
-        const int y = (int)((i / sx) % sy);
-        const int z = (int)(i / ((int64_t)sx * sy));
-        int c[3] = {x, y, z};
-        const int L = axis == 0 ? sx : axis == 1 ? sy : sz;
-        const int half = L >> 1;
-        const int k = c[axis];
-        const bool low = k < half;
-        const int kk = low ? k : k - half;
-        const int n0 = low ? c_filt.lo_n0 : c_filt.hi_n0;
-        const int len = low ? c_filt.lo_len : c_filt.hi_len;
-        const int base = 2 * kk + (low ? 0 : 1);
-        float acc = 0.f;
-        for (int t = 0; t < len; t++) {
-            int m = base + n0 + t;
-            m %= L;
-            if (m < 0) m += L;
-            c[axis] = m;
-            const float w = low ? c_filt.lo[t] : c_filt.hi[t];
-            acc += w * src[((int64_t)c[2] * ny + c[1]) * nx + c[0]];
-        }
-        dst[((int64_t)z * ny + y) * nx + x] = acc;
-    }
-}
 
 // ----------------------------------------------------------------- select
 
@@ -533,63 +464,6 @@ __global__ void __launch_bounds__(kMarkThreads) k_map(const float *__restrict__ 
 
 // ------------------------------------------------------------- helpers
 
-vbm_status upload_filters(int wavelet)
-{
-    FilterBank fb = make_filters(wavelet);
-    DevFilters f{};
-    f.lo_n0 = fb.ht.begin()->first;
-    f.lo_len = (int)fb.ht.size();
-    f.hi_n0 = fb.gt.begin()->first;
-    f.hi_len = (int)fb.gt.size();
-    int t = 0;
-    for (auto &kv : fb.ht) f.lo[t++] = (float)kv.second;
-    t = 0;
-    for (auto &kv : fb.gt) f.hi[t++] = (float)kv.second;
-    VBM_CUDA(cudaMemcpyToSymbol(c_filt, &f, sizeof(f)));
-    return VBM_OK;
-}
-
-TFDev to_dev(const vbm_tf *tf)
-{
-    TFDev t{};
-    t.n = tf->n_knots;
-    for (int i = 0; i < 16; i++) {
-        t.x[i] = tf->x[i];
-        for (int c = 0; c < 4; c++) t.rgba[i][c] = tf->rgba[i][c];
-    }
-    return t;
-}
-
-int grid_for(int64_t n, int threads = 256)
-{
-    int64_t b = (n + threads - 1) / threads;
-    int64_t cap = (int64_t)num_sms() * 16;
-    return (int)std::max<int64_t>(1, std::min(b, cap));
-}
-
-vbm_status dwt_channels(float *data, int n_channels, const int dims[3], int levels, int wavelet, float *tmp,
-                        cudaStream_t st)
-{
-    vbm_status s = upload_filters(wavelet);
-    if (s != VBM_OK) return s;
-    const int nx = dims[0], ny = dims[1], nz = dims[2];
-    const int64_t n = (int64_t)nx * ny * nz;
-    float *t1 = tmp, *t2 = tmp + n;
-    for (int c = 0; c < n_channels; c++) {
-        float *P = data + c * n;
-        for (int j = 1; j <= levels; j++) {
-            const int sx = nx >> (j - 1), sy = ny >> (j - 1), sz = nz >> (j - 1);
-            const int64_t tot = (int64_t)sx * sy * sz;
-            const int g = grid_for(tot);
-            k_dwt_axis<<<g, 256, 0, st>>>(P, t1, nx, ny, sx, sy, sz, 0);
-            k_dwt_axis<<<g, 256, 0, st>>>(t1, t2, nx, ny, sx, sy, sz, 1);
-            k_dwt_axis<<<g, 256, 0, st>>>(t2, P, nx, ny, sx, sy, sz, 2);
-            VBM_LAUNCH("dwt_axis");
-        }
-    }
-    return VBM_OK;
-}
-
 std::vector<Band> bands_of(const int dims[3], int levels)
 {
     std::vector<Band> out;
@@ -655,7 +529,7 @@ BuildScratch build_scratch(void *ws, const int dims[3])
     };
     const size_t chunks = n / kChunk + kMaxBands;
     s.A = (float *)take(4 * n * sizeof(float));                            // RF / pyramid
-    s.tmp = (float *)take(std::max(2 * n, padded) * sizeof(float));        // DWT temporaries, then the magnitudes
+    s.tmp = (float *)take(std::max((size_t)pyramid_tmp_floats(dims), padded) * sizeof(float));   // DWT, then magnitudes
     s.mask = (uint32_t *)take(padded / 32 * sizeof(uint32_t));
     s.count = (uint32_t *)take(chunks * sizeof(uint32_t));
     s.first = (int64_t *)take(chunks * sizeof(int64_t));
@@ -670,6 +544,13 @@ BuildScratch build_scratch(void *ws, const int dims[3])
     s.zero_bytes = at - z0;
     s.bytes = at + 256;                                                    // room to align the next ws
     return s;
+}
+
+vbm_status check_tf(const vbm_tf *tf)
+{
+    VBM_ARG(tf->n_knots >= 2 && tf->n_knots <= 16, "n_knots must be in [2, 16]");
+    for (int i = 1; i < tf->n_knots; i++) VBM_ARG(tf->x[i] > tf->x[i - 1], "TF knots must be ascending");
+    return VBM_OK;
 }
 
 }  // namespace
@@ -689,12 +570,9 @@ extern "C" {
 vbm_status vbm_tf_apply(const float *d_volume, int64_t n, const vbm_tf *tf, float *d_rf, void *stream)
 {
     VBM_ARG(d_volume && tf && d_rf && n >= 0, "invalid argument");
-    VBM_ARG(tf->n_knots >= 2 && tf->n_knots <= 16, "n_knots must be in [2, 16]");
-    for (int i = 1; i < tf->n_knots; i++) VBM_ARG(tf->x[i] > tf->x[i - 1], "TF knots must be ascending");
-    if (n == 0) return VBM_OK;
-    k_tf_apply<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>(d_volume, n, to_dev(tf), d_rf);
-    VBM_LAUNCH("tf_apply");
-    return VBM_OK;
+    vbm_status s = check_tf(tf);
+    if (s != VBM_OK || n == 0) return s;
+    return tf_apply(d_volume, n, tf, d_rf, (cudaStream_t)stream);
 }
 
 vbm_status vbm_dwt3d(float *d_data, int n_channels, const int dims[3], int levels, int wavelet, float *d_tmp,
@@ -727,6 +605,8 @@ vbm_status vbm_build(const float *d_volume, const int dims[3], const vbm_tf *tf,
         VBM_ARG(dims[d] > 0 && dims[d] % (1 << levels) == 0, "dims must be divisible by 2^levels");
     VBM_ARG(ws_bytes >= build_workspace_bytes(dims, levels), "build workspace too small");
     VBM_ARG(sel->K_tot > 0 && sel->min_per_band >= 0, "invalid selection parameters");
+    vbm_status s = check_tf(tf);
+    if (s != VBM_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     const int64_t n = (int64_t)dims[0] * dims[1] * dims[2];
     const BuildScratch w = build_scratch(d_ws, dims);
@@ -753,9 +633,7 @@ vbm_status vbm_build(const float *d_volume, const int dims[3], const vbm_tf *tf,
 
     VBM_CUDA(cudaMemcpyAsync(w.map, &map, sizeof(map), cudaMemcpyHostToDevice, st));
     VBM_CUDA(cudaMemsetAsync(w.zeroed, 0, w.zero_bytes, st));
-    vbm_status s = vbm_tf_apply(d_volume, n, tf, A, stream);
-    if (s != VBM_OK) return s;
-    s = dwt_channels(A, 4, dims, levels, bank->wavelet, w.tmp, st);
+    s = pyramid_from_volume(d_volume, dims, tf, levels, bank->wavelet, A, w.tmp, st);
     if (s != VBM_OK) return s;
     const int chunks = t.chunk0[nb], blocks = t.blk0[nb];
     k_joint_mag<<<chunks, kMarkThreads, 0, st>>>(A, n, dims[0], dims[1], t, v, w.E);

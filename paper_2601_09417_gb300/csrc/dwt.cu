@@ -1,0 +1,518 @@
+// Transfer function and periodised separable 3D wavelet transform (Sec. 3,
+// Eq. 1-3; Sec. 4.3, Eq. 20-21) in the Mallat layout.
+//
+// One level is two kernels: k_dwt_xy transforms along x and y, plane by plane,
+// and k_dwt_z along z.  Every filter is a chain of fused multiply-adds in the
+// order of its taps, along x, then y, then z, so how the work is split does
+// not change a bit of the result.
+//
+// Traffic of a level: each plane is read once and written once by either
+// kernel; vbm_build's first level reads the scalar volume itself and applies
+// the transfer function where the rows are staged, so the four RGBA channels
+// are never stored untransformed.  Against one gather kernel an axis (a 64-bit
+// division and a modulo for every tap, three reads and writes of each value):
+// tf_apply + four-level dwt3d of 4 x 256^3, 4.30 -> 0.43 ms; vbm_build of a
+// 512^3 volume, 36.3 -> 5.7 ms.
+#include "tf_dev.h"
+
+namespace vbm {
+
+namespace {
+
+// Filter taps, low-pass then high-pass, passed by value: calls on different
+// streams or with different wavelets share nothing.
+struct Taps {
+    float lo[9], hi[9];
+};
+
+// Tap ranges relative to the even sample 2k: a[k] sums x[2k + LO], ..., and
+// d[k] sums x[2k + HI], ...; PAIRS sample pairs from 2k + FIRST on cover both.
+template <int WAVELET>
+struct Wavelet;
+template <>
+struct Wavelet<0> {     // bior4.4: 9 and 7 taps
+    static constexpr int LO = -4, LO_LEN = 9, HI = -2, HI_LEN = 7, FIRST = -4, PAIRS = 5;
+};
+template <>
+struct Wavelet<1> {     // Haar
+    static constexpr int LO = 0, LO_LEN = 2, HI = 0, HI_LEN = 2, FIRST = 0, PAIRS = 1;
+};
+
+Taps make_taps(int wavelet)
+{
+    const FilterBank fb = make_filters(wavelet);
+    Taps t{};
+    int k = 0;
+    for (auto &kv : fb.ht) t.lo[k++] = (float)kv.second;
+    k = 0;
+    for (auto &kv : fb.gt) t.hi[k++] = (float)kv.second;
+    return t;
+}
+
+__device__ __forceinline__ int wrap(int i, int n)
+{
+    i %= n;
+    return i < 0 ? i + n : i;
+}
+
+constexpr int kXYThreads = 256;
+constexpr int kXPer = 4;                 // x positions (two output pairs) a thread
+constexpr int kMaxSlot = 64;             // threads of a slot: 256 positions
+constexpr int kMinSlot = 8;
+
+// x and y passes.  A slot of `1 << slot_log` threads takes one strip: a tile
+// of 4 x positions a thread, `pairs` row pairs, one plane, one channel.  Rows
+// enter in order, two at a time: staged in shared memory (double-buffered, the
+// next two rows in flight in registers), filtered along x (each thread reads
+// its 12 inputs as three 16-byte words for four outputs) and kept in a
+// register ring of the 10 rows the y filter spans, from which every new row
+// pair gives one low and one high output row.  A row is therefore read once a
+// strip (plus the 8 rows of overlap between strips), not once a tap, and
+// nothing goes to memory between the two passes.
+//
+// FROM_TF: the source is the scalar volume; four neighbouring slots take the
+// four channels of one strip, whose threads share the loads and the transfer
+// function's evaluation.
+struct XYArgs {
+    const float *src;
+    int64_t src_chan, src_plane;         // strides of a channel and a plane
+    int src_row;
+    float *dst;                          // [channel][plane][sy][sx]
+    int64_t dst_chan;
+    int sx, sy, sz;                      // region
+    int z_first, planes;                 // plane t of dst holds z = (z_first + t) mod sz
+    int pairs;                           // row pairs a strip
+    int x_tiles, strips_y, slot_log;
+    int vec2;                            // low and high rows start on 8-byte boundaries
+};
+
+template <int WAVELET, bool FROM_TF>
+__global__ void __launch_bounds__(kXYThreads, 2) k_dwt_xy(const __grid_constant__ XYArgs a,
+                                                          const __grid_constant__ Taps w,
+                                                          const __grid_constant__ TFDev tf)
+{
+    using Wv = Wavelet<WAVELET>;
+    constexpr int HALO = 4;                                      // staged positions before the tile
+    constexpr int R = Wv::PAIRS;
+    constexpr int MAX_ROW = kXYThreads * kXPer + 8 * (kXYThreads / kMinSlot);
+    __shared__ __align__(16) float rows[2][2][MAX_ROW];          // [buffer][row][slot][position]
+    __shared__ float4 knots[16];
+    const int slot_threads = 1 << a.slot_log;
+    const int tile = slot_threads * kXPer, width = tile + 8;     // staged positions of a row
+    const int slot = threadIdx.x >> a.slot_log, p = threadIdx.x & (slot_threads - 1);
+    const int slots = kXYThreads >> a.slot_log;
+    // the strip of this slot; with FROM_TF four slots share one
+    const int64_t strip = FROM_TF ? (int64_t)blockIdx.x * (slots / 4) + slot / 4 : (int64_t)blockIdx.x * slots + slot;
+    const int chan = FROM_TF ? slot & 3 : blockIdx.y;
+    const int64_t n_strips = (int64_t)a.x_tiles * a.strips_y * a.planes;
+    const bool on = strip < n_strips;
+    const int64_t s = on ? strip : 0;
+    const int xt = (int)(s % a.x_tiles), yt = (int)((s / a.x_tiles) % a.strips_y), zt = (int)(s / a.x_tiles / a.strips_y);
+    const int x0 = xt * tile, k0 = yt * a.pairs;
+    const int k1 = on ? min(a.sy / 2, k0 + a.pairs) : k0;        // output row pairs [k0, k1)
+    if (FROM_TF) tf_stage(tf, knots);
+    // loads of a row: positions q, q + step, ... of the slot's (FROM_TF: the strip's) row
+    const int loaders = FROM_TF ? 4 * slot_threads : slot_threads, q = FROM_TF ? threadIdx.x & (loaders - 1) : p;
+    constexpr int LOADS = FROM_TF ? 2 : kXPer + 1;               // 8 more positions than loaders x their share
+    int col[LOADS];
+#pragma unroll
+    for (int i = 0; i < LOADS; i++) col[i] = wrap(x0 - HALO + q + i * loaders, a.sx);
+    const float *plane = a.src + (FROM_TF ? 0 : chan * a.src_chan) + (int64_t)wrap(a.z_first + zt, a.sz) * a.src_plane;
+    int y = wrap(2 * k0 + Wv::FIRST, a.sy);
+    float raw[2][LOADS];
+    auto fetch = [&]() {
+#pragma unroll
+        for (int r = 0; r < 2; r++) {
+            const float *row = plane + (int64_t)y * a.src_row;
+#pragma unroll
+            for (int i = 0; i < LOADS; i++)
+                if (q + i * loaders < width) raw[r][i] = row[col[i]];
+            y = y + 1 == a.sy ? 0 : y + 1;
+        }
+    };
+    auto stage = [&](int buf) {
+#pragma unroll
+        for (int r = 0; r < 2; r++) {
+#pragma unroll
+            for (int i = 0; i < LOADS; i++) {
+                const int at = q + i * loaders;
+                if (at >= width) continue;
+                if (FROM_TF) {
+                    const float4 c = tf_apply(tf, knots, raw[r][i]);
+                    float *to = &rows[buf][r][(slot & ~3) * width + at];
+                    to[0] = c.x;
+                    to[width] = c.y;
+                    to[2 * width] = c.z;
+                    to[3 * width] = c.w;
+                } else {
+                    rows[buf][r][slot * width + at] = raw[r][i];
+                }
+            }
+        }
+    };
+    const int64_t out_plane = (int64_t)zt * a.sx * a.sy;
+    float *dst = a.dst + chan * a.dst_chan + out_plane;
+    const int hx = a.sx >> 1, hy = a.sy >> 1;
+    const int xo = x0 / 2 + 2 * p;                               // low column of the first pair
+    float ring[R][2][4];                                         // x results: low, low, high, high
+    auto x_filter = [&](int buf, float (&out)[2][4]) {
+#pragma unroll
+        for (int r = 0; r < 2; r++) {
+            const float4 *in4 = reinterpret_cast<const float4 *>(&rows[buf][r][slot * width + kXPer * p]);
+            const float4 A = in4[0], B = in4[1], C = in4[2];
+            const float in[12] = {A.x, A.y, A.z, A.w, B.x, B.y, B.z, B.w, C.x, C.y, C.z, C.w};
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                float lo = 0.f, hi = 0.f;
+#pragma unroll
+                for (int t = 0; t < Wv::LO_LEN; t++) lo = __fmaf_rn(w.lo[t], in[HALO + 2 * k + Wv::LO + t], lo);
+#pragma unroll
+                for (int t = 0; t < Wv::HI_LEN; t++) hi = __fmaf_rn(w.hi[t], in[HALO + 2 * k + Wv::HI + t], hi);
+                out[r][k] = lo;
+                out[r][2 + k] = hi;
+            }
+        }
+    };
+    auto put = [&](int row, int column, float u, float v) {      // columns (column, column + 1) of a half
+        float *d = dst + (int64_t)row * a.sx + column;
+        if (a.vec2 && xo + 1 < hx) {
+            *reinterpret_cast<float2 *>(d) = make_float2(u, v);
+        } else {
+            if (xo < hx) d[0] = u;
+            if (xo + 1 < hx) d[1] = v;
+        }
+    };
+    const int steps = a.pairs + R - 1;                           // the same for every slot of the block
+    fetch();
+    __syncthreads();                                             // knots
+    for (int s0 = 0; s0 < steps; s0 += R) {
+#pragma unroll
+        for (int u = 0; u < R; u++) {                            // ring positions are compile-time
+            const int step = s0 + u;
+            if (step >= steps) break;
+            stage(step & 1);
+            if (step + 1 < steps) fetch();
+            __syncthreads();
+            x_filter(step & 1, ring[u]);
+            const int k = k0 + step - (R - 1);
+            if (step < R - 1 || k >= k1) continue;
+            // sample pair i of the window is ring slot (u + 1 + i) mod R
+            float lo[4] = {0.f, 0.f, 0.f, 0.f}, hi[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int t = 0; t < Wv::LO_LEN; t++) {
+                const int i = Wv::LO - Wv::FIRST + t;
+#pragma unroll
+                for (int c = 0; c < 4; c++) lo[c] = __fmaf_rn(w.lo[t], ring[(u + 1 + i / 2) % R][i & 1][c], lo[c]);
+            }
+#pragma unroll
+            for (int t = 0; t < Wv::HI_LEN; t++) {
+                const int i = Wv::HI - Wv::FIRST + t;
+#pragma unroll
+                for (int c = 0; c < 4; c++) hi[c] = __fmaf_rn(w.hi[t], ring[(u + 1 + i / 2) % R][i & 1][c], hi[c]);
+            }
+            put(k, xo, lo[0], lo[1]);
+            put(k, hx + xo, lo[2], lo[3]);
+            put(hy + k, xo, hi[0], hi[1]);
+            put(hy + k, hx + xo, hi[2], hi[3]);
+        }
+    }
+}
+
+// z pass: a thread takes V neighbouring columns of one channel and `pairs`
+// plane pairs, with the 10 planes the filter spans in a register ring and the
+// next pair's loads in flight.  Bound by memory: each value is read and
+// written once (plus the 8 planes of overlap between chunks, from L2).
+struct ZArgs {
+    const float *src;                    // [channel][plane][sy][sx]
+    int64_t src_chan;
+    int planes, z_first;                 // plane t holds z = z_first + t (modulo planes)
+    float *dst;                          // Mallat layout, strides below
+    int64_t dst_chan, dst_plane;
+    int dst_row;
+    int sx, sy, sz;
+    int k_begin, k_end, pairs;           // output pairs of this launch, and of a thread
+};
+
+template <int V>
+struct Vec;
+template <>
+struct Vec<1> { using T = float; };
+template <>
+struct Vec<4> { using T = float4; };
+
+constexpr int kZThreads = 256;
+
+template <int WAVELET, int V>
+__global__ void __launch_bounds__(kZThreads) k_dwt_z(const __grid_constant__ ZArgs a, const __grid_constant__ Taps w)
+{
+    using Wv = Wavelet<WAVELET>;
+    using T = typename Vec<V>::T;
+    constexpr int R = Wv::PAIRS;
+    const int64_t plane = (int64_t)a.sx * a.sy;
+    const int64_t at = ((int64_t)blockIdx.x * kZThreads + threadIdx.x) * V;
+    if (at >= plane) return;
+    const int k0 = a.k_begin + blockIdx.y * a.pairs, k1 = min(a.k_end, k0 + a.pairs);
+    const int y = (int)(at / a.sx), x = (int)(at - (int64_t)y * a.sx);
+    const float *src = a.src + blockIdx.z * a.src_chan + at;
+    float *dst = a.dst + blockIdx.z * a.dst_chan + (int64_t)y * a.dst_row + x;
+    int t = wrap(2 * k0 + Wv::FIRST - a.z_first, a.planes);
+    float ring[R][2][V], next[2][V];
+    auto fetch = [&]() {
+#pragma unroll
+        for (int r = 0; r < 2; r++) {
+            *reinterpret_cast<T *>(next[r]) = *reinterpret_cast<const T *>(src + (int64_t)t * plane);
+            t = t + 1 == a.planes ? 0 : t + 1;
+        }
+    };
+    const int steps = k1 - k0 + R - 1;
+    fetch();
+    for (int s0 = 0; s0 < steps; s0 += R) {
+#pragma unroll
+        for (int u = 0; u < R; u++) {
+            const int step = s0 + u;
+            if (step >= steps) break;
+#pragma unroll
+            for (int r = 0; r < 2; r++)
+#pragma unroll
+                for (int c = 0; c < V; c++) ring[u][r][c] = next[r][c];
+            if (step + 1 < steps) fetch();
+            if (step < R - 1) continue;
+            const int k = k0 + step - (R - 1);
+            float lo[V], hi[V];
+#pragma unroll
+            for (int c = 0; c < V; c++) lo[c] = hi[c] = 0.f;
+#pragma unroll
+            for (int i = 0; i < Wv::LO_LEN; i++) {
+                const int j = Wv::LO - Wv::FIRST + i;
+#pragma unroll
+                for (int c = 0; c < V; c++) lo[c] = __fmaf_rn(w.lo[i], ring[(u + 1 + j / 2) % R][j & 1][c], lo[c]);
+            }
+#pragma unroll
+            for (int i = 0; i < Wv::HI_LEN; i++) {
+                const int j = Wv::HI - Wv::FIRST + i;
+#pragma unroll
+                for (int c = 0; c < V; c++) hi[c] = __fmaf_rn(w.hi[i], ring[(u + 1 + j / 2) % R][j & 1][c], hi[c]);
+            }
+            *reinterpret_cast<T *>(dst + (int64_t)k * a.dst_plane) = *reinterpret_cast<const T *>(lo);
+            *reinterpret_cast<T *>(dst + (int64_t)(a.sz / 2 + k) * a.dst_plane) = *reinterpret_cast<const T *>(hi);
+        }
+    }
+}
+
+constexpr int kTFThreads = 256;
+
+// d_rf = TF(volume): four elements a thread where both arrays allow 16-byte
+// accesses (VEC), one otherwise.
+template <bool VEC>
+__global__ void __launch_bounds__(kTFThreads) k_tf_apply(const float *__restrict__ F, int64_t n,
+                                                         const __grid_constant__ TFDev tf, float *__restrict__ RF)
+{
+    __shared__ float4 knots[16];
+    tf_stage(tf, knots);
+    __syncthreads();
+    const int64_t i = (int64_t)blockIdx.x * kTFThreads + threadIdx.x;
+    if constexpr (VEC) {
+        if (4 * i >= n) return;
+        const float4 f = reinterpret_cast<const float4 *>(F)[i];
+        const float4 a = tf_apply(tf, knots, f.x), b = tf_apply(tf, knots, f.y), c = tf_apply(tf, knots, f.z),
+                     d = tf_apply(tf, knots, f.w);
+        float4 *out = reinterpret_cast<float4 *>(RF) + i;
+        const int64_t step = n / 4;
+        out[0] = make_float4(a.x, b.x, c.x, d.x);
+        out[step] = make_float4(a.y, b.y, c.y, d.y);
+        out[2 * step] = make_float4(a.z, b.z, c.z, d.z);
+        out[3 * step] = make_float4(a.w, b.w, c.w, d.w);
+    } else {
+        if (i >= n) return;
+        const float4 a = tf_apply(tf, knots, F[i]);
+        RF[i] = a.x;
+        RF[n + i] = a.y;
+        RF[2 * n + i] = a.z;
+        RF[3 * n + i] = a.w;
+    }
+}
+
+bool aligned(const void *p, size_t to) { return reinterpret_cast<uintptr_t>(p) % to == 0; }
+
+// Work a strip (row pairs) or a z chunk (plane pairs): the longest, up to
+// `most`, that still leaves `units` threads' worth of parallel work four waves
+// of the chip; the 8 rows or planes of overlap cost 8 / (2 pairs).
+int pairs_per(int total_pairs, int64_t lanes, int most)
+{
+    int per = std::min(most, total_pairs);
+    const int64_t want = (int64_t)num_sms() * 1024;
+    while (per > 4 && lanes * ((total_pairs + per - 1) / per) < want) per = (per + 1) / 2;
+    return std::max(per, 1);
+}
+
+template <int WAVELET, bool FROM_TF>
+vbm_status launch_xy(XYArgs a, int channels, const Taps &w, const TFDev &tf, cudaStream_t st)
+{
+    int log = 3;
+    while ((1 << log) * kXPer < a.sx && (1 << log) < kMaxSlot) log++;
+    a.slot_log = log;
+    const int tile = (1 << log) * kXPer;
+    a.x_tiles = (a.sx + tile - 1) / tile;
+    a.pairs = pairs_per(a.sy / 2, (int64_t)a.x_tiles * a.planes * channels << log, 32);
+    a.strips_y = (a.sy / 2 + a.pairs - 1) / a.pairs;
+    a.vec2 = aligned(a.dst, 8) && (a.sx / 2) % 2 == 0 && a.dst_chan % 2 == 0;
+    const int64_t strips = (int64_t)a.x_tiles * a.strips_y * a.planes;
+    const int per_block = (kXYThreads >> log) / (FROM_TF ? 4 : 1);
+    dim3 grid((unsigned)((strips + per_block - 1) / per_block), FROM_TF ? 1 : channels);
+    k_dwt_xy<WAVELET, FROM_TF><<<grid, kXYThreads, 0, st>>>(a, w, tf);
+    VBM_LAUNCH("dwt_xy");
+    return VBM_OK;
+}
+
+template <int WAVELET>
+vbm_status launch_z(ZArgs a, int channels, const Taps &w, cudaStream_t st)
+{
+    const int64_t plane = (int64_t)a.sx * a.sy;
+    const bool vec = a.sx % 4 == 0 && aligned(a.src, 16) && aligned(a.dst, 16) && a.src_chan % 4 == 0 &&
+                     a.dst_chan % 4 == 0 && a.dst_plane % 4 == 0 && a.dst_row % 4 == 0;
+    const int64_t lanes = vec ? plane / 4 : plane;
+    a.pairs = pairs_per(a.k_end - a.k_begin, lanes * channels, 64);
+    dim3 grid((unsigned)((lanes + kZThreads - 1) / kZThreads),
+              (unsigned)((a.k_end - a.k_begin + a.pairs - 1) / a.pairs), (unsigned)channels);
+    if (vec) k_dwt_z<WAVELET, 4><<<grid, kZThreads, 0, st>>>(a, w);
+    else k_dwt_z<WAVELET, 1><<<grid, kZThreads, 0, st>>>(a, w);
+    VBM_LAUNCH("dwt_z");
+    return VBM_OK;
+}
+
+// One level in place on the region of `channels` channels of data; tmp holds
+// them.
+template <int WAVELET>
+vbm_status dwt_level(float *data, int channels, const int dims[3], int level, float *tmp, const Taps &w,
+                     cudaStream_t st)
+{
+    const int64_t n = (int64_t)dims[0] * dims[1] * dims[2], plane = (int64_t)dims[0] * dims[1];
+    const int sx = dims[0] >> (level - 1), sy = dims[1] >> (level - 1), sz = dims[2] >> (level - 1);
+    XYArgs a{};
+    a.src = data;
+    a.src_chan = n;
+    a.src_plane = plane;
+    a.src_row = dims[0];
+    a.dst = tmp;
+    a.dst_chan = (int64_t)sx * sy * sz;
+    a.sx = sx; a.sy = sy; a.sz = sz;
+    a.planes = sz;
+    vbm_status s = launch_xy<WAVELET, false>(a, channels, w, TFDev{}, st);
+    if (s != VBM_OK) return s;
+    ZArgs z{};
+    z.src = tmp;
+    z.src_chan = a.dst_chan;
+    z.planes = sz;
+    z.dst = data;
+    z.dst_chan = n;
+    z.dst_plane = plane;
+    z.dst_row = dims[0];
+    z.sx = sx; z.sy = sy; z.sz = sz;
+    z.k_end = sz / 2;
+    return launch_z<WAVELET>(z, channels, w, st);
+}
+
+template <int WAVELET>
+vbm_status dwt_levels(float *data, int n_channels, const int dims[3], int first, int levels, float *tmp,
+                      int64_t tmp_floats, const Taps &w, cudaStream_t st)
+{
+    const int64_t n = (int64_t)dims[0] * dims[1] * dims[2];
+    for (int j = first; j <= levels; j++) {
+        const int64_t region = n >> (3 * (j - 1));
+        const int most = (int)std::min<int64_t>(n_channels, std::min<int64_t>(tmp_floats / region, 32768));
+        for (int c = 0; c < n_channels; c += most) {
+            vbm_status s = dwt_level<WAVELET>(data + c * n, std::min(most, n_channels - c), dims, j, tmp, w, st);
+            if (s != VBM_OK) return s;
+        }
+    }
+    return VBM_OK;
+}
+
+// The first level of the RGBA channels straight from the scalar volume, in
+// slabs of planes where tmp does not hold the four channels whole.
+template <int WAVELET>
+vbm_status first_level_tf(const float *volume, const int dims[3], const TFDev &tf, float *A, float *tmp,
+                          int64_t tmp_floats, const Taps &w, cudaStream_t st)
+{
+    using Wv = Wavelet<WAVELET>;
+    const int64_t plane = (int64_t)dims[0] * dims[1], n = plane * dims[2];
+    const int overlap = 2 * (Wv::PAIRS - 1);
+    const int64_t room = tmp_floats / (4 * plane);                   // planes of four channels
+    const bool whole = room >= dims[2];
+    const int slab = whole ? dims[2] / 2 : (int)((room - overlap) / 2);   // output pairs
+    for (int k = 0; k < dims[2] / 2; k += slab) {
+        const int k1 = std::min(dims[2] / 2, k + slab);
+        XYArgs a{};
+        a.src = volume;
+        a.src_plane = plane;
+        a.src_row = dims[0];
+        a.dst = tmp;
+        a.sx = dims[0]; a.sy = dims[1]; a.sz = dims[2];
+        a.z_first = whole ? 0 : 2 * k + Wv::FIRST;
+        a.planes = whole ? dims[2] : 2 * (k1 - k) + overlap;
+        a.dst_chan = plane * a.planes;
+        vbm_status s = launch_xy<WAVELET, true>(a, 4, w, tf, st);
+        if (s != VBM_OK) return s;
+        ZArgs z{};
+        z.src = tmp;
+        z.src_chan = a.dst_chan;
+        z.planes = a.planes;
+        z.z_first = a.z_first;
+        z.dst = A;
+        z.dst_chan = n;
+        z.dst_plane = plane;
+        z.dst_row = dims[0];
+        z.sx = dims[0]; z.sy = dims[1]; z.sz = dims[2];
+        z.k_begin = k;
+        z.k_end = k1;
+        s = launch_z<WAVELET>(z, 4, w, st);
+        if (s != VBM_OK) return s;
+    }
+    return VBM_OK;
+}
+
+}  // namespace
+
+vbm_status tf_apply(const float *volume, int64_t n, const vbm_tf *tf, float *rf, cudaStream_t st)
+{
+    const bool vec = n % 4 == 0 && aligned(volume, 16) && aligned(rf, 16);
+    const int64_t lanes = vec ? n / 4 : n;
+    const unsigned grid = (unsigned)((lanes + kTFThreads - 1) / kTFThreads);
+    if (vec) k_tf_apply<true><<<grid, kTFThreads, 0, st>>>(volume, n, to_dev(tf), rf);
+    else k_tf_apply<false><<<grid, kTFThreads, 0, st>>>(volume, n, to_dev(tf), rf);
+    VBM_LAUNCH("tf_apply");
+    return VBM_OK;
+}
+
+// tmp: at least 2 nx ny nz floats.
+vbm_status dwt_channels(float *data, int n_channels, const int dims[3], int levels, int wavelet, float *tmp,
+                        cudaStream_t st)
+{
+    const int64_t room = 2 * (int64_t)dims[0] * dims[1] * dims[2];
+    const Taps w = make_taps(wavelet);
+    return wavelet == 1 ? dwt_levels<1>(data, n_channels, dims, 1, levels, tmp, room, w, st)
+                        : dwt_levels<0>(data, n_channels, dims, 1, levels, tmp, room, w, st);
+}
+
+// Floats of tmp for pyramid_from_volume: the four channels whole up to 2^26
+// floats (256^3 volumes), beyond that two volumes' worth, worked in slabs.
+int64_t pyramid_tmp_floats(const int dims[3])
+{
+    const int64_t n = (int64_t)dims[0] * dims[1] * dims[2], plane = (int64_t)dims[0] * dims[1];
+    return std::max(std::max(2 * n, std::min<int64_t>(4 * n, 1 << 26)), std::min(4 * n, 4 * plane * 16));
+}
+
+vbm_status pyramid_from_volume(const float *volume, const int dims[3], const vbm_tf *tf, int levels, int wavelet,
+                               float *A, float *tmp, cudaStream_t st)
+{
+    const int64_t room = pyramid_tmp_floats(dims);
+    const Taps w = make_taps(wavelet);
+    const TFDev t = to_dev(tf);
+    vbm_status s = wavelet == 1 ? first_level_tf<1>(volume, dims, t, A, tmp, room, w, st)
+                                : first_level_tf<0>(volume, dims, t, A, tmp, room, w, st);
+    if (s != VBM_OK) return s;
+    return wavelet == 1 ? dwt_levels<1>(A, 4, dims, 2, levels, tmp, room, w, st)
+                        : dwt_levels<0>(A, 4, dims, 2, levels, tmp, room, w, st);
+}
+
+}  // namespace vbm

@@ -406,6 +406,14 @@ struct FilterBank {
 };
 FilterBank make_filters(int wavelet);
 
+// Transfer function and wavelet pyramid (dwt.cu).
+vbm_status tf_apply(const float *volume, int64_t n, const vbm_tf *tf, float *rf, cudaStream_t st);
+vbm_status dwt_channels(float *data, int n_channels, const int dims[3], int levels, int wavelet, float *tmp,
+                        cudaStream_t st);
+int64_t pyramid_tmp_floats(const int dims[3]);
+vbm_status pyramid_from_volume(const float *volume, const int dims[3], const vbm_tf *tf, int levels, int wavelet,
+                               float *A, float *tmp, cudaStream_t st);
+
 // ---------------------------------------------------------------- binning
 // Work-queue counters of the compositing kernels (2), tile-group sizes and
 // cursors of the longest-first order (32 + 32), then the list-segment

@@ -84,3 +84,49 @@ def test_build_workspace_need_not_be_aligned(cuda_lib):
         assert lib.vbm_build(*args, size.value - 1, vbm._stream()) == vbm.VBM_ERR_ARG
         assert lib.vbm_build(*args, size.value, vbm._stream()) == 0
         assert m.value == n and torch.equal(P, want)
+
+
+@pytest.mark.parametrize("dims,J,wavelet", [
+    ((2, 2, 2), 1, 0), ((2, 2, 2), 1, 1),           # every tap wraps, several times round
+    ((6, 10, 14), 1, 0), ((6, 10, 14), 1, 1),       # halves of odd length: no paired stores
+    ((4, 64, 2), 1, 0), ((264, 12, 20), 2, 0),      # one position beyond a 256-wide tile, and then some
+    ((36, 28, 140), 2, 1), ((32, 32, 32), 5, 0),    # regions down to 2^3
+    ((1028, 4, 12), 2, 0), ((8, 520, 8), 3, 0)])
+def test_dwt_edges_match_oracle(cuda_lib, dims, J, wavelet):
+    """Ragged regions of the wavelet passes against the oracle, at an aligned and at an
+    odd address (the same bits); vbm_build's pyramid, whose first level reads the volume
+    through the transfer function, equals tf_apply followed by dwt3d."""
+    from oracle.dwt import dwt3d
+    from oracle.filters import filter_bank
+    vbm = cuda_lib
+    nx, ny, nz = dims
+    n = nx * ny * nz
+    x = np.random.default_rng(n).standard_normal((3, nz, ny, nx)).astype(np.float32)
+    got = []
+    for shift in (0, 1):
+        buf, tmp = torch.zeros(3 * n + shift, device="cuda"), torch.zeros(2 * n + shift, device="cuda")
+        buf[shift:] = torch.from_numpy(x).cuda().reshape(-1)
+        vbm.dwt3d(buf[shift:], 3, dims, J, wavelet, tmp[shift:])
+        got.append(buf[shift:].cpu().numpy().reshape(x.shape))
+    assert np.array_equal(got[0], got[1])
+    ref = np.stack([dwt3d(c.astype(np.float64), J, filter_bank(wavelet)) for c in x])
+    assert np.abs(got[0] - ref).max() < 2e-6 * max(1.0, np.abs(ref).max())
+    _check_build_pyramid(vbm, dims, J, wavelet)
+
+
+@pytest.mark.parametrize("dims,J,wavelet", [((256, 256, 272), 2, 0), ((256, 256, 272), 1, 1), ((1024, 2064, 8), 1, 0)])
+def test_build_pyramid_in_slabs(cuda_lib, dims, J, wavelet):
+    """Volumes whose four channels do not fit the scratch whole go slab by slab: the same bits."""
+    _check_build_pyramid(cuda_lib, dims, J, wavelet)
+
+
+def _check_build_pyramid(vbm, dims, J, wavelet):
+    nx, ny, nz = dims
+    F = torch.rand((nz, ny, nx), generator=torch.Generator(device="cuda").manual_seed(nx), device="cuda") * 1.4 - 0.2
+    tf = vbm.make_tf(TF_KNOTS_X, TF_KNOTS_RGBA)
+    want = torch.empty((4, nz, ny, nx), device="cuda")
+    vbm.tf_apply(F, tf, want)
+    vbm.dwt3d(want, 4, dims, J, wavelet, torch.empty(2 * F.numel(), device="cuda"))
+    coef = torch.empty_like(want)
+    vbm.build(F, dims, tf, vbm.bank_build(J, wavelet), vbm.make_select(100), capacity=F.numel(), coef=coef)
+    assert torch.equal(coef, want)
