@@ -11,8 +11,8 @@
 // the transfer function where the rows are staged, so the four RGBA channels
 // are never stored untransformed.  Against one gather kernel an axis (a 64-bit
 // division and a modulo for every tap, three reads and writes of each value):
-// tf_apply + four-level dwt3d of 4 x 256^3, 4.30 -> 0.43 ms; vbm_build of a
-// 512^3 volume, 36.3 -> 5.7 ms.
+// tf_apply + four-level dwt3d of 4 x 256^3, 4.30 -> 0.39 ms; vbm_build of a
+// 512^3 volume, 36.3 -> 4.6 ms.
 #include "tf_dev.h"
 
 namespace vbm {
@@ -60,6 +60,11 @@ constexpr int kXPer = 4;                 // x positions (two output pairs) a thr
 constexpr int kMaxSlot = 64;             // threads of a slot: 256 positions
 constexpr int kMinSlot = 8;
 
+// Where the rows of the x and y passes come from: an array read one value or
+// (rows of whole, aligned 16-byte words) four values at a time, or the scalar
+// volume through the transfer function.
+enum Source { kScalar, kQuads, kTransfer };
+
 // x and y passes.  A slot of `1 << slot_log` threads takes one strip: a tile
 // of 4 x positions a thread, `pairs` row pairs, one plane, one channel.  Rows
 // enter in order, two at a time: staged in shared memory (double-buffered, the
@@ -68,11 +73,16 @@ constexpr int kMinSlot = 8;
 // register ring of the 10 rows the y filter spans, from which every new row
 // pair gives one low and one high output row.  A row is therefore read once a
 // strip (plus the 8 rows of overlap between strips), not once a tap, and
-// nothing goes to memory between the two passes.
+// nothing goes to memory between the two passes.  The y filter takes a
+// thread's columns in pairs (FP32x2) and rows of whole 16-byte words are
+// staged four values at a time: the kernel is bound by instruction issue, not
+// by the arithmetic itself (4 x 256^3, all levels: 200 -> 170 us; with the
+// transfer function on 512^3, first level: 2.76 -> 1.63 ms).
 //
-// FROM_TF: the source is the scalar volume; four neighbouring slots take the
+// kTransfer: the source is the scalar volume; four neighbouring slots take the
 // four channels of one strip, whose threads share the loads and the transfer
-// function's evaluation.
+// function's evaluation (the two rows' positions in one sequence, so that the
+// 16 beyond the threads cost one warp one more evaluation, not two).
 struct XYArgs {
     const float *src;
     int64_t src_chan, src_plane;         // strides of a channel and a plane
@@ -86,7 +96,7 @@ struct XYArgs {
     int vec2;                            // low and high rows start on 8-byte boundaries
 };
 
-template <int WAVELET, bool FROM_TF>
+template <int WAVELET, int SOURCE>
 __global__ void __launch_bounds__(kXYThreads, 2) k_dwt_xy(const __grid_constant__ XYArgs a,
                                                           const __grid_constant__ Taps w,
                                                           const __grid_constant__ TFDev tf)
@@ -95,96 +105,147 @@ __global__ void __launch_bounds__(kXYThreads, 2) k_dwt_xy(const __grid_constant_
     constexpr int HALO = 4;                                      // staged positions before the tile
     constexpr int R = Wv::PAIRS;
     constexpr int MAX_ROW = kXYThreads * kXPer + 8 * (kXYThreads / kMinSlot);
+    constexpr bool TF = SOURCE == kTransfer;
     __shared__ __align__(16) float rows[2][2][MAX_ROW];          // [buffer][row][slot][position]
-    __shared__ float4 knots[16];
+    __shared__ TFTable table;
     const int slot_threads = 1 << a.slot_log;
     const int tile = slot_threads * kXPer, width = tile + 8;     // staged positions of a row
     const int slot = threadIdx.x >> a.slot_log, p = threadIdx.x & (slot_threads - 1);
     const int slots = kXYThreads >> a.slot_log;
-    // the strip of this slot; with FROM_TF four slots share one
-    const int64_t strip = FROM_TF ? (int64_t)blockIdx.x * (slots / 4) + slot / 4 : (int64_t)blockIdx.x * slots + slot;
-    const int chan = FROM_TF ? slot & 3 : blockIdx.y;
+    // the strip of this slot; with TF four slots share one
+    const int64_t strip = TF ? (int64_t)blockIdx.x * (slots / 4) + slot / 4 : (int64_t)blockIdx.x * slots + slot;
+    const int chan = TF ? slot & 3 : blockIdx.y;
     const int64_t n_strips = (int64_t)a.x_tiles * a.strips_y * a.planes;
     const bool on = strip < n_strips;
     const int64_t s = on ? strip : 0;
     const int xt = (int)(s % a.x_tiles), yt = (int)((s / a.x_tiles) % a.strips_y), zt = (int)(s / a.x_tiles / a.strips_y);
     const int x0 = xt * tile, k0 = yt * a.pairs;
     const int k1 = on ? min(a.sy / 2, k0 + a.pairs) : k0;        // output row pairs [k0, k1)
-    if (FROM_TF) tf_stage(tf, knots);
-    // loads of a row: positions q, q + step, ... of the slot's (FROM_TF: the strip's) row
-    const int loaders = FROM_TF ? 4 * slot_threads : slot_threads, q = FROM_TF ? threadIdx.x & (loaders - 1) : p;
-    constexpr int LOADS = FROM_TF ? 2 : kXPer + 1;               // 8 more positions than loaders x their share
+    if (TF) tf_stage(tf, table);
+    const float *row0 = a.src + (TF ? 0 : chan * a.src_chan) + (int64_t)wrap(a.z_first + zt, a.sz) * a.src_plane;
+    int y = wrap(2 * k0 + Wv::FIRST, a.sy);
+    const float *row = row0 + (int64_t)y * a.src_row;
+    auto next_row = [&]() {
+        y++;
+        row += a.src_row;
+        if (y == a.sy) {
+            y = 0;
+            row = row0;
+        }
+    };
+    // this thread's part of two rows in flight, and where it goes
+    constexpr int LOADS = TF ? 3 : SOURCE == kQuads ? 4 : 2 * (kXPer + 1);
+    float raw[SOURCE == kQuads ? 1 : LOADS];
+    float4 raw4[SOURCE == kQuads ? LOADS : 1];
+    const int loaders = 4 * slot_threads, q = threadIdx.x & (loaders - 1);   // TF: the strip's threads
     int col[LOADS];
 #pragma unroll
-    for (int i = 0; i < LOADS; i++) col[i] = wrap(x0 - HALO + q + i * loaders, a.sx);
-    const float *plane = a.src + (FROM_TF ? 0 : chan * a.src_chan) + (int64_t)wrap(a.z_first + zt, a.sz) * a.src_plane;
-    int y = wrap(2 * k0 + Wv::FIRST, a.sy);
-    float raw[2][LOADS];
+    for (int i = 0; i < LOADS; i++) {
+        if (TF) {
+            const int at = q + i * loaders;
+            col[i] = wrap(x0 - HALO + (at < width ? at : at - width), a.sx);
+        } else if (SOURCE == kQuads) {
+            col[i] = wrap(i & 1 ? (p == 0 ? x0 - HALO : x0 + tile) : x0 + 4 * p, a.sx);
+        } else {
+            col[i] = wrap(x0 - HALO + p + (i >> 1) * slot_threads, a.sx);
+        }
+    }
+    const bool second_is_row1 = q + loaders >= width;            // TF: the row of the second load
     auto fetch = [&]() {
-#pragma unroll
-        for (int r = 0; r < 2; r++) {
-            const float *row = plane + (int64_t)y * a.src_row;
+        const float *r0 = row;
+        next_row();
+        const float *r1 = row;
+        next_row();
+        if constexpr (TF) {
+            raw[0] = r0[col[0]];
+            raw[1] = (second_is_row1 ? r1 : r0)[col[1]];
+            if (q < 16) raw[2] = r1[col[2]];
+        } else if constexpr (SOURCE == kQuads) {
+            raw4[0] = *reinterpret_cast<const float4 *>(r0 + col[0]);
+            raw4[2] = *reinterpret_cast<const float4 *>(r1 + col[2]);
+            if (p < 2) {
+                raw4[1] = *reinterpret_cast<const float4 *>(r0 + col[1]);
+                raw4[3] = *reinterpret_cast<const float4 *>(r1 + col[3]);
+            }
+        } else {
 #pragma unroll
             for (int i = 0; i < LOADS; i++)
-                if (q + i * loaders < width) raw[r][i] = row[col[i]];
-            y = y + 1 == a.sy ? 0 : y + 1;
+                if (p + (i >> 1) * slot_threads < width) raw[i] = (i & 1 ? r1 : r0)[col[i]];
         }
     };
     auto stage = [&](int buf) {
-#pragma unroll
-        for (int r = 0; r < 2; r++) {
+        if constexpr (TF) {
+            // a loop, so that the evaluation is compiled once a step: inlined
+            // three times in each of the five unrolled steps it overran the
+            // instruction cache
+            float *to = &rows[buf][0][(slot & ~3) * width];
+            float v = raw[0];
+            const int count = q < 16 ? 3 : 2;
+#pragma unroll 1
+            for (int i = 0; i < count; i++) {
+                const float4 c = tf_apply(tf, table, v);
+                int at = q + i * loaders;
+                at += at < width ? 0 : MAX_ROW - width;          // the second row
+                to[at] = c.x;
+                to[at + width] = c.y;
+                to[at + 2 * width] = c.z;
+                to[at + 3 * width] = c.w;
+                v = i == 0 ? raw[1] : raw[2];
+            }
+        } else if constexpr (SOURCE == kQuads) {
+            float *to = &rows[buf][0][slot * width];
+            *reinterpret_cast<float4 *>(to + HALO + 4 * p) = raw4[0];
+            *reinterpret_cast<float4 *>(to + MAX_ROW + HALO + 4 * p) = raw4[2];
+            if (p < 2) {
+                const int at = p == 0 ? 0 : HALO + tile;
+                *reinterpret_cast<float4 *>(to + at) = raw4[1];
+                *reinterpret_cast<float4 *>(to + MAX_ROW + at) = raw4[3];
+            }
+        } else {
 #pragma unroll
             for (int i = 0; i < LOADS; i++) {
-                const int at = q + i * loaders;
-                if (at >= width) continue;
-                if (FROM_TF) {
-                    const float4 c = tf_apply(tf, knots, raw[r][i]);
-                    float *to = &rows[buf][r][(slot & ~3) * width + at];
-                    to[0] = c.x;
-                    to[width] = c.y;
-                    to[2 * width] = c.z;
-                    to[3 * width] = c.w;
-                } else {
-                    rows[buf][r][slot * width + at] = raw[r][i];
-                }
+                const int at = p + (i >> 1) * slot_threads;
+                if (at < width) rows[buf][i & 1][slot * width + at] = raw[i];
             }
         }
     };
-    const int64_t out_plane = (int64_t)zt * a.sx * a.sy;
-    float *dst = a.dst + chan * a.dst_chan + out_plane;
     const int hx = a.sx >> 1, hy = a.sy >> 1;
     const int xo = x0 / 2 + 2 * p;                               // low column of the first pair
-    float ring[R][2][4];                                         // x results: low, low, high, high
-    auto x_filter = [&](int buf, float (&out)[2][4]) {
+    float *dst = a.dst + chan * a.dst_chan + (int64_t)zt * a.sx * a.sy + xo;
+    const int64_t high_rows = (int64_t)hy * a.sx;
+    const bool two = a.vec2 && xo + 1 < hx;                      // both pairs exist and can be stored as one
+    float2 ring[R][2][2];                                        // x results: low pair, high pair
+    auto x_filter = [&](int buf, float2 (&out)[2][2]) {
 #pragma unroll
         for (int r = 0; r < 2; r++) {
             const float4 *in4 = reinterpret_cast<const float4 *>(&rows[buf][r][slot * width + kXPer * p]);
             const float4 A = in4[0], B = in4[1], C = in4[2];
             const float in[12] = {A.x, A.y, A.z, A.w, B.x, B.y, B.z, B.w, C.x, C.y, C.z, C.w};
+            float lo[2], hi[2];
 #pragma unroll
             for (int k = 0; k < 2; k++) {
-                float lo = 0.f, hi = 0.f;
+                lo[k] = hi[k] = 0.f;
 #pragma unroll
-                for (int t = 0; t < Wv::LO_LEN; t++) lo = __fmaf_rn(w.lo[t], in[HALO + 2 * k + Wv::LO + t], lo);
+                for (int t = 0; t < Wv::LO_LEN; t++) lo[k] = __fmaf_rn(w.lo[t], in[HALO + 2 * k + Wv::LO + t], lo[k]);
 #pragma unroll
-                for (int t = 0; t < Wv::HI_LEN; t++) hi = __fmaf_rn(w.hi[t], in[HALO + 2 * k + Wv::HI + t], hi);
-                out[r][k] = lo;
-                out[r][2 + k] = hi;
+                for (int t = 0; t < Wv::HI_LEN; t++) hi[k] = __fmaf_rn(w.hi[t], in[HALO + 2 * k + Wv::HI + t], hi[k]);
             }
+            out[r][0] = make_float2(lo[0], lo[1]);
+            out[r][1] = make_float2(hi[0], hi[1]);
         }
     };
-    auto put = [&](int row, int column, float u, float v) {      // columns (column, column + 1) of a half
-        float *d = dst + (int64_t)row * a.sx + column;
-        if (a.vec2 && xo + 1 < hx) {
-            *reinterpret_cast<float2 *>(d) = make_float2(u, v);
+    auto put = [&](float *d, float2 v) {                         // two neighbouring outputs
+        if (two) {
+            *reinterpret_cast<float2 *>(d) = v;
         } else {
-            if (xo < hx) d[0] = u;
-            if (xo + 1 < hx) d[1] = v;
+            if (xo < hx) d[0] = v.x;
+            if (xo + 1 < hx) d[1] = v.y;
         }
     };
     const int steps = a.pairs + R - 1;                           // the same for every slot of the block
+    float *out = dst + (int64_t)k0 * a.sx;
     fetch();
-    __syncthreads();                                             // knots
+    __syncthreads();                                             // the table
     for (int s0 = 0; s0 < steps; s0 += R) {
 #pragma unroll
         for (int u = 0; u < R; u++) {                            // ring positions are compile-time
@@ -194,26 +255,29 @@ __global__ void __launch_bounds__(kXYThreads, 2) k_dwt_xy(const __grid_constant_
             if (step + 1 < steps) fetch();
             __syncthreads();
             x_filter(step & 1, ring[u]);
-            const int k = k0 + step - (R - 1);
-            if (step < R - 1 || k >= k1) continue;
+            if (step < R - 1 || k0 + step - (R - 1) >= k1) continue;
             // sample pair i of the window is ring slot (u + 1 + i) mod R
-            float lo[4] = {0.f, 0.f, 0.f, 0.f}, hi[4] = {0.f, 0.f, 0.f, 0.f};
+            float2 lo[2], hi[2];
+            lo[0] = lo[1] = hi[0] = hi[1] = make_float2(0.f, 0.f);
 #pragma unroll
             for (int t = 0; t < Wv::LO_LEN; t++) {
                 const int i = Wv::LO - Wv::FIRST + t;
 #pragma unroll
-                for (int c = 0; c < 4; c++) lo[c] = __fmaf_rn(w.lo[t], ring[(u + 1 + i / 2) % R][i & 1][c], lo[c]);
+                for (int c = 0; c < 2; c++)
+                    lo[c] = __ffma2_rn(make_float2(w.lo[t], w.lo[t]), ring[(u + 1 + i / 2) % R][i & 1][c], lo[c]);
             }
 #pragma unroll
             for (int t = 0; t < Wv::HI_LEN; t++) {
                 const int i = Wv::HI - Wv::FIRST + t;
 #pragma unroll
-                for (int c = 0; c < 4; c++) hi[c] = __fmaf_rn(w.hi[t], ring[(u + 1 + i / 2) % R][i & 1][c], hi[c]);
+                for (int c = 0; c < 2; c++)
+                    hi[c] = __ffma2_rn(make_float2(w.hi[t], w.hi[t]), ring[(u + 1 + i / 2) % R][i & 1][c], hi[c]);
             }
-            put(k, xo, lo[0], lo[1]);
-            put(k, hx + xo, lo[2], lo[3]);
-            put(hy + k, xo, hi[0], hi[1]);
-            put(hy + k, hx + xo, hi[2], hi[3]);
+            put(out, lo[0]);
+            put(out + hx, lo[1]);
+            put(out + high_rows, hi[0]);
+            put(out + high_rows + hx, hi[1]);
+            out += a.sx;
         }
     }
 }
@@ -307,15 +371,15 @@ template <bool VEC>
 __global__ void __launch_bounds__(kTFThreads) k_tf_apply(const float *__restrict__ F, int64_t n,
                                                          const __grid_constant__ TFDev tf, float *__restrict__ RF)
 {
-    __shared__ float4 knots[16];
-    tf_stage(tf, knots);
+    __shared__ TFTable table;
+    tf_stage(tf, table);
     __syncthreads();
     const int64_t i = (int64_t)blockIdx.x * kTFThreads + threadIdx.x;
     if constexpr (VEC) {
         if (4 * i >= n) return;
         const float4 f = reinterpret_cast<const float4 *>(F)[i];
-        const float4 a = tf_apply(tf, knots, f.x), b = tf_apply(tf, knots, f.y), c = tf_apply(tf, knots, f.z),
-                     d = tf_apply(tf, knots, f.w);
+        const float4 a = tf_apply(tf, table, f.x), b = tf_apply(tf, table, f.y), c = tf_apply(tf, table, f.z),
+                     d = tf_apply(tf, table, f.w);
         float4 *out = reinterpret_cast<float4 *>(RF) + i;
         const int64_t step = n / 4;
         out[0] = make_float4(a.x, b.x, c.x, d.x);
@@ -324,7 +388,7 @@ __global__ void __launch_bounds__(kTFThreads) k_tf_apply(const float *__restrict
         out[3 * step] = make_float4(a.w, b.w, c.w, d.w);
     } else {
         if (i >= n) return;
-        const float4 a = tf_apply(tf, knots, F[i]);
+        const float4 a = tf_apply(tf, table, F[i]);
         RF[i] = a.x;
         RF[n + i] = a.y;
         RF[2 * n + i] = a.z;
@@ -345,7 +409,7 @@ int pairs_per(int total_pairs, int64_t lanes, int most)
     return std::max(per, 1);
 }
 
-template <int WAVELET, bool FROM_TF>
+template <int WAVELET, bool TF>
 vbm_status launch_xy(XYArgs a, int channels, const Taps &w, const TFDev &tf, cudaStream_t st)
 {
     int log = 3;
@@ -353,13 +417,18 @@ vbm_status launch_xy(XYArgs a, int channels, const Taps &w, const TFDev &tf, cud
     a.slot_log = log;
     const int tile = (1 << log) * kXPer;
     a.x_tiles = (a.sx + tile - 1) / tile;
-    a.pairs = pairs_per(a.sy / 2, (int64_t)a.x_tiles * a.planes * channels << log, 32);
+    a.pairs = pairs_per(a.sy / 2, ((int64_t)a.x_tiles * a.planes * channels) << log, 32);
     a.strips_y = (a.sy / 2 + a.pairs - 1) / a.pairs;
     a.vec2 = aligned(a.dst, 8) && (a.sx / 2) % 2 == 0 && a.dst_chan % 2 == 0;
     const int64_t strips = (int64_t)a.x_tiles * a.strips_y * a.planes;
-    const int per_block = (kXYThreads >> log) / (FROM_TF ? 4 : 1);
-    dim3 grid((unsigned)((strips + per_block - 1) / per_block), FROM_TF ? 1 : channels);
-    k_dwt_xy<WAVELET, FROM_TF><<<grid, kXYThreads, 0, st>>>(a, w, tf);
+    const int per_block = (kXYThreads >> log) / (TF ? 4 : 1);
+    dim3 grid((unsigned)((strips + per_block - 1) / per_block), TF ? 1 : channels);
+    // whole 16-byte words: the region's rows wrap at a multiple of four values
+    // and every row starts on a 16-byte boundary
+    const bool quads = a.sx % 4 == 0 && aligned(a.src, 16) && a.src_row % 4 == 0 && a.src_plane % 4 == 0 &&
+                       a.src_chan % 4 == 0;
+    auto kernel = TF ? k_dwt_xy<WAVELET, kTransfer> : quads ? k_dwt_xy<WAVELET, kQuads> : k_dwt_xy<WAVELET, kScalar>;
+    kernel<<<grid, kXYThreads, 0, st>>>(a, w, tf);
     VBM_LAUNCH("dwt_xy");
     return VBM_OK;
 }
