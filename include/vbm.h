@@ -235,16 +235,19 @@ typedef struct {
     int32_t tile_w, tile_h;
     int64_t pair_capacity;
     int32_t flags;
-    int32_t pixels_per_thread;     /* 0 = default (2); 1, 2 or 4 */
-    int32_t group_lanes;           /* 0 = default (32); 4, 8, 16 or 32 lanes per compositing group */
-    int32_t segment_len;           /* persistent plans: the backward walks a tile list longer than
+    int32_t pixels_per_thread;     /* 1, 2 or 4; 0 = the library's choice (2; 1 in the forward of a batch
+                                      below 2^20 pixels) */
+    int32_t group_lanes;           /* 4, 8, 16 or 32 lanes per compositing group; 0 = the library's choice (8) */
+    int32_t segment_len;           /* the backward walks a tile list longer than
                                       this many entries as segments that different warps take at
                                       once (the forward stores each pixel's transmittance and
                                       colour still to come at every segment boundary, and with
                                       VBM_PLAN_RECOMPUTE the tile's final per-pixel state; the
                                       plan holds checkpoints for about 2 pairs per (view, Gaussian)
-                                      item, at most 1 GiB; tiles beyond that are walked whole).  0 = default (256); a positive multiple of 32 up to
-                                      65536; -1 = never split.  Ignored by other plans.  Results
+                                      item, at most 1 GiB; tiles beyond that are walked whole).  0 = the library's choice (256; 64 for a batch
+                                      below 2^20 pixels); a positive multiple of 32 up to
+                                      65536; -1 = never split.  A plan that is not persistent does
+                                      without segments when their memory cannot be had.  Results
                                       equal the unsplit walk's up to FP32 rounding of the
                                       transmittance and of the colour sums. */
     int32_t bwd_pixels_per_thread; /* the backward compositing kernel's own pixels per thread and */
@@ -330,7 +333,7 @@ typedef struct {
     const float *T_final;     /* [V][H][W] (absolute views; NULL in recompute mode) */
     const int32_t *n_contrib; /* [V][H][W]                                         */
     const float *g_splat;     /* [n_items][12] after a backward: du dv dA dB dC dopac dr dg db, 3 unused */
-    const int32_t *seg_count; /* persistent plans, device [4]: backward units of the segmented tiles,
+    const int32_t *seg_count; /* device [4]: backward units of the segmented tiles,
                                  segmented tiles, checkpoint slots requested (may exceed
                                  checkpoint_slots: the tiles that found none were walked whole), -;
                                  NULL when lists are never split */

@@ -182,22 +182,6 @@ vbm_status vbm_plan_create(const vbm_plan_desc *d, vbm_plan **out)
     ALLOC(p->ranges, tiles);
     ALLOC(p->tile_order, tiles);
     ALLOC(p->tile_queue, kTileQueueWords);
-    if ((d->flags & VBM_PLAN_PERSISTENT) && d->segment_len >= 0) {
-        p->seg_len = d->segment_len ? d->segment_len : kDefaultSegmentLen;
-        const int64_t tile_px = (int64_t)d->tile_w * d->tile_h;
-        // boundary slots for about kCheckpointPairsPerItem pairs per item (the
-        // workloads list about two per item before fine-tuning shrinks the
-        // splats, fewer after), one final-state slot per tile in recompute
-        // plans; never more than the pair capacity can use or kCheckpointBytes
-        const bool rc = (d->flags & VBM_PLAN_RECOMPUTE) != 0;
-        const int64_t want = (kCheckpointPairsPerItem * items + p->seg_len - 1) / p->seg_len + (rc ? tiles : 0);
-        const int64_t usable = (pairs + p->seg_len - 1) / p->seg_len * (rc ? 2 : 1);
-        p->ckpt_cap = std::max<int64_t>(1, std::min({want, usable,
-                                                     kCheckpointBytes / (tile_px * (int64_t)sizeof(float4))}));
-        ALLOC(p->ckpt, p->ckpt_cap * tile_px);
-        ALLOC(p->ckpt_base, tiles);
-        ALLOC(p->seg_units, 2 * p->ckpt_cap);
-    }
     if (d->flags & VBM_PLAN_RADIX_SORT) {
         p->radix_blocks = radix_blocks();
         p->scan_blocks = scan_blocks();
@@ -222,6 +206,30 @@ vbm_status vbm_plan_create(const vbm_plan_desc *d, vbm_plan **out)
     ALLOC(p->bin_scratch.long_count, 3);
     ALLOC(p->d_n_pairs, 1);
     ALLOC(p->d_status, 2);
+    if (d->segment_len >= 0) {
+        p->seg_len = d->segment_len ? d->segment_len : default_segment_len(pixels);
+        const int64_t tile_px = (int64_t)d->tile_w * d->tile_h;
+        // boundary slots for about kCheckpointPairsPerItem pairs per item (the
+        // workloads list about two per item before fine-tuning shrinks the
+        // splats, fewer after), one final-state slot per tile in recompute
+        // plans; never more than the pair capacity can use or kCheckpointBytes
+        const bool rc = (d->flags & VBM_PLAN_RECOMPUTE) != 0;
+        const int64_t want = (kCheckpointPairsPerItem * items + p->seg_len - 1) / p->seg_len + (rc ? tiles : 0);
+        const int64_t usable = (pairs + p->seg_len - 1) / p->seg_len * (rc ? 2 : 1);
+        p->ckpt_cap = std::max<int64_t>(1, std::min({want, usable,
+                                                     kCheckpointBytes / (tile_px * (int64_t)sizeof(float4))}));
+        ALLOC(p->ckpt_base, tiles);
+        ALLOC(p->seg_units, 2 * p->ckpt_cap);
+        const vbm_status before = s;
+        ALLOC(p->ckpt, p->ckpt_cap * tile_px);
+        // a plan that did not ask for persistence does without segments rather
+        // than fail for their memory
+        if (before == VBM_OK && s == VBM_ERR_NOMEM && !(d->flags & VBM_PLAN_PERSISTENT)) {
+            cudaGetLastError();
+            s = VBM_OK;
+            p->seg_len = 0;
+        }
+    }
 #undef ALLOC
     if (s != VBM_OK) {
         plan_free(p);

@@ -38,14 +38,16 @@
 //
 // Launch: blocks of kWarps warps; each warp takes work items (tile, region)
 // either by its global warp index or, persistent, from an atomic queue whose
-// items follow the tiles' longest-list-first order.  In persistent plans a
+// items follow the tiles' longest-list-first order.  A
 // tile whose list is longer than the segment length L is walked by the
-// backward as independent units (tile, segment, region) of L entries, taken
+// backward (then always persistent) as independent units (tile, segment, region) of L entries, taken
 // ahead of the whole tiles: the forward stores, per pixel still compositing
 // at each segment boundary, the transmittance and the colour still to come
 // (and, in recompute plans, the tile's final per-pixel state), from which a
 // unit starts its walk; one warp's walk of a very long list otherwise
-// outlasted the rest of the launch.  The backward may run its own pixels per
+// outlasted the rest of the launch (16 x 16 tiles, forward not persistent:
+// backward call of 1 x 128^2 / 3 x 509 x 347 / 8 x 512^2, 189 / 318 / 912 ->
+// 48 / 65 / 378 us).  The backward may run its own pixels per
 // thread and lane groups: its regions are independent of the forward's.
 #include "vbm_internal.h"
 
@@ -929,12 +931,21 @@ __global__ void __launch_bounds__(kWarps * 32)
 // backward compositing kernel; the backward takes the forward's unless the
 // plan sets its own.  Each kernel's warp regions are its own: the backward
 // reads only per-pixel state and tile-indexed checkpoints of the forward.
+//
+// Left to the library (0), the groups have 8 lanes: finer groups skip more of
+// the entries that miss their pixels (forward call of 1 x 128^2 / 8 x 512^2 /
+// 4 x 800^2 with 32 lanes 116 / 493 / 1008, with 8 105 / 431 / 880, with 4 105
+// / 434 / 874 us; segmented backward 48 / 419 / 842, 48 / 378 / 728, 51 / 414
+// / 788 us), and a thread two pixels, or one in the forward of a batch below
+// 2^20 pixels, which two would leave with too few warps (105 -> 96 us on 1 x
+// 128^2; 431 -> 460 us on 8 x 512^2).
 int pixels_per_thread(const vbm_plan *p, bool bwd = false)
 {
     const int th = p->desc.tile_h;
     const int want = bwd && p->desc.bwd_pixels_per_thread > 0 ? p->desc.bwd_pixels_per_thread
                                                                : p->desc.pixels_per_thread;
-    int ppt = want > 0 ? want : 2;
+    const int64_t pixels = (int64_t)p->desc.n_views * p->desc.width * p->desc.height;
+    int ppt = want > 0 ? want : !bwd && pixels < (1 << 20) ? 1 : 2;
     while (ppt > 1 && th % (kRegionRows * ppt) != 0) ppt >>= 1;
     return ppt;
 }
@@ -942,7 +953,7 @@ int pixels_per_thread(const vbm_plan *p, bool bwd = false)
 int group_lanes(const vbm_plan *p, bool bwd = false)
 {
     const int want = bwd && p->desc.bwd_group_lanes > 0 ? p->desc.bwd_group_lanes : p->desc.group_lanes;
-    return want > 0 ? want : 32;
+    return want > 0 ? want : 8;
 }
 
 int regions_per_tile(const vbm_plan *p, int ppt)
@@ -983,7 +994,7 @@ vbm_status launch_fwd(vbm_plan *p, int vb, int vc, const float bg[3], float *img
         kernel<<<(n_items_w + kWarps - 1) / kWarps, kWarps * 32, 0, st>>>(
             nullptr, nullptr, n_items_w, nr, p->ranges, p->pair_item, p->rec, p->desc.width, p->desc.height,
             p->desc.tile_w, p->desc.tile_h, p->TX, p->TY, vb, bg[0], bg[1], bg[2], img, alpha, p->T_final, nc_out,
-            p->prof_n_eval, nullptr, nullptr, 0);
+            p->prof_n_eval, p->ckpt, p->seg_len ? p->ckpt_base : nullptr, p->seg_len);
     }
     VBM_LAUNCH("raster_fwd");
     record_event(p->prof_ev[1], st);
@@ -999,7 +1010,7 @@ vbm_status launch_bwd(vbm_plan *p, int vb, int vc, const float bg[3], const floa
     const int nr = regions_per_tile(p, PPT);
     const int n_items_w = n_tiles * nr;
     record_event(p->prof_ev[2], st);
-    if (p->desc.flags & VBM_PLAN_PERSISTENT) {
+    if ((p->desc.flags & VBM_PLAN_PERSISTENT) || p->seg_len) {
         // a second backward of the same forward finds the backward's queue
         // counter spent: clear it (the binning clears it for the first)
         if (p->bwd_queue_used) VBM_CUDA(cudaMemsetAsync(p->tile_queue + 1, 0, sizeof(int), st));

@@ -39,8 +39,8 @@ constexpr int kScanItems = 16;                        // tiles per thread of a s
 constexpr int kTilesPerChunk = kScanThreads * kScanItems;
 constexpr uint64_t kPadKey = ~0ull;
 
-// Longest-list-first order of the tiles for the persistent compositing
-// kernels: tiles are grouped by floor(log2(length + 1)), longest group first
+// Longest-list-first order of the tiles for the compositing kernels that pull
+// from a work queue: tiles are grouped by floor(log2(length + 1)), longest group first
 // (order within a group is arbitrary; each tile is processed independently).
 // A grid-stride kernel after the range scan counts the groups (and claims the
 // list segments), and the warp sort places each tile into the order before it
@@ -58,7 +58,7 @@ constexpr uint64_t kPadKey = ~0ull;
 // has at least two segments, so the units claimed never exceed twice the slots
 // claimed: seg_units holds 2 ckpt_cap entries.
 struct TileOrder {
-    int *q;              // queue words (NULL: no ordering, non-persistent plans)
+    int *q;              // queue words (NULL: no ordering, non-persistent plans without segments)
     int *order;          // [tiles]
     int seg_len;         // 0: lists are never split
     int final_slot;      // 1 in plans that keep no per-pixel state
@@ -1218,7 +1218,7 @@ vbm_status binning(vbm_plan *p, int vb, int vc, cudaStream_t st)
     const int chunks = bin_chunks(n_tiles);
     // 1. ranges from the per-tile counts of the projection
     TileOrder o{};
-    if (p->desc.flags & VBM_PLAN_PERSISTENT) {
+    if ((p->desc.flags & VBM_PLAN_PERSISTENT) || p->seg_len) {
         o.q = p->tile_queue;
         o.order = p->tile_order;
         o.seg_len = p->seg_len;

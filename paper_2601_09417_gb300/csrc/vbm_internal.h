@@ -422,7 +422,7 @@ vbm_status pyramid_from_volume(const float *volume, const int dims[3], const vbm
 constexpr int kTileQueueWords = 2 + 32 + 32 + 4;
 constexpr int kQSegUnits = 66, kQSegTiles = 67, kQSegSlots = 68, kQSegCursor = 69;
 
-// List segments (persistent plans): a tile whose list is longer than the
+// List segments: a tile whose list is longer than the
 // segment length L is walked by the backward as ceil(len / L) independent
 // work units of L entries.  The forward stores, per pixel of such a tile, the
 // transmittance and the colour still to come at each segment boundary (one
@@ -431,7 +431,14 @@ constexpr int kQSegUnits = 66, kQSegTiles = 67, kQSegSlots = 68, kQSegCursor = 6
 // (transmittance, last contributor) in one more slot, so the backward replays
 // only the short lists.  Checkpoint memory is bounded; tiles that find no
 // free slot are walked whole.
-constexpr int kDefaultSegmentLen = 256;
+// Segment length of a plan that leaves it to the library, by the pixels of its
+// batch.  A batch of fewer than 2^20 pixels (16384 warp regions of 64, about
+// four to a resident warp of the backward) does not fill the chip with whole
+// lists, so it splits finer: backward of 1 x 128^2 / 3 x 509 x 347 / 4 x 256^2
+// at 16 x 16 tiles with segments of 64 against 256: 48 / 65 / 75 against 85 /
+// 116 / 126 us; of 8 x 512^2 and 4 x 800^2: 385 and 801 against 378 and 728
+// us, and their forward, which writes the checkpoints, 10% slower.
+inline int default_segment_len(int64_t pixels) { return pixels < (1 << 20) ? 64 : 256; }
 constexpr int64_t kCheckpointPairsPerItem = 2;
 constexpr int64_t kCheckpointBytes = 1ll << 30;
 
@@ -486,7 +493,7 @@ struct vbm_plan {
     uint32_t *tile_count = nullptr;          // [V * TX * TY] listed pairs per tile, then the placement's
                                              // claim cursor (zero between calls)
     int2 *ranges = nullptr;                  // [V * TX * TY]
-    int *tile_order = nullptr;               // [V * TX * TY] longest list first (persistent mode)
+    int *tile_order = nullptr;               // [V * TX * TY] longest list first
     int *tile_queue = nullptr;               // [kTileQueueWords]: work-queue counters (forward, backward),
                                              // then tile-group sizes and cursors of the ordering
     int seg_len = 0;                         // list segment length L (0: lists are never split)
