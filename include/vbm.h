@@ -196,6 +196,18 @@ VBM_API vbm_status vbm_render_dvr(const float *d_volume, const int dims[3], cons
                           const vbm_camera *d_cams, int n_views, int width, int height, float step,
                           float *d_rgba, void *stream);
 
+/* Workspace bytes of vbm_render_dvr_ws for a volume of dims (one bit per
+ * block of 8^3 cells: 32 KiB for 512^3). */
+VBM_API vbm_status vbm_render_dvr_workspace_size(const int dims[3], size_t *bytes);
+
+/* vbm_render_dvr with scratch (d_ws, 4-byte aligned): the call first marks
+ * the blocks of the volume that the transfer function leaves any opacity in
+ * and its rays then pass over the others.  The images are the same; nothing
+ * is kept in d_ws between calls.  d_ws NULL: vbm_render_dvr. */
+VBM_API vbm_status vbm_render_dvr_ws(const float *d_volume, const int dims[3], const vbm_tf *tf,
+                             const vbm_camera *d_cams, int n_views, int width, int height, float step,
+                             float *d_rgba, void *d_ws, size_t ws_bytes, void *stream);
+
 /* ----------------------------------------------------- fine-tuning step */
 
 /* A raster plan owns every buffer of the splatting forward/backward for a

@@ -51,7 +51,8 @@ vbm_status loss_fwd_bwd(const float *img, const float *target, int n_images, int
 vbm_status adam_step(float *P, const float *G, float *M, float *V, int64_t n, int64_t stride, int32_t *step,
                      const float lrs[5], float beta1, float beta2, float eps, uint32_t *nonfinite, cudaStream_t st);
 vbm_status render_dvr(const float *F, const int dims[3], const vbm_tf *tf, const vbm_camera *cams, int n_views,
-                      int W, int H, float step, float *out, cudaStream_t st);
+                      int W, int H, float step, float *out, void *ws, cudaStream_t st);
+size_t dvr_workspace_bytes(const int dims[3]);
 
 template <typename T>
 static vbm_status plan_alloc(vbm_plan *p, T **ptr, size_t count)
@@ -404,8 +405,17 @@ vbm_status vbm_adam(float *params, const float *grad, float *m, float *v, int64_
     return adam_step(params, grad, m, v, n, stride, step, lrs, beta1, beta2, eps, nonfinite, (cudaStream_t)stream);
 }
 
-vbm_status vbm_render_dvr(const float *volume, const int dims[3], const vbm_tf *tf, const vbm_camera *cams,
-                          int n_views, int width, int height, float step, float *rgba, void *stream)
+vbm_status vbm_render_dvr_workspace_size(const int dims[3], size_t *bytes)
+{
+    VBM_ARG(dims && bytes, "null argument");
+    VBM_ARG(dims[0] > 0 && dims[1] > 0 && dims[2] > 0, "invalid volume size");
+    *bytes = dvr_workspace_bytes(dims);
+    return VBM_OK;
+}
+
+vbm_status vbm_render_dvr_ws(const float *volume, const int dims[3], const vbm_tf *tf, const vbm_camera *cams,
+                             int n_views, int width, int height, float step, float *rgba, void *ws, size_t ws_bytes,
+                             void *stream)
 {
     VBM_ARG(volume && dims && tf && cams && rgba, "null argument");
     VBM_ARG(dims[0] > 0 && dims[1] > 0 && dims[2] > 0, "invalid volume size");
@@ -413,7 +423,15 @@ vbm_status vbm_render_dvr(const float *volume, const int dims[3], const vbm_tf *
     VBM_ARG(step > 0.f, "step must be positive");
     VBM_ARG(tf->n_knots >= 2 && tf->n_knots <= 16, "n_knots must be in [2, 16]");
     for (int i = 1; i < tf->n_knots; i++) VBM_ARG(tf->x[i] > tf->x[i - 1], "TF knots must be ascending");
-    return render_dvr(volume, dims, tf, cams, n_views, width, height, step, rgba, (cudaStream_t)stream);
+    VBM_ARG(!ws || (ws_bytes >= dvr_workspace_bytes(dims) && reinterpret_cast<uintptr_t>(ws) % 4 == 0),
+            "DVR workspace too small or not 4-byte aligned");
+    return render_dvr(volume, dims, tf, cams, n_views, width, height, step, rgba, ws, (cudaStream_t)stream);
+}
+
+vbm_status vbm_render_dvr(const float *volume, const int dims[3], const vbm_tf *tf, const vbm_camera *cams,
+                          int n_views, int width, int height, float step, float *rgba, void *stream)
+{
+    return vbm_render_dvr_ws(volume, dims, tf, cams, n_views, width, height, step, rgba, nullptr, 0, stream);
 }
 
 }  // extern "C"

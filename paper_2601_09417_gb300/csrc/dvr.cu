@@ -1,92 +1,161 @@
 // Emission-absorption ray marching of the supervision images (Sec. 4.4:
 // "we render 64 images through volumetric integration").
 //
-// One thread per pixel, 16 x 16 pixel blocks so neighbouring rays sample
+// One thread per pixel, warps of 8 x 4 pixels so neighbouring rays sample
 // neighbouring voxels (L1/L2 reuse).  Segments of length `step` along the
 // clipped ray, sampled at their midpoints with manual trilinear
 // interpolation (hardware texture filtering uses 8-bit fractional weights,
 // too coarse for 1e-4 images); TF on the interpolated scalar; opacity
-// correction a' = 1 - (1 - a)^len = 1 - exp2(len log2(1 - a)); front to back;
+// correction a' = 1 - (1 - a)^len; front to back;
 // the march stops once T < 1e-6, which changes the result by less than 1e-6.
-#include "vbm_internal.h"
+//
+// Empty space.  Where the transfer function has no opacity a sample adds
+// nothing, and most of a volume is such space.  With a workspace, k_occupancy
+// first marks, one bit a block of 8^3 cells, the blocks that some sample with
+// opacity may lie in; a ray then asks once a block, passes an empty one in a
+// single step and marches an occupied one without further tests.  Only samples
+// whose opacity is 0 are passed over, so the images are those of the full
+// march.  The marks cost one read of the volume.
+#include <type_traits>
+
+#include "tf_dev.h"
 
 namespace vbm {
 namespace {
 
-struct TFDev {
-    int n;
-    float x[16];
-    float rgba[16][4];
+constexpr int kCellShift = 3, kCell = 1 << kCellShift;   // cells of a block along each axis
+constexpr int kOccupancyCols = 32 * kCell;   // columns of one occupancy word
+constexpr int kOccupancyThreads = kOccupancyCols + 32;
+
+// Scalars f <= lo and f >= hi have no opacity: the transfer function's alpha is
+// 0 (or less) from its first knot up to a knot at lo, and from a knot at hi to
+// its last.  The margins cover the rounding of the interpolated value, so that
+// a block all of whose corners lie beyond one of them holds no sample with
+// opacity; with lo = 0 (alpha rises from the first knot) corners of at most 0
+// interpolate to at most 0 exactly.
+struct NoOpacity {
+    float lo, hi;
 };
 
-__device__ __forceinline__ void tf_eval(const TFDev &tf, float f, float out[4])
+NoOpacity no_opacity(const vbm_tf *tf)
 {
-    f = fminf(fmaxf(f, 0.f), 1.f);
-    if (f <= tf.x[0]) {
-#pragma unroll
-        for (int c = 0; c < 4; c++) out[c] = tf.rgba[0][c];
-        return;
-    }
-    if (f >= tf.x[tf.n - 1]) {
-#pragma unroll
-        for (int c = 0; c < 4; c++) out[c] = tf.rgba[tf.n - 1][c];
-        return;
-    }
-    int i = 0;
-    while (i < tf.n - 2 && tf.x[i + 1] <= f) i++;
-    const float t = (f - tf.x[i]) / (tf.x[i + 1] - tf.x[i]);
-#pragma unroll
-    for (int c = 0; c < 4; c++) out[c] = (1.f - t) * tf.rgba[i][c] + t * tf.rgba[i + 1][c];
+    const float inf = std::numeric_limits<float>::infinity();
+    NoOpacity r{-inf, inf};
+    const int n = tf->n_knots;
+    int k = 0;
+    while (k < n && tf->rgba[k][3] <= 0.f) k++;
+    if (k == n) return NoOpacity{inf, inf};                  // no opacity anywhere
+    if (k > 0 && tf->x[k - 1] >= 0.f) r.lo = tf->x[k - 1] * (1.f - 1e-5f);
+    k = n - 1;
+    while (k >= 0 && tf->rgba[k][3] <= 0.f) k--;
+    if (k < n - 1 && tf->x[k + 1] <= 1.f) r.hi = std::max(tf->x[k + 1], 0.f) * (1.f + 1e-5f);
+    return r;
 }
 
-__device__ __forceinline__ float sample(const float *__restrict__ F, int nx, int ny, int nz, float qx, float qy,
-                                        float qz)
+// Occupancy words: bit b of word (bz, by, w) is block (32 w + b, by, bz).  One
+// thread a column of x, over the 9 x 9 rows whose voxels are corners of the
+// blocks' cells; a block then takes its 9 columns.  A voxel that is not
+// comparable (NaN) counts as occupied.
+__global__ void __launch_bounds__(kOccupancyThreads) k_occupancy(const float *__restrict__ F, int nx, int ny, int nz,
+                                                                 NoOpacity none, uint32_t *__restrict__ words)
 {
-    qx = fminf(fmaxf(qx, 0.f), (float)(nx - 1));
-    qy = fminf(fmaxf(qy, 0.f), (float)(ny - 1));
-    qz = fminf(fmaxf(qz, 0.f), (float)(nz - 1));
-    const int x0 = min((int)floorf(qx), max(nx - 2, 0));
-    const int y0 = min((int)floorf(qy), max(ny - 2, 0));
-    const int z0 = min((int)floorf(qz), max(nz - 2, 0));
-    const float fx = qx - x0, fy = qy - y0, fz = qz - z0;
-    const int x1 = min(x0 + 1, nx - 1), y1 = min(y0 + 1, ny - 1), z1 = min(z0 + 1, nz - 1);
-    const int64_t sy = nx, sz = (int64_t)nx * ny;
-    const float c00 = F[z0 * sz + y0 * sy + x0] * (1.f - fx) + F[z0 * sz + y0 * sy + x1] * fx;
-    const float c10 = F[z0 * sz + y1 * sy + x0] * (1.f - fx) + F[z0 * sz + y1 * sy + x1] * fx;
-    const float c01 = F[z1 * sz + y0 * sy + x0] * (1.f - fx) + F[z1 * sz + y0 * sy + x1] * fx;
-    const float c11 = F[z1 * sz + y1 * sy + x0] * (1.f - fx) + F[z1 * sz + y1 * sy + x1] * fx;
-    const float c0 = c00 * (1.f - fy) + c10 * fy;
-    const float c1 = c01 * (1.f - fy) + c11 * fy;
-    return c0 * (1.f - fz) + c1 * fz;
+    __shared__ uint8_t low[kOccupancyCols + 1], high[kOccupancyCols + 1];
+    const int x = blockIdx.x * kOccupancyCols + threadIdx.x;
+    const int y0 = blockIdx.y * kCell, z0 = blockIdx.z * kCell;
+    if (threadIdx.x <= kOccupancyCols) {
+        bool lo = true, hi = true;
+        if (x < nx) {
+            for (int z = z0; z <= min(z0 + kCell, nz - 1); z++) {
+                const float *row = F + ((int64_t)z * ny + y0) * nx + x;
+                float v[kCell + 1];
+#pragma unroll
+                for (int k = 0; k <= kCell; k++) v[k] = row[(int64_t)min(k, ny - 1 - y0) * nx];
+#pragma unroll
+                for (int k = 0; k <= kCell; k++) {
+                    lo &= v[k] <= none.lo;
+                    hi &= v[k] >= none.hi;
+                }
+            }
+        }
+        low[threadIdx.x] = lo;
+        high[threadIdx.x] = hi;
+    }
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    bool lo = true, hi = true;
+#pragma unroll
+    for (int k = 0; k <= kCell; k++) {
+        lo &= low[threadIdx.x * kCell + k] != 0;
+        hi &= high[threadIdx.x * kCell + k] != 0;
+    }
+    const uint32_t word = __ballot_sync(0xffffffffu, !lo && !hi);
+    if (threadIdx.x == 0) words[((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = word;
 }
 
-__global__ void __launch_bounds__(256) k_dvr(const float *__restrict__ F, int nx, int ny, int nz, TFDev tf,
+// Lower cell corner and fraction of a clamped coordinate q (n voxels): adding
+// 2^23 rounding down leaves floor(q) in the low mantissa bits, without
+// conversions.
+constexpr float kFloorMagic = 8388608.f;
+constexpr int kFloorBits = 0x4B000000;
+
+__device__ __forceinline__ int cell_of(float q, float last, float top, float &frac)
+{
+    q = fminf(fmaxf(q, 0.f), last);
+    const float f = fminf(__fadd_rd(q, kFloorMagic), top);
+    frac = q - (f - kFloorMagic);
+    return __float_as_int(f) - kFloorBits;
+}
+
+// The march's roundings are spelled out, so that a ray's samples are the same
+// bits whether or not it passes over empty blocks.
+__device__ __forceinline__ float dot3(float a, float b, float c, float d, float e, float f)
+{
+    return __fmaf_rn(e, f, __fmaf_rn(c, d, __fmul_rn(a, b)));
+}
+
+__device__ __forceinline__ float mix(float a, float wa, float b, float wb)
+{
+    return __fmaf_rn(a, wa, __fmul_rn(b, wb));
+}
+
+// SKIP: use the occupancy words.  WIDE: the volume has more than 2^31 voxels.
+template <bool SKIP, bool WIDE>
+__global__ void __launch_bounds__(256) k_dvr(const float *__restrict__ F, int nx, int ny, int nz,
+                                             const __grid_constant__ TFDev tf, NoOpacity none,
                                              const vbm_camera *__restrict__ cams, int W, int H, float step,
-                                             float *__restrict__ out)
+                                             const uint32_t *__restrict__ words, float *__restrict__ out)
 {
+    using Index = typename std::conditional<WIDE, int64_t, int>::type;
+    __shared__ TFTable table;
+    tf_stage(tf, table);
+    __syncthreads();
     const int v = blockIdx.z;
-    const int px = blockIdx.x * 16 + (threadIdx.x & 15);
-    const int py = blockIdx.y * 16 + (threadIdx.x >> 4);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int px = blockIdx.x * 16 + (warp & 1) * 8 + (lane & 7);
+    const int py = blockIdx.y * 16 + (warp >> 1) * 4 + (lane >> 3);
     if (px >= W || py >= H) return;
     const vbm_camera cam = cams[v];
     const float dcx = (px + 0.5f - cam.cx) / cam.fx, dcy = (py + 0.5f - cam.cy) / cam.fy, dcz = 1.f;
     const float *R = cam.R;
     float d[3], o[3];
 #pragma unroll
-    for (int k = 0; k < 3; k++) d[k] = R[k] * dcx + R[3 + k] * dcy + R[6 + k] * dcz;   // R^T dc
-    const float inv_len = rsqrtf(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+    for (int k = 0; k < 3; k++) d[k] = dot3(R[k], dcx, R[3 + k], dcy, R[6 + k], dcz);   // R^T dc
+    const float inv_len = rsqrtf(dot3(d[0], d[0], d[1], d[1], d[2], d[2]));
 #pragma unroll
     for (int k = 0; k < 3; k++) {
         d[k] *= inv_len;
-        o[k] = -(R[k] * cam.t[0] + R[3 + k] * cam.t[1] + R[6 + k] * cam.t[2]);   // -R^T t
+        o[k] = -dot3(R[k], cam.t[0], R[3 + k], cam.t[1], R[6 + k], cam.t[2]);   // -R^T t
     }
     const float box[3] = {(float)nx, (float)ny, (float)nz};
     float t0 = 0.f, t1 = 3.4e38f;
     bool miss = false;
+    float inv_d[3];
 #pragma unroll
     for (int k = 0; k < 3; k++) {
+        inv_d[k] = 1e30f;
         if (d[k] != 0.f) {
             const float inv = 1.f / d[k];
+            inv_d[k] = inv;
             float ta = (0.f - o[k]) * inv, tb = (box[k] - o[k]) * inv;
             t0 = fmaxf(t0, fminf(ta, tb));
             t1 = fminf(t1, fmaxf(ta, tb));
@@ -98,22 +167,65 @@ __global__ void __launch_bounds__(256) k_dvr(const float *__restrict__ F, int nx
     if (!miss && t1 > t0) {
         const float len = t1 - t0;
         const int nseg = (int)ceilf(len / step);
-        for (int m = 0; m < nseg && T >= 1e-6f; m++) {
-            const float a0 = t0 + m * step;
-            const float seg = fminf(step, t1 - a0);
-            if (!(seg > 0.f)) break;
-            const float tm = a0 + 0.5f * seg;
-            const float val = sample(F, nx, ny, nz, o[0] + tm * d[0] - 0.5f, o[1] + tm * d[1] - 0.5f,
-                                     o[2] + tm * d[2] - 0.5f);
-            float rgba[4];
-            tf_eval(tf, val, rgba);
-            if (rgba[3] <= 0.f) continue;
-            const float ac = rgba[3] >= 1.f ? 1.f : -expm1f(seg * log1pf(-rgba[3]));
-            const float wgt = T * ac;
-            C0 += wgt * rgba[0];
-            C1 += wgt * rgba[1];
-            C2 += wgt * rgba[2];
-            T *= (1.f - ac);
+        const float last[3] = {(float)(nx - 1), (float)(ny - 1), (float)(nz - 1)};
+        // a cell's upper corner exists: the lower one is at most n - 2 (0 where n = 1)
+        const float top[3] = {kFloorMagic + (float)max(nx - 2, 0), kFloorMagic + (float)max(ny - 2, 0),
+                              kFloorMagic + (float)max(nz - 2, 0)};
+        const int dx = nx > 1, dy = ny > 1 ? nx : 0;
+        const Index dz = nz > 1 ? (Index)nx * ny : 0;
+        const float inv_step = 1.f / step;
+        const int word_cols = (nx + kOccupancyCols - 1) / kOccupancyCols, block_rows = (ny + kCell - 1) / kCell;
+        for (int m = 0; m < nseg && T >= 1e-6f;) {
+            int m_end = nseg;
+            if constexpr (SKIP) {
+                const float a0 = __fmaf_rn((float)m, step, t0), tm = __fmaf_rn(0.5f, fminf(step, t1 - a0), a0);
+                float q[3], f;
+                int c[3];
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    q[k] = __fadd_rn(__fmaf_rn(tm, d[k], o[k]), -0.5f);
+                    c[k] = cell_of(q[k], last[k], top[k], f) >> kCellShift;
+                }
+                // samples from m on that lie in this block for certain (0.01
+                // of a step short of the ray's exit covers the rounding)
+                float leave = 1e6f;
+#pragma unroll
+                for (int k = 0; k < 3; k++)
+                    leave = fminf(leave, ((float)(kCell * (c[k] + (d[k] > 0.f))) - q[k]) * inv_d[k]);
+                m_end = m + min(nseg - m, 1 + max(0, (int)fminf(leave * inv_step - 0.01f, 1e6f)));
+                const uint32_t word = words[((int64_t)c[2] * block_rows + c[1]) * word_cols + (c[0] >> 5)];
+                if (!((word >> (c[0] & 31)) & 1u)) {
+                    m = m_end;
+                    continue;
+                }
+            }
+            for (; m < m_end && T >= 1e-6f; m++) {
+                const float a0 = __fmaf_rn((float)m, step, t0);
+                const float seg = fminf(step, t1 - a0);
+                if (!(seg > 0.f)) {
+                    m = nseg;
+                    break;
+                }
+                const float tm = __fmaf_rn(0.5f, seg, a0);
+                float fx, fy, fz;
+                const int x = cell_of(__fadd_rn(__fmaf_rn(tm, d[0], o[0]), -0.5f), last[0], top[0], fx);
+                const int y = cell_of(__fadd_rn(__fmaf_rn(tm, d[1], o[1]), -0.5f), last[1], top[1], fy);
+                const int z = cell_of(__fadd_rn(__fmaf_rn(tm, d[2], o[2]), -0.5f), last[2], top[2], fz);
+                const float *p = F + (((Index)z * ny + y) * nx + x), *r = p + dz;
+                const float gx = 1.f - fx, gy = 1.f - fy;
+                const float c00 = mix(p[0], gx, p[dx], fx), c10 = mix(p[dy], gx, p[dy + dx], fx);
+                const float c01 = mix(r[0], gx, r[dx], fx), c11 = mix(r[dy], gx, r[dy + dx], fx);
+                const float val = mix(mix(c00, gy, c10, fy), 1.f - fz, mix(c01, gy, c11, fy), fz);
+                if (val <= none.lo || val >= none.hi) continue;      // opacity 0
+                const float4 rgba = tf_apply(tf, table, val);
+                if (rgba.w <= 0.f) continue;
+                const float ac = rgba.w >= 1.f ? 1.f : -expm1f(seg * log1pf(-rgba.w));
+                const float wgt = T * ac;
+                C0 = __fmaf_rn(wgt, rgba.x, C0);
+                C1 = __fmaf_rn(wgt, rgba.y, C1);
+                C2 = __fmaf_rn(wgt, rgba.z, C2);
+                T *= 1.f - ac;
+            }
         }
     }
     const int64_t HW = (int64_t)H * W, pix = (int64_t)py * W + px;
@@ -123,19 +235,40 @@ __global__ void __launch_bounds__(256) k_dvr(const float *__restrict__ F, int nx
     out[((int64_t)v * 4 + 3) * HW + pix] = 1.f - T;
 }
 
+dim3 occupancy_grid(const int dims[3])
+{
+    return dim3((dims[0] + kOccupancyCols - 1) / kOccupancyCols, (dims[1] + kCell - 1) / kCell,
+                (dims[2] + kCell - 1) / kCell);
+}
+
 }  // namespace
 
-vbm_status render_dvr(const float *F, const int dims[3], const vbm_tf *tf, const vbm_camera *cams, int n_views,
-                      int W, int H, float step, float *out, cudaStream_t st)
+size_t dvr_workspace_bytes(const int dims[3])
 {
-    TFDev t;
-    t.n = tf->n_knots;
-    for (int i = 0; i < 16; i++) {
-        t.x[i] = tf->x[i];
-        for (int c = 0; c < 4; c++) t.rgba[i][c] = tf->rgba[i][c];
-    }
+    const dim3 g = occupancy_grid(dims);
+    return (size_t)g.x * g.y * g.z * sizeof(uint32_t);
+}
+
+// ws: dvr_workspace_bytes(dims) of scratch, or NULL for a march without the
+// occupancy marks.
+vbm_status render_dvr(const float *F, const int dims[3], const vbm_tf *tf, const vbm_camera *cams, int n_views,
+                      int W, int H, float step, float *out, void *ws, cudaStream_t st)
+{
+    const TFDev t = to_dev(tf);
+    const NoOpacity none = no_opacity(tf);
+    const dim3 marks = occupancy_grid(dims);
+    uint32_t *words = (uint32_t *)ws;
+    if (marks.y > 65535 || marks.z > 65535) words = nullptr;     // beyond a grid's extent
     dim3 grid((W + 15) / 16, (H + 15) / 16, n_views);
-    k_dvr<<<grid, 256, 0, st>>>(F, dims[0], dims[1], dims[2], t, cams, W, H, step, out);
+    const bool wide = (int64_t)dims[0] * dims[1] * dims[2] > INT_MAX;
+    if (words) {
+        k_occupancy<<<marks, kOccupancyThreads, 0, st>>>(F, dims[0], dims[1], dims[2], none, words);
+        VBM_LAUNCH("occupancy");
+        note_launches(1);
+    }
+    auto kernel = words ? (wide ? k_dvr<true, true> : k_dvr<true, false>)
+                        : (wide ? k_dvr<false, true> : k_dvr<false, false>);
+    kernel<<<grid, 256, 0, st>>>(F, dims[0], dims[1], dims[2], t, none, cams, W, H, step, words, out);
     VBM_LAUNCH("render_dvr");
     note_launches(1);
     return VBM_OK;

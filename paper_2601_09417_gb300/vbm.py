@@ -23,7 +23,7 @@ EXPORTED = ["vbm_last_error", "vbm_version", "vbm_bank_build", "vbm_tf_apply", "
             "vbm_plan_destroy", "vbm_plan_check", "vbm_raster_fwd", "vbm_raster_bwd",
             "vbm_plan_get_buffers", "vbm_loss_workspace_size", "vbm_loss", "vbm_adam",
             "vbm_kernel_launches", "vbm_plan_set_profile", "vbm_loss_static", "vbm_bank_ablate",
-            "vbm_peak_probe", "vbm_raster_bwd_adam"]
+            "vbm_peak_probe", "vbm_raster_bwd_adam", "vbm_render_dvr_workspace_size", "vbm_render_dvr_ws"]
 
 
 class VbmError(RuntimeError):
@@ -102,6 +102,9 @@ def load():
                             ctypes.POINTER(Select), V, I64, ctypes.POINTER(I64), V, V, V, S, V]),
         "vbm_render_dvr": (I32, [V, ctypes.POINTER(ctypes.c_int * 3), ctypes.POINTER(TF), V, I32, I32, I32, F32,
                                  V, V]),
+        "vbm_render_dvr_workspace_size": (I32, [ctypes.POINTER(ctypes.c_int * 3), ctypes.POINTER(S)]),
+        "vbm_render_dvr_ws": (I32, [V, ctypes.POINTER(ctypes.c_int * 3), ctypes.POINTER(TF), V, I32, I32, I32, F32,
+                                    V, V, S, V]),
         "vbm_plan_create": (I32, [ctypes.POINTER(PlanDesc), ctypes.POINTER(V)]),
         "vbm_plan_destroy": (I32, [V]),
         "vbm_plan_check": (I32, [V, V, ctypes.POINTER(I64)]),
@@ -252,8 +255,13 @@ def build(volume, dims, tf, bank, sel, capacity, coef=None, keep=None):
 
 
 def render_dvr(volume, dims, tf, cams_dev, n_views, width, height, step, out):
-    _check(load().vbm_render_dvr(_ptr(volume), _dims(dims), ctypes.byref(tf), _ptr(cams_dev), n_views, width,
-                                 height, float(step), _ptr(out), _stream()))
+    import torch
+    lib = load()
+    size = ctypes.c_size_t()
+    _check(lib.vbm_render_dvr_workspace_size(_dims(dims), ctypes.byref(size)))
+    ws = torch.empty(size.value, dtype=torch.uint8, device="cuda")
+    _check(lib.vbm_render_dvr_ws(_ptr(volume), _dims(dims), ctypes.byref(tf), _ptr(cams_dev), n_views, width,
+                                 height, float(step), _ptr(out), _ptr(ws), size.value, _stream()))
 
 
 MAX_PAIR_CAPACITY = (1 << 31) - 1
