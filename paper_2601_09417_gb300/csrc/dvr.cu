@@ -16,8 +16,6 @@
 // single step and marches an occupied one without further tests.  Only samples
 // whose opacity is 0 are passed over, so the images are those of the full
 // march.  The marks cost one read of the volume.
-#include <type_traits>
-
 #include "tf_dev.h"
 
 namespace vbm {
@@ -118,22 +116,78 @@ __device__ __forceinline__ float mix(float a, float wa, float b, float wb)
     return __fmaf_rn(a, wa, __fmul_rn(b, wb));
 }
 
-// SKIP: use the occupancy words.  WIDE: the volume has more than 2^31 voxels.
-template <bool SKIP, bool WIDE>
+// Transfer function and opacity correction as a ray evaluates them, in shared
+// memory.  Interval k of the transfer function: x_k and 1 / (x_{k+1} - x_k),
+// the colour at x_k and its change to the next knot.  corr: the Taylor
+// polynomial of 1 - (1 - a)^step in (a - i / kCorr) kCorr about a = i / kCorr,
+// good to 1e-9 for steps up to kMaxCorrStep and alphas below kMaxCorr; the
+// last segment of a ray (shorter than the step), larger alphas and larger
+// steps evaluate the power itself.
+constexpr int kCorr = 256;
+constexpr int kCorrCells = 192;
+constexpr float kMaxCorr = (float)kCorrCells / kCorr;
+constexpr float kMaxCorrStep = 4.f;
+
+struct MarchTable {
+    float4 rgba[16], change[16];
+    float2 seg[16];
+    float4 corr[kCorrCells];
+};
+
+__device__ __forceinline__ void march_stage(const TFDev &tf, float step, MarchTable &tab)
+{
+    const int i = threadIdx.x;
+    if (i < 16) {
+        const int j = min(i + 1, 15);
+        tab.rgba[i] = make_float4(tf.rgba[i][0], tf.rgba[i][1], tf.rgba[i][2], tf.rgba[i][3]);
+        tab.change[i] = make_float4(tf.rgba[j][0] - tf.rgba[i][0], tf.rgba[j][1] - tf.rgba[i][1],
+                                    tf.rgba[j][2] - tf.rgba[i][2], tf.rgba[j][3] - tf.rgba[i][3]);
+        tab.seg[i] = make_float2(tf.x[i], 1.f / (tf.x[j] - tf.x[i]));
+    }
+    if (i < kCorrCells) {
+        const float a = (float)i / kCorr, log_rest = log1pf(-a), h = 1.f / kCorr, ratio = h / (1.f - a);
+        const float c1 = step * expf((step - 1.f) * log_rest) * h;
+        const float c2 = 0.5f * (1.f - step) * c1 * ratio;
+        tab.corr[i] = make_float4(-expm1f(step * log_rest), c1, c2, (1.f / 3.f) * (2.f - step) * c2 * ratio);
+    }
+}
+
+// Colour and opacity at the scalar f.
+__device__ __forceinline__ float4 march_tf(const TFDev &tf, const MarchTable &tab, float f)
+{
+    f = fminf(fmaxf(f, 0.f), 1.f);
+    if (f <= tf.x[0]) return tab.rgba[0];
+    if (f >= tf.x[tf.n - 1]) return tab.rgba[tf.n - 1];
+    int k = 0;
+#pragma unroll
+    for (int i = 0; i < 6; i++) k += tf.xs[i] <= f;
+    if (tf.n > 8) {
+#pragma unroll
+        for (int i = 6; i < 14; i++) k += tf.xs[i] <= f;
+    }
+    const float2 seg = tab.seg[k];
+    const float4 a = tab.rgba[k], c = tab.change[k];
+    const float t = __fmul_rn(__fsub_rn(f, seg.x), seg.y);
+    return make_float4(__fmaf_rn(t, c.x, a.x), __fmaf_rn(t, c.y, a.y), __fmaf_rn(t, c.z, a.z),
+                       __fmaf_rn(t, c.w, a.w));
+}
+
+// SKIP: use the occupancy words.  GENERAL: any volume; otherwise every edge has
+// at least two voxels and the volume less than 2^30 (32-bit byte offsets).
+template <bool SKIP, bool GENERAL>
 __global__ void __launch_bounds__(256) k_dvr(const float *__restrict__ F, int nx, int ny, int nz,
                                              const __grid_constant__ TFDev tf, NoOpacity none,
                                              const vbm_camera *__restrict__ cams, int W, int H, float step,
                                              const uint32_t *__restrict__ words, float *__restrict__ out)
 {
-    using Index = typename std::conditional<WIDE, int64_t, int>::type;
-    __shared__ TFTable table;
-    tf_stage(tf, table);
+    __shared__ MarchTable table;
+    march_stage(tf, step, table);
     __syncthreads();
     const int v = blockIdx.z;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int px = blockIdx.x * 16 + (warp & 1) * 8 + (lane & 7);
     const int py = blockIdx.y * 16 + (warp >> 1) * 4 + (lane >> 3);
-    if (px >= W || py >= H) return;
+    const bool inside = px < W && py < H;                // every lane stays for the warp's votes
     const vbm_camera cam = cams[v];
     const float dcx = (px + 0.5f - cam.cx) / cam.fx, dcy = (py + 0.5f - cam.cy) / cam.fy, dcz = 1.f;
     const float *R = cam.R;
@@ -164,20 +218,24 @@ __global__ void __launch_bounds__(256) k_dvr(const float *__restrict__ F, int nx
         }
     }
     float C0 = 0.f, C1 = 0.f, C2 = 0.f, T = 1.f;
-    if (!miss && t1 > t0) {
-        const float len = t1 - t0;
-        const int nseg = (int)ceilf(len / step);
-        const float last[3] = {(float)(nx - 1), (float)(ny - 1), (float)(nz - 1)};
-        // a cell's upper corner exists: the lower one is at most n - 2 (0 where n = 1)
-        const float top[3] = {kFloorMagic + (float)max(nx - 2, 0), kFloorMagic + (float)max(ny - 2, 0),
-                              kFloorMagic + (float)max(nz - 2, 0)};
-        const int dx = nx > 1, dy = ny > 1 ? nx : 0;
-        const Index dz = nz > 1 ? (Index)nx * ny : 0;
-        const float inv_step = 1.f / step;
-        const int word_cols = (nx + kOccupancyCols - 1) / kOccupancyCols, block_rows = (ny + kCell - 1) / kCell;
-        for (int m = 0; m < nseg && T >= 1e-6f;) {
-            int m_end = nseg;
-            if constexpr (SKIP) {
+    const bool hit = inside && !miss && t1 > t0;
+    const int nseg = hit ? (int)ceilf((t1 - t0) / step) : 0;
+    const float last[3] = {(float)(nx - 1), (float)(ny - 1), (float)(nz - 1)};
+    // a cell's upper corner exists: the lower one is at most n - 2 (0 where n = 1)
+    const float top[3] = {kFloorMagic + (float)max(nx - 2, 0), kFloorMagic + (float)max(ny - 2, 0),
+                          kFloorMagic + (float)max(nz - 2, 0)};
+    const float table_max = step <= kMaxCorrStep ? kMaxCorr : 0.f;   // alphas below it use the table
+    const int64_t plane = (int64_t)nx * ny;
+    const float *F10 = F + nx, *F01 = F + plane, *F11 = F01 + nx;
+    const float inv_step = 1.f / step;
+    const int word_cols = (nx + kOccupancyCols - 1) / kOccupancyCols, block_rows = (ny + kCell - 1) / kCell;
+    // samples [m, m_end) lie in an occupied block; m = nseg: the ray is done
+    int m = 0, m_end = SKIP ? 0 : nseg;
+    for (;;) {
+        // 1. every ray that has left its block passes to its next occupied one
+        if constexpr (SKIP) {
+            while (__any_sync(0xffffffffu, m < nseg && m >= m_end)) {
+                if (m >= nseg || m < m_end) continue;
                 const float a0 = __fmaf_rn((float)m, step, t0), tm = __fmaf_rn(0.5f, fminf(step, t1 - a0), a0);
                 float q[3], f;
                 int c[3];
@@ -194,40 +252,68 @@ __global__ void __launch_bounds__(256) k_dvr(const float *__restrict__ F, int nx
                     leave = fminf(leave, ((float)(kCell * (c[k] + (d[k] > 0.f))) - q[k]) * inv_d[k]);
                 m_end = m + min(nseg - m, 1 + max(0, (int)fminf(leave * inv_step - 0.01f, 1e6f)));
                 const uint32_t word = words[((int64_t)c[2] * block_rows + c[1]) * word_cols + (c[0] >> 5)];
-                if (!((word >> (c[0] & 31)) & 1u)) {
-                    m = m_end;
-                    continue;
-                }
-            }
-            for (; m < m_end && T >= 1e-6f; m++) {
-                const float a0 = __fmaf_rn((float)m, step, t0);
-                const float seg = fminf(step, t1 - a0);
-                if (!(seg > 0.f)) {
-                    m = nseg;
-                    break;
-                }
-                const float tm = __fmaf_rn(0.5f, seg, a0);
-                float fx, fy, fz;
-                const int x = cell_of(__fadd_rn(__fmaf_rn(tm, d[0], o[0]), -0.5f), last[0], top[0], fx);
-                const int y = cell_of(__fadd_rn(__fmaf_rn(tm, d[1], o[1]), -0.5f), last[1], top[1], fy);
-                const int z = cell_of(__fadd_rn(__fmaf_rn(tm, d[2], o[2]), -0.5f), last[2], top[2], fz);
-                const float *p = F + (((Index)z * ny + y) * nx + x), *r = p + dz;
-                const float gx = 1.f - fx, gy = 1.f - fy;
-                const float c00 = mix(p[0], gx, p[dx], fx), c10 = mix(p[dy], gx, p[dy + dx], fx);
-                const float c01 = mix(r[0], gx, r[dx], fx), c11 = mix(r[dy], gx, r[dy + dx], fx);
-                const float val = mix(mix(c00, gy, c10, fy), 1.f - fz, mix(c01, gy, c11, fy), fz);
-                if (val <= none.lo || val >= none.hi) continue;      // opacity 0
-                const float4 rgba = tf_apply(tf, table, val);
-                if (rgba.w <= 0.f) continue;
-                const float ac = rgba.w >= 1.f ? 1.f : -expm1f(seg * log1pf(-rgba.w));
-                const float wgt = T * ac;
-                C0 = __fmaf_rn(wgt, rgba.x, C0);
-                C1 = __fmaf_rn(wgt, rgba.y, C1);
-                C2 = __fmaf_rn(wgt, rgba.z, C2);
-                T *= 1.f - ac;
+                if (!((word >> (c[0] & 31)) & 1u)) m = m_end;
             }
         }
+        // 2. one sample a round for every ray inside its block, until fewer
+        // than three quarters of the unfinished ones still are
+        const int enough = SKIP ? __popc(__ballot_sync(0xffffffffu, m < nseg)) * 3 / 4 : 0;
+        int going;
+        do {
+            if (m < min(m_end, nseg)) {
+                const float a0 = __fmaf_rn((float)m, step, t0);
+                const float seg = fminf(step, t1 - a0);
+                m++;
+                if (seg > 0.f) {
+                    const float tm = __fmaf_rn(0.5f, seg, a0);
+                    float fx, fy, fz;
+                    const int x = cell_of(__fadd_rn(__fmaf_rn(tm, d[0], o[0]), -0.5f), last[0], top[0], fx);
+                    const int y = cell_of(__fadd_rn(__fmaf_rn(tm, d[1], o[1]), -0.5f), last[1], top[1], fy);
+                    const int z = cell_of(__fadd_rn(__fmaf_rn(tm, d[2], o[2]), -0.5f), last[2], top[2], fz);
+                    const float gx = 1.f - fx, gy = 1.f - fy;
+                    float c00, c10, c01, c11;
+                    if constexpr (GENERAL) {
+                        const float *p = F + (((int64_t)z * ny + y) * nx + x), *r = p + (nz > 1 ? plane : 0);
+                        const int dx = nx > 1, dy = ny > 1 ? nx : 0;
+                        c00 = mix(p[0], gx, p[dx], fx), c10 = mix(p[dy], gx, p[dy + dx], fx);
+                        c01 = mix(r[0], gx, r[dx], fx), c11 = mix(r[dy], gx, r[dy + dx], fx);
+                    } else {
+                        const uint32_t at = ((uint32_t)(z * ny + y) * nx + x) * 4u;
+                        auto row = [&](const float *f) {
+                            const float *p = reinterpret_cast<const float *>(reinterpret_cast<const char *>(f) + at);
+                            return mix(p[0], gx, p[1], fx);
+                        };
+                        c00 = row(F), c10 = row(F10), c01 = row(F01), c11 = row(F11);
+                    }
+                    const float val = mix(mix(c00, gy, c10, fy), 1.f - fz, mix(c01, gy, c11, fy), fz);
+                    if (!(val <= none.lo || val >= none.hi)) {       // otherwise no opacity
+                        const float4 rgba = march_tf(tf, table, val);
+                        if (rgba.w > 0.f) {
+                            float ac = 1.f;
+                            if (seg == step && rgba.w < table_max) {
+                                const float u = rgba.w * kCorr, i = floorf(u), e = u - i;
+                                const float4 c = table.corr[(int)i];
+                                ac = __fmaf_rn(e, __fmaf_rn(e, __fmaf_rn(e, c.w, c.z), c.y), c.x);
+                            } else if (rgba.w < 1.f) {
+                                ac = -expm1f(seg * log1pf(-rgba.w));
+                            }
+                            const float wgt = T * ac;
+                            C0 = __fmaf_rn(wgt, rgba.x, C0);
+                            C1 = __fmaf_rn(wgt, rgba.y, C1);
+                            C2 = __fmaf_rn(wgt, rgba.z, C2);
+                            T *= 1.f - ac;
+                            if (T < 1e-6f) m = nseg;
+                        }
+                    }
+                } else {
+                    m = nseg;
+                }
+            }
+            going = __popc(__ballot_sync(0xffffffffu, m < min(m_end, nseg)));
+        } while (going > enough);
+        if (going == 0 && !__any_sync(0xffffffffu, m < nseg)) break;
     }
+    if (!inside) return;
     const int64_t HW = (int64_t)H * W, pix = (int64_t)py * W + px;
     out[((int64_t)v * 4 + 0) * HW + pix] = C0;
     out[((int64_t)v * 4 + 1) * HW + pix] = C1;
@@ -260,14 +346,15 @@ vbm_status render_dvr(const float *F, const int dims[3], const vbm_tf *tf, const
     uint32_t *words = (uint32_t *)ws;
     if (marks.y > 65535 || marks.z > 65535) words = nullptr;     // beyond a grid's extent
     dim3 grid((W + 15) / 16, (H + 15) / 16, n_views);
-    const bool wide = (int64_t)dims[0] * dims[1] * dims[2] > INT_MAX;
+    const bool general = std::min({dims[0], dims[1], dims[2]}) < 2 ||
+                         (int64_t)dims[0] * dims[1] * dims[2] >= (int64_t)1 << 30;
     if (words) {
         k_occupancy<<<marks, kOccupancyThreads, 0, st>>>(F, dims[0], dims[1], dims[2], none, words);
         VBM_LAUNCH("occupancy");
         note_launches(1);
     }
-    auto kernel = words ? (wide ? k_dvr<true, true> : k_dvr<true, false>)
-                        : (wide ? k_dvr<false, true> : k_dvr<false, false>);
+    auto kernel = words ? (general ? k_dvr<true, true> : k_dvr<true, false>)
+                        : (general ? k_dvr<false, true> : k_dvr<false, false>);
     kernel<<<grid, 256, 0, st>>>(F, dims[0], dims[1], dims[2], t, none, cams, W, H, step, words, out);
     VBM_LAUNCH("render_dvr");
     note_launches(1);
