@@ -103,6 +103,14 @@ __device__ __forceinline__ bool tile_listed(float u, float v, float A, float B, 
     return tile_min_q(u, v, A, B, C, bc, ba, x0, x1, y0, y1) <= tau;
 }
 
+// a / b and sqrt(x), correctly rounded.  A zero operand is taken out first: its
+// result is itself (with the sign), but the division's and the root's range
+// checks send it to their slow path, and many gradients are exactly zero
+// (splats that no pixel sees): a warp with one such lane paid for the slow
+// path of each of the 56 divisions and roots of a Gaussian.
+__device__ __forceinline__ float div_rn(float a, float b) { return a == 0.f && b > 0.f ? a : __fdiv_rn(a, b); }
+__device__ __forceinline__ float sqrt_rn(float x) { return x == 0.f ? x : __fsqrt_rn(x); }
+
 // One Adam update of a scalar (p, m, v in place; Sec. 5.2 trains with Adam);
 // false when g is not finite (nothing is changed).  Every rounding is
 // explicit, so the separate Adam kernels and the backward fused with Adam
@@ -113,9 +121,9 @@ __device__ __forceinline__ bool adam_elem(float &p, float &m, float &v, float g,
     if (!isfinite(g)) return false;
     m = __fmaf_rn(beta1, m, __fmul_rn(1.f - beta1, g));
     v = __fmaf_rn(beta2, v, __fmul_rn(__fmul_rn(1.f - beta2, g), g));
-    const float mhat = __fdiv_rn(m, bc1);
-    const float vhat = __fdiv_rn(v, bc2);
-    p = __fsub_rn(p, __fdiv_rn(__fmul_rn(lr, mhat), __fadd_rn(__fsqrt_rn(vhat), eps)));
+    const float mhat = div_rn(m, bc1);
+    const float vhat = div_rn(v, bc2);
+    p = __fsub_rn(p, div_rn(__fmul_rn(lr, mhat), __fadd_rn(sqrt_rn(vhat), eps)));
     return true;
 }
 
