@@ -110,19 +110,12 @@ __global__ void k_adam_rows(float *__restrict__ P, const float *__restrict__ G, 
 
 }  // namespace
 
-vbm_status adam_step_inc(int32_t *step, cudaStream_t st)
+vbm_status adam_step(float *P, const float *G, float *M, float *V, int64_t n, int64_t stride, int32_t *step,
+                     const float lrs[5], float beta1, float beta2, float eps, uint32_t *nonfinite, cudaStream_t st)
 {
     k_step_inc<<<1, 32, 0, st>>>(step);
     VBM_LAUNCH("adam_step_inc");
     note_launches(1);
-    return VBM_OK;
-}
-
-vbm_status adam_step(float *P, const float *G, float *M, float *V, int64_t n, int64_t stride, int32_t *step,
-                     const float lrs[5], float beta1, float beta2, float eps, uint32_t *nonfinite, cudaStream_t st)
-{
-    vbm_status s = adam_step_inc(step, st);
-    if (s != VBM_OK) return s;
     if (n == 0) return VBM_OK;
     const bool flat = stride == n && ((reinterpret_cast<uintptr_t>(P) | reinterpret_cast<uintptr_t>(G) |
                                        reinterpret_cast<uintptr_t>(M) | reinterpret_cast<uintptr_t>(V)) & 15) == 0;

@@ -207,6 +207,7 @@ vbm_status vbm_plan_create(const vbm_plan_desc *d, vbm_plan **out)
     ALLOC(p->bin_scratch.long_count, 3);
     ALLOC(p->d_n_pairs, 1);
     ALLOC(p->d_status, 2);
+    ALLOC(p->d_bias, 1);
     if (d->segment_len >= 0) {
         p->seg_len = d->segment_len ? d->segment_len : default_segment_len(pixels);
         const int64_t tile_px = (int64_t)d->tile_w * d->tile_h;
@@ -323,7 +324,7 @@ vbm_status vbm_raster_bwd(vbm_plan *p, const float *params, int64_t stride, cons
     VBM_ARG(vb == p->last_view_begin && vc == p->last_view_count,
             "backward views differ from the last forward call on this plan");
     cudaStream_t st = (cudaStream_t)stream;
-    s = raster_bwd(p, params, stride, vb, vc, bg, dimg, dalpha, grad, st);
+    s = raster_bwd(p, vb, vc, bg, dimg, dalpha, nullptr, st);
     if (s == VBM_OK) s = preprocess_bwd(p, params, stride, cams, vb, vc, grad, accumulate, st);
     record_event(p->prof_ev[6], st);
     return s;
@@ -352,8 +353,8 @@ vbm_status vbm_raster_bwd_adam(vbm_plan *p, float *params, int64_t stride, const
     a.beta2 = beta2;
     a.eps = eps;
     a.nonfinite = nonfinite;
-    s = raster_bwd(p, params, stride, vb, vc, bg, dimg, dalpha, nullptr, st);
-    if (s == VBM_OK) s = adam_step_inc(step, st);
+    a.bias = p->d_bias;
+    s = raster_bwd(p, vb, vc, bg, dimg, dalpha, &a, st);
     if (s == VBM_OK) s = preprocess_bwd(p, params, stride, cams, vb, vc, nullptr, 0, st, &a);
     record_event(p->prof_ev[6], st);
     return s;

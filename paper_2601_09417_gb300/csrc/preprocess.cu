@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(256, 4)
 __device__ __forceinline__ void adam_gaussian(const AdamArgs &a, int64_t stride, int64_t g, const float (&g14)[14],
                                               bool seen)
 {
-    const float2 bc = adam_bias_corrections(*a.step, a.beta1, a.beta2);
+    const float2 bc = *a.bias;
     uint32_t bad = 0;
 #pragma unroll
     for (int k0 = 0; k0 < 14; k0 += 7) {

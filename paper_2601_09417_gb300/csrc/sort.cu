@@ -199,6 +199,70 @@ __global__ void __launch_bounds__(kScanThreads) k_tile_scan(uint32_t *__restrict
     }
 }
 
+// The three steps above and the group counting of k_tile_group_count for a call
+// of at most kTilesPerChunk tiles, in one block: sums, ranges, length groups
+// and segment claims, with the queue words in shared memory until the end (the
+// claims' atomics then cost shared-memory latency).  A small image's step is
+// bound by its chain of launches: one instead of three.
+__global__ void __launch_bounds__(kScanThreads) k_tile_scan_small(uint32_t *__restrict__ tile_count, int n_tiles,
+                                                                  int64_t capacity, int2 *__restrict__ ranges,
+                                                                  int64_t *__restrict__ n_pairs,
+                                                                  int64_t *__restrict__ status,
+                                                                  uint32_t *__restrict__ long_count, TileOrder o)
+{
+    __shared__ int64_t warp_sum[kScanThreads / 32];
+    __shared__ int q[kTileQueueWords];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < kTileQueueWords; i += kScanThreads) q[i] = 0;
+    // consecutive tiles of a thread, spread over all threads
+    const int per = (n_tiles + kScanThreads - 1) / kScanThreads, t0 = threadIdx.x * per;
+    uint32_t c[kScanItems];
+    int64_t local = 0;
+#pragma unroll
+    for (int it = 0; it < kScanItems; it++) {
+        c[it] = it < per && t0 + it < n_tiles ? tile_count[t0 + it] : 0u;
+        local += c[it];
+    }
+    int64_t incl = local;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int64_t y = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += y;
+    }
+    if (lane == 31) warp_sum[warp] = incl;
+    __syncthreads();
+    int64_t run = incl - local, total = 0;
+    for (int w = 0; w < kScanThreads / 32; w++) {
+        if (w < warp) run += warp_sum[w];
+        total += warp_sum[w];
+    }
+    const bool overflow = total > capacity;
+    if (threadIdx.x == 0) {
+        *n_pairs = overflow ? 0 : total;
+        long_count[0] = long_count[1] = long_count[2] = 0;
+        if (overflow) {
+            atomicOr((unsigned long long *)&status[0], (unsigned long long)kStatusCapacity);
+            atomicMax((unsigned long long *)&status[1], (unsigned long long)total);
+        }
+    }
+    TileOrder so = o;
+    so.q = q;
+#pragma unroll
+    for (int it = 0; it < kScanItems; it++) {
+        const int t = t0 + it;
+        if (it >= per || t >= n_tiles) break;
+        const int len = overflow ? 0 : (int)c[it];
+        ranges[t] = len ? make_int2((int)run, (int)run + len) : make_int2(0, 0);
+        if (overflow) tile_count[t] = 0u;
+        else if (len) tile_count[t] = (uint32_t)run + (uint32_t)len;   // claim cursor: the range's end
+        run += len;
+        if (o.q && !(o.ckpt_base && claim_segments(len, t, so))) atomicAdd(&q[2 + length_group(len)], 1);
+    }
+    __syncthreads();
+    if (o.q)
+        for (int i = threadIdx.x; i < kTileQueueWords; i += kScanThreads) o.q[i] = q[i];
+}
+
 // Tile counts of each length group and the list-segment claims, one tile per
 // thread over a grid-stride loop (segmented tiles are placed ahead of the
 // groups); one shared atomic per group among a warp's lanes.  A kernel of its
@@ -1227,19 +1291,26 @@ vbm_status binning(vbm_plan *p, int vb, int vc, cudaStream_t st)
         o.ckpt_base = p->seg_len ? p->ckpt_base : nullptr;
         o.seg_units = p->seg_units;
     }
-    k_tile_chunk_sums<<<chunks, kScanThreads, 0, st>>>(p->tile_count, n_tiles, b.chunk_sums, o.q);
-    VBM_LAUNCH("tile_chunk_sums");
-    k_tile_scan<<<chunks, kScanThreads, 0, st>>>(p->tile_count, n_tiles, b.chunk_sums, chunks,
-                                                 p->desc.pair_capacity, p->ranges, p->d_n_pairs, p->d_status,
-                                                 b.long_count);
-    VBM_LAUNCH("tile_scan");
-    note_launches(2);
-    if (o.q) {
-        const int og = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms() * 4,
-                                                                   (n_tiles + kScanThreads - 1) / kScanThreads));
-        k_tile_group_count<<<og, kScanThreads, 0, st>>>(p->ranges, n_tiles, o);
-        VBM_LAUNCH("tile_group_count");
+    if (chunks == 1) {
+        k_tile_scan_small<<<1, kScanThreads, 0, st>>>(p->tile_count, (int)n_tiles, p->desc.pair_capacity, p->ranges,
+                                                      p->d_n_pairs, p->d_status, b.long_count, o);
+        VBM_LAUNCH("tile_scan_small");
         note_launches(1);
+    } else {
+        k_tile_chunk_sums<<<chunks, kScanThreads, 0, st>>>(p->tile_count, n_tiles, b.chunk_sums, o.q);
+        VBM_LAUNCH("tile_chunk_sums");
+        k_tile_scan<<<chunks, kScanThreads, 0, st>>>(p->tile_count, n_tiles, b.chunk_sums, chunks,
+                                                     p->desc.pair_capacity, p->ranges, p->d_n_pairs, p->d_status,
+                                                     b.long_count);
+        VBM_LAUNCH("tile_scan");
+        note_launches(2);
+        if (o.q) {
+            const int og = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms() * 4,
+                                                                       (n_tiles + kScanThreads - 1) / kScanThreads));
+            k_tile_group_count<<<og, kScanThreads, 0, st>>>(p->ranges, n_tiles, o);
+            VBM_LAUNCH("tile_group_count");
+            note_launches(1);
+        }
     }
     const bool radix = (p->desc.flags & VBM_PLAN_RADIX_SORT) != 0;
     if (radix) {
@@ -1276,14 +1347,17 @@ vbm_status binning(vbm_plan *p, int vb, int vc, cudaStream_t st)
                                                                    kSortWarps * 32, 0));
             medium_per_sm = std::max(medium_per_sm, 1);
         }
-        k_tile_sort_medium<<<num_sms() * medium_per_sm, kSortWarps * 32, 0, st>>>(
+        // a queue holds at most the call's tiles: no more blocks than those
+        const int medium = (int)std::min<int64_t>((int64_t)num_sms() * medium_per_sm,
+                                                  (n_tiles + kSortWarps - 1) / kSortWarps);
+        k_tile_sort_medium<<<medium, kSortWarps * 32, 0, st>>>(
             p->ranges, n_tiles, p->pair_key, p->pair_tile, p->pair_item, b.long_tiles, b.long_count);
         VBM_LAUNCH("tile_sort_medium");
         note_launches(1);
-        k_tile_sort_mid<<<num_sms() * 8, kMidSortThreads, 0, st>>>(p->ranges, p->pair_key, p->pair_tile,
-                                                                    p->pair_item, b.long_tiles, b.long_count);
+        k_tile_sort_mid<<<(int)std::min<int64_t>(num_sms() * 8, n_tiles), kMidSortThreads, 0, st>>>(
+            p->ranges, p->pair_key, p->pair_tile, p->pair_item, b.long_tiles, b.long_count);
         VBM_LAUNCH("tile_sort_mid");
-        k_tile_sort_block<<<num_sms() * 2, kBlockSortThreads, kBlockSortSmem, st>>>(
+        k_tile_sort_block<<<(int)std::min<int64_t>(num_sms() * 2, n_tiles), kBlockSortThreads, kBlockSortSmem, st>>>(
             p->ranges, p->pair_key, p->pair_tile, p->pair_item, b.long_tiles, b.long_count, n_tiles);
         VBM_LAUNCH("tile_sort_block");
         note_launches(2);

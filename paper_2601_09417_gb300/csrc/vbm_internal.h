@@ -50,11 +50,15 @@ constexpr int kProfileEvents = 7;       // timing events a plan can record (vbm_
 
 // Adam step fused into the projection backward (vbm_raster_bwd_adam): the
 // first n columns of P, M, V ([14][stride], updated in place), the device
-// step counter (already incremented for this step), per-row-group learning
-// rates, and the optional non-finite gradient counter.
+// step counter, per-row-group learning
+// rates, and the optional non-finite gradient counter.  The backward
+// compositing kernel, which runs before, increments the counter and leaves the
+// step's bias corrections in bias (one launch less, and no two powers a
+// Gaussian).
 struct AdamArgs {
     float *P = nullptr, *M = nullptr, *V = nullptr;
-    const int32_t *step = nullptr;
+    int32_t *step = nullptr;
+    float2 *bias = nullptr;
     int64_t n = 0;
     float lr[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
     float beta1 = 0.f, beta2 = 0.f, eps = 0.f;
@@ -530,6 +534,7 @@ struct vbm_plan {
     vbm::BinScratch bin_scratch;
     int64_t *d_n_pairs = nullptr;            // pairs of the last call
     int64_t *d_status = nullptr;             // [0] status bits, [1] max pairs needed
+    float2 *d_bias = nullptr;                // Adam bias corrections of the fused step
 
     // profiling hooks
     cudaEvent_t prof_ev[vbm::kProfileEvents] = {};
@@ -547,9 +552,8 @@ vbm_status preprocess_fwd(vbm_plan *p, const float *params, int64_t stride, cons
                           cudaStream_t st);
 vbm_status binning(vbm_plan *p, int vb, int vc, cudaStream_t st);
 vbm_status raster_fwd(vbm_plan *p, int vb, int vc, const float bg[3], float *img, float *alpha, cudaStream_t st);
-vbm_status raster_bwd(vbm_plan *p, const float *params, int64_t stride, int vb, int vc, const float bg[3],
-                      const float *dimg, const float *dalpha, float *grad, cudaStream_t st);
+vbm_status raster_bwd(vbm_plan *p, int vb, int vc, const float bg[3], const float *dimg, const float *dalpha,
+                      const AdamArgs *adam, cudaStream_t st);
 vbm_status preprocess_bwd(vbm_plan *p, const float *params, int64_t stride, const vbm_camera *cams, int vb, int vc,
                           float *grad, int accumulate, cudaStream_t st, const AdamArgs *adam = nullptr);
-vbm_status adam_step_inc(int32_t *step, cudaStream_t st);
 }  // namespace vbm
