@@ -199,11 +199,11 @@ __global__ void __launch_bounds__(kScanThreads) k_tile_scan(uint32_t *__restrict
     }
 }
 
-// The three steps above and the group counting of k_tile_group_count for a call
-// of at most kTilesPerChunk tiles, in one block: sums, ranges, length groups
-// and segment claims, with the queue words in shared memory until the end (the
-// claims' atomics then cost shared-memory latency).  A small image's step is
-// bound by its chain of launches: one instead of three.
+// The two kernels above, the group counting of k_tile_group_count and the
+// tiles' order for a call of at most kTilesPerChunk tiles, in one block: sums,
+// ranges, length groups and segment claims, with the queue words in shared
+// memory until the end (the claims' atomics then cost shared-memory latency).
+// A small image's step is bound by its chain of launches.
 __global__ void __launch_bounds__(kScanThreads) k_tile_scan_small(uint32_t *__restrict__ tile_count, int n_tiles,
                                                                   int64_t capacity, int2 *__restrict__ ranges,
                                                                   int64_t *__restrict__ n_pairs,
@@ -247,6 +247,7 @@ __global__ void __launch_bounds__(kScanThreads) k_tile_scan_small(uint32_t *__re
     }
     TileOrder so = o;
     so.q = q;
+    uint32_t segmented = 0;              // bit it: the thread's it-th tile
 #pragma unroll
     for (int it = 0; it < kScanItems; it++) {
         const int t = t0 + it;
@@ -256,11 +257,33 @@ __global__ void __launch_bounds__(kScanThreads) k_tile_scan_small(uint32_t *__re
         if (overflow) tile_count[t] = 0u;
         else if (len) tile_count[t] = (uint32_t)run + (uint32_t)len;   // claim cursor: the range's end
         run += len;
-        if (o.q && !(o.ckpt_base && claim_segments(len, t, so))) atomicAdd(&q[2 + length_group(len)], 1);
+        if (!o.q) continue;
+        if (o.ckpt_base && claim_segments(len, t, so)) segmented |= 1u << it;
+        else atomicAdd(&q[2 + length_group(len)], 1);
+    }
+    if (!o.q) return;                    // grid-uniform
+    __syncthreads();
+    __shared__ int base[32];
+    if (threadIdx.x < 32) {
+        const int cnt = q[2 + lane];
+        int before = cnt;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, before, off);
+            if (lane >= off) before += y;
+        }
+        base[lane] = before - cnt + q[kQSegTiles];
     }
     __syncthreads();
-    if (o.q)
-        for (int i = threadIdx.x; i < kTileQueueWords; i += kScanThreads) o.q[i] = q[i];
+#pragma unroll
+    for (int it = 0; it < kScanItems; it++) {
+        const int t = t0 + it;
+        if (it >= per || t >= n_tiles) break;
+        const int g = length_group(overflow ? 0 : (int)c[it]);
+        o.order[(segmented >> it) & 1u ? atomicAdd(&q[kQSegCursor], 1) : base[g] + atomicAdd(&q[34 + g], 1)] = t;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kTileQueueWords; i += kScanThreads) o.q[i] = q[i];
 }
 
 // Tile counts of each length group and the list-segment claims, one tile per
@@ -702,6 +725,46 @@ __global__ void __launch_bounds__(kMidSortThreads) k_tile_sort_mid(const int2 *_
         for (int i = t; i < n; i += kMidSortThreads) write_sorted(src[padded(i)], r.x + i, tile, pair_tile, pair_item);
         __syncthreads();
     }
+}
+
+// Every list of a small call (k_tile_scan_small has ordered its tiles), one
+// 128-thread block a tile: up to 32 keys by a warp in registers, up to
+// kMidSortMax by the block; longer ones are queued for k_tile_sort_block.  Also
+// clears the tile's counter for the next call.  One launch instead of three:
+// they are latency there, not work (1 x 128^2: 23 -> 9 us of kernels).
+__global__ void __launch_bounds__(kMidSortThreads) k_tile_sort_small(const int2 *__restrict__ ranges, int64_t n_tiles,
+                                                                     const uint64_t *__restrict__ pair_key,
+                                                                     uint32_t *__restrict__ pair_tile,
+                                                                     uint32_t *__restrict__ pair_item,
+                                                                     uint32_t *__restrict__ tile_count,
+                                                                     uint32_t *__restrict__ long_tiles,
+                                                                     uint32_t *__restrict__ long_count)
+{
+    __shared__ uint64_t buf[2][kMidBufWords];
+    __shared__ uint32_t cnt[kMidSortMax / 2], cur[kMidSortMax / 2], scratch[4 + kMidSortThreads / 32];
+    const uint32_t tile = blockIdx.x;
+    const int t = threadIdx.x;
+    const int2 r = ranges[tile];
+    const int n = r.y - r.x;
+    if (t == 0) tile_count[tile] = 0u;
+    const uint64_t *keys = pair_key + r.x;
+    if (n <= 32) {
+        if (t >= 32 || n == 0) return;
+        const uint64_t a = warp_bitonic32(t < n ? keys[t] : kPadKey);
+        if (t < n) write_sorted(a, r.x + t, tile, pair_tile, pair_item);
+        return;
+    }
+    if (n > kMidSortMax) {
+        if (t == 0) long_tiles[n_tiles - 1 - atomicAdd(&long_count[1], 1u)] = tile;
+        return;
+    }
+    const uint64_t *b = bucket_rank_sort<kMidSortThreads>(keys, n, buf[0], buf[1], cnt, cur, scratch, t);
+    if (b) {
+        for (int i = t; i < n; i += kMidSortThreads) write_sorted(b[i], r.x + i, tile, pair_tile, pair_item);
+        return;
+    }
+    b = group_merge_sort<kMidSortThreads, true>(keys, n, buf[0], buf[1], t);
+    for (int i = t; i < n; i += kMidSortThreads) write_sorted(b[padded(i)], r.x + i, tile, pair_tile, pair_item);
 }
 
 // Ascending compare-exchange of s[i] and s[l] (i < l).
@@ -1328,6 +1391,19 @@ vbm_status binning(vbm_plan *p, int vb, int vc, cudaStream_t st)
         note_launches(1);
     }
     // 3. each tile's list sorted by (depth, item)
+    const int long_blocks = (int)std::min<int64_t>(num_sms() * 2, n_tiles);
+    if (chunks == 1 && !radix) {
+        k_tile_sort_small<<<(unsigned)n_tiles, kMidSortThreads, 0, st>>>(p->ranges, n_tiles, p->pair_key, p->pair_tile,
+                                                                         p->pair_item, p->tile_count, b.long_tiles,
+                                                                         b.long_count);
+        VBM_LAUNCH("tile_sort_small");
+        k_tile_sort_block<<<long_blocks, kBlockSortThreads, kBlockSortSmem, st>>>(
+            p->ranges, p->pair_key, p->pair_tile, p->pair_item, b.long_tiles, b.long_count, n_tiles);
+        VBM_LAUNCH("tile_sort_block");
+        note_launches(2);
+        return VBM_OK;
+    }
+    if (chunks == 1) o.q = nullptr;      // k_tile_scan_small has ordered the tiles
     // one wave of blocks (more would leave a partial second wave on a few SMs)
     static int sort_per_sm = 0;
     if (sort_per_sm == 0) {
@@ -1357,7 +1433,7 @@ vbm_status binning(vbm_plan *p, int vb, int vc, cudaStream_t st)
         k_tile_sort_mid<<<(int)std::min<int64_t>(num_sms() * 8, n_tiles), kMidSortThreads, 0, st>>>(
             p->ranges, p->pair_key, p->pair_tile, p->pair_item, b.long_tiles, b.long_count);
         VBM_LAUNCH("tile_sort_mid");
-        k_tile_sort_block<<<(int)std::min<int64_t>(num_sms() * 2, n_tiles), kBlockSortThreads, kBlockSortSmem, st>>>(
+        k_tile_sort_block<<<long_blocks, kBlockSortThreads, kBlockSortSmem, st>>>(
             p->ranges, p->pair_key, p->pair_tile, p->pair_item, b.long_tiles, b.long_count, n_tiles);
         VBM_LAUNCH("tile_sort_block");
         note_launches(2);
