@@ -48,12 +48,13 @@ struct BandTab {
     int nb;
     int ox[kMaxBands], oy[kMaxBands], oz[kMaxBands], mx[kMaxBands], my[kMaxBands];
     int64_t n[kMaxBands], voff[kMaxBands];
+    double n_beta[kMaxBands];            // N^beta of the budget
     int chunk0[kMaxBands + 1], blk0[kMaxBands + 1];
 };
 
 // Budget of Supp. Sec. 1.1, evaluated on the device from the band energies.
 struct Budget {
-    double alpha_E, beta_N, K_tot;
+    double alpha_E, K_tot;
     int64_t min_per_band;
     float lambda;
 };
@@ -85,37 +86,6 @@ __device__ __forceinline__ int64_t pyramid_index(const BandTab &t, int b, int64_
     z = t.n[b] <= INT_MAX ? (int)((uint32_t)row / (uint32_t)t.my[b]) : (int)(row / t.my[b]);
     y = (int)(row - (int64_t)z * t.my[b]);
     return ((int64_t)(t.oz[b] + z) * ny + (t.oy[b] + y)) * nx + (t.ox[b] + x);
-}
-
-// Joint magnitudes of every band, and the bands' opacity energies in double.
-__global__ void __launch_bounds__(kMarkThreads) k_joint_mag(const float *__restrict__ A, int64_t chan, int nx, int ny,
-                                                            const __grid_constant__ BandTab t, float *__restrict__ v,
-                                                            double *__restrict__ E)
-{
-    const int b = band_of(t.chunk0, t.nb, blockIdx.x);
-    const int64_t i0 = (int64_t)(blockIdx.x - t.chunk0[b]) * kChunk;
-    const int64_t i1 = min(t.n[b], i0 + kChunk);
-    double s = 0.0;
-    for (int64_t i = i0 + threadIdx.x; i < i1; i += kMarkThreads) {
-        int x, y, z;
-        const int64_t e = pyramid_index(t, b, i, nx, ny, x, y, z);
-        const float a0 = A[e], a1 = A[chan + e], a2 = A[2 * chan + e], a3 = A[3 * chan + e];
-        float acc = __fmul_rn(a0, a0);
-        acc = __fadd_rn(acc, __fmul_rn(a1, a1));
-        acc = __fadd_rn(acc, __fmul_rn(a2, a2));
-        acc = __fadd_rn(acc, __fmul_rn(a3, a3));
-        v[t.voff[b] + i] = __fsqrt_rn(acc);
-        s += (double)a3 * (double)a3;
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    __shared__ double red[kMarkThreads / 32];
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < kMarkThreads / 32; w++) s += red[w];
-        atomicAdd(E + b, s);
-    }
 }
 
 // Exclusive block scan of one count per thread; `total` is the block's sum.
@@ -151,7 +121,182 @@ struct Digit {
     static constexpr int bits = DIGIT == 1 ? 11 : 10;
 };
 
-// One radix-select pass over every band at once: digit DIGIT of the magnitudes
+// Shared memory of a block that picks digits.
+struct Pick {
+    uint32_t sums[kTargets][32];
+    uint32_t digit[kTargets], rest[kTargets], prefix[kTargets];
+    long long rank[kTargets];
+};
+
+// The digit of each of N targets: the bin of its histogram (count(k, bin)) in
+// which its rank falls; the rank becomes the rest inside that bin and the digit
+// joins the prefix.  All kSelThreads threads; the targets share the barriers.
+template <int BITS, int N, typename F>
+__device__ __forceinline__ void pick_digits(Pick &s, F count)
+{
+    constexpr int PER = (1 << BITS) / kSelThreads;
+    static_assert(PER >= 1 && kSelThreads == 1024, "whole bins a thread, one warp sum a lane");
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t c[N][PER], mine[N], incl[N];
+#pragma unroll
+    for (int k = 0; k < N; k++) {
+        mine[k] = 0;
+#pragma unroll
+        for (int i = 0; i < PER; i++) mine[k] += c[k][i] = count(k, threadIdx.x * PER + i);
+        incl[k] = mine[k];
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl[k], off);
+            if (lane >= off) incl[k] += y;
+        }
+        if (lane == 31) s.sums[k][w] = incl[k];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < N; k++) {
+        const uint32_t before = __reduce_add_sync(0xffffffffu, lane < w ? s.sums[k][lane] : 0u);
+        long long at = s.rank[k] - (long long)(before + incl[k] - mine[k]);
+        if (at >= 0 && at < (long long)mine[k]) {
+            int i = 0;
+            while (i < PER - 1 && at >= (long long)c[k][i]) at -= c[k][i++];
+            s.digit[k] = (uint32_t)(threadIdx.x * PER + i);
+            s.rest[k] = (uint32_t)at;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < N) {
+        const int k = threadIdx.x;
+        s.rank[k] = s.rest[k];
+        s.prefix[k] = (s.prefix[k] << BITS) | s.digit[k];
+    }
+    __syncthreads();
+}
+
+// The budget of band b (Supp. Sec. 1.1): K = max(min_per_band, floor(K_tot S /
+// sum S)), S = E^alpha N^beta, in thread 0's result.  All threads call it;
+// share: kMaxBands doubles.  Double precision is slow here, so only the
+// powers' threads and one adder use it.
+__device__ __forceinline__ int64_t band_budget(const BandTab &t, const Budget &bud, const double *E, int b,
+                                               double *share)
+{
+    if (threadIdx.x < (unsigned)t.nb) share[threadIdx.x] = pow(__ldcg(E + threadIdx.x), bud.alpha_E) * t.n_beta[threadIdx.x];
+    __syncthreads();
+    if (threadIdx.x != 0) return 0;
+    double sum = 0.0;
+    for (int k = 0; k < t.nb; k++) sum += share[k];
+    const double mine = sum > 0 ? bud.K_tot * share[b] / sum : 0.0;
+    return max(bud.min_per_band, (int64_t)floor(mine));
+}
+
+// The median of n values from its lower and upper middle value.
+__device__ __forceinline__ float median_of(int64_t n, uint32_t lower, uint32_t upper)
+{
+    const float a = __uint_as_float(lower), c = __uint_as_float(upper);
+    return (n & 1) ? c : __fmul_rn(__fadd_rn(a, c), 0.5f);
+}
+
+// Keep v >= max(T, v_(K')), K' = min(K, #{v >= T}): where fewer than K values
+// reach T, v_(K) < T and the maximum is T itself, the same set.
+__device__ __forceinline__ float threshold(float mad, float lambda, bool none, float vk)
+{
+    const float T = __fmul_rn(lambda, __fdiv_rn(mad, 0.6745f));
+    return none || T != T ? __int_as_float(0x7f800000) : fmaxf(T, vk);
+}
+
+// Bands of at most kSmallBand elements: one block holds the band in registers
+// and runs all six digit passes beside the larger bands' first one (a pass over
+// 15 such bands cost 10 us as a launch of its own, nearly all of it latency).
+constexpr int kSmallPer = 8;
+constexpr int kSmallBand = kSmallPer * kSelThreads;
+
+template <int DIGIT, int N>
+__device__ __forceinline__ void small_digit(Pick &s, uint32_t (&h)[kTargets][kBins], uint32_t *zeros,
+                                            const float (&x)[kSmallPer], int n)
+{
+    using D = Digit<DIGIT>;
+    constexpr int NB = 1 << D::bits, NT = DIGIT == 0 ? 1 : N;
+    const int tid = threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < NT; k++)
+        for (int i = tid; i < NB; i += kSelThreads) h[k][i] = 0;
+    if (DIGIT == 0 && tid == 0) *zeros = 0;
+    uint32_t p[N];
+#pragma unroll
+    for (int k = 0; k < N; k++) p[k] = s.prefix[k];
+    __syncthreads();
+    uint32_t zero = 0;
+#pragma unroll
+    for (int e = 0; e < kSmallPer; e++) {
+        if (tid + e * kSelThreads >= n) continue;
+        const uint32_t bits = __float_as_uint(x[e]);
+        if (bits == 0) {
+            zero++;
+            continue;
+        }
+        const uint32_t d = (bits >> D::shift) & (NB - 1), pre = bits >> (D::shift + D::bits);
+        if (DIGIT == 0) {
+            atomicAdd(&h[0][d], 1u);
+        } else {
+#pragma unroll
+            for (int k = 0; k < N; k++) {            // into the first target of its prefix
+                if (pre != p[k]) continue;
+                atomicAdd(&h[k][d], 1u);
+                break;
+            }
+        }
+    }
+    if (DIGIT == 0) {
+        zero = __reduce_add_sync(0xffffffffu, zero);
+        if ((tid & 31) == 0 && zero) atomicAdd(zeros, zero);
+    }
+    __syncthreads();
+    const uint32_t z = *zeros;
+    pick_digits<D::bits, N>(s, [&](int k, int bin) {
+        int src = 0;
+        if (DIGIT > 0)
+            while (p[src] != p[k]) src++;
+        return h[src][bin] + (bin == 0 && p[k] == 0 ? z : 0u);
+    });
+}
+
+__device__ void select_small(const float *__restrict__ v, const BandTab &t, const Budget &bud,
+                             const double *__restrict__ E, SubState *__restrict__ st, int b,
+                             uint32_t (&h)[kTargets][kBins], double *share, Pick &s, uint32_t *zeros)
+{
+    const int tid = threadIdx.x;
+    const int n = (int)t.n[b];
+    float x[kSmallPer];
+#pragma unroll
+    for (int e = 0; e < kSmallPer; e++)
+        x[e] = tid + e * kSelThreads < n ? v[t.voff[b] + tid + e * kSelThreads] : 0.f;
+    const int64_t K = band_budget(t, bud, E, b, share);
+    if (tid == 0) {
+        s.rank[0] = (n - 1) / 2;                     // the middle value, or the lower one of an even count
+        s.rank[1] = n / 2;
+        s.rank[2] = n - min(max(K, (int64_t)1), (int64_t)n);
+        s.prefix[0] = s.prefix[1] = s.prefix[2] = 0;
+    }
+    __syncthreads();
+    small_digit<0, 3>(s, h, zeros, x, n);
+    small_digit<1, 3>(s, h, zeros, x, n);
+    small_digit<2, 3>(s, h, zeros, x, n);
+    const float med = median_of(n, s.prefix[0], s.prefix[1]), vk = __uint_as_float(s.prefix[2]);
+    __syncthreads();
+    if (tid == 0) {
+        s.rank[0] = (n - 1) / 2;
+        s.rank[1] = n / 2;
+        s.prefix[0] = s.prefix[1] = 0;
+    }
+#pragma unroll
+    for (int e = 0; e < kSmallPer; e++) x[e] = fabsf(__fsub_rn(x[e], med));
+    __syncthreads();
+    small_digit<0, 2>(s, h, zeros, x, n);
+    small_digit<1, 2>(s, h, zeros, x, n);
+    small_digit<2, 2>(s, h, zeros, x, n);
+    if (tid == 0) st[b].thr = threshold(median_of(n, s.prefix[0], s.prefix[1]), bud.lambda, K <= 0, vk);
+}
+
+// One radix-select pass over every larger band at once: digit DIGIT of the magnitudes
 // (DEV = false: both median ranks and the K-th largest in the same pass) or of
 // their absolute deviations from the median (DEV = true: both median ranks),
 // which are formed on the fly.  A block counts one band's digits in shared
@@ -176,16 +321,26 @@ __global__ void __launch_bounds__(kSelThreads) k_select_pass(const float *__rest
     constexpr int NB = 1 << D::bits;
     constexpr int NT = DIGIT == 0 ? 1 : DEV ? 2 : 3;             // histograms
     constexpr int COPIES = DIGIT == 0 ? 8 : 1;
-    __shared__ uint32_t h[NT * NB * COPIES];
-    __shared__ uint32_t warp_sum[kSelThreads / 32];
+    constexpr int WORDS = NT * NB * COPIES;
+    __shared__ uint32_t h[WORDS];
+    __shared__ Pick pick;
     __shared__ double share[kMaxBands];
-    __shared__ uint32_t s_last, s_digit;
-    __shared__ long long s_rank;
+    __shared__ uint32_t s_last;
     const int tid = threadIdx.x;
+    if constexpr (DIGIT == 0 && !DEV) {
+        static_assert(WORDS >= kTargets * kBins, "a small band's histograms fit");
+        const int small = (int)blockIdx.x - t.blk0[t.nb];        // the blocks beyond the passes': one a band
+        if (small >= 0) {
+            if (t.n[small] <= kSmallBand)
+                select_small(v, t, bud, E, st, small, reinterpret_cast<uint32_t(&)[kTargets][kBins]>(h), share, pick,
+                             &s_last);
+            return;
+        }
+    }
     const int b = band_of(t.blk0, t.nb, blockIdx.x);
     SubState *sb = st + b;
     uint32_t *gh = hist + (int64_t)b * kTargets * kBins;
-    for (int i = tid; i < NT * NB * COPIES; i += kSelThreads) h[i] = 0;
+    for (int i = tid; i < WORDS; i += kSelThreads) h[i] = 0;
     __syncthreads();
     const uint32_t p0 = sb->prefix[0], p1 = sb->prefix[1], p2 = sb->prefix[2];
     const float med = DEV ? sb->med : 0.f;
@@ -253,68 +408,41 @@ __global__ void __launch_bounds__(kSelThreads) k_select_pass(const float *__rest
     // ---- the band's last block: pick the digits
     const int64_t n = t.n[b];
     const uint32_t n_zero = (uint32_t)__ldcg(&sb->zeros[DEV]);
-    if (DIGIT == 0 && !DEV) {
-        // K of this band: max(min_per_band, floor(K_tot S / sum S)), S = E^alpha N^beta
-        if (tid < t.nb) share[tid] = pow(__ldcg(E + tid), bud.alpha_E) * pow((double)t.n[tid], bud.beta_N);
-        __syncthreads();
-        if (tid == 0) {
-            double sum = 0.0;
-            for (int k = 0; k < t.nb; k++) sum += share[k];
-            const double mine = sum > 0 ? bud.K_tot * share[b] / sum : 0.0;
-            const int64_t K = max(bud.min_per_band, (int64_t)floor(mine));
-            sb->none = K <= 0;
-            sb->rank[2] = n - min(max(K, (int64_t)1), n);
+    constexpr int N = DEV ? 2 : kTargets;
+    int64_t K = 0;
+    if (DIGIT == 0 && !DEV) K = band_budget(t, bud, E, b, share);
+    if (tid == 0) {
+        if (DIGIT == 0) {
+            pick.rank[0] = (n - 1) / 2;      // the middle value, or the lower one of an even count
+            pick.rank[1] = n / 2;
+            pick.rank[2] = n - min(max(K, (int64_t)1), n);
+            if (!DEV) sb->none = K <= 0;
+        }
+        for (int k = 0; k < N; k++) {
+            if (DIGIT > 0) pick.rank[k] = sb->rank[k];
+            pick.prefix[k] = DIGIT > 0 ? sb->prefix[k] : 0u;
         }
     }
-    if (DIGIT == 0 && tid == 0) {
-        sb->rank[0] = (n - 1) / 2;       // the middle value, or the lower one of an even count
-        sb->rank[1] = n / 2;
-        sb->prefix[0] = sb->prefix[1] = 0;
-        if (!DEV) sb->prefix[2] = 0;
-    }
     __syncthreads();
-    const int n_target = DEV ? 2 : kTargets;
-    uint32_t old[kTargets];
-    for (int k = 0; k < n_target; k++) old[k] = sb->prefix[k];
-    __syncthreads();
-    for (int k = 0; k < n_target; k++) {
-        // the histogram that counted this target's prefix
-        const int src = DIGIT == 0 ? 0 : old[k] == old[0] ? 0 : old[k] == old[1] ? 1 : 2;
-        const long long rank = sb->rank[k];
-        constexpr int PER = (NB + kSelThreads - 1) / kSelThreads;
-        uint32_t c[PER], mine = 0, total;
+    uint32_t old[N];
 #pragma unroll
-        for (int i = 0; i < PER; i++) {
-            const int bin = tid * PER + i;
-            c[i] = __ldcg(&gh[src * kBins + bin]) + (bin == 0 && old[k] == 0 ? n_zero : 0u);
-            mine += c[i];
-        }
-        long long at = rank - (long long)block_scan<kSelThreads>(mine, warp_sum, total);
-        if (at >= 0 && at < (long long)mine) {
-            int i = 0;
-            while (i < PER - 1 && at >= (long long)c[i]) at -= c[i++];
-            s_digit = (uint32_t)(tid * PER + i);
-            s_rank = at;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            sb->rank[k] = s_rank;
-            sb->prefix[k] = (old[k] << D::bits) | s_digit;
-        }
-        __syncthreads();
-    }
+    for (int k = 0; k < N; k++) old[k] = pick.prefix[k];
+    pick_digits<D::bits, N>(pick, [&](int k, int bin) {
+        // the histogram that counted this target's prefix
+        const int src = DIGIT == 0 || old[k] == old[0] ? 0 : old[k] == old[1] ? 1 : 2;
+        return __ldcg(&gh[src * kBins + bin]) + (bin == 0 && old[k] == 0 ? n_zero : 0u);
+    });
     for (int i = tid; i < kTargets * kBins; i += kSelThreads) gh[i] = 0;
+    if (tid >= N) return;
+    sb->rank[tid] = pick.rank[tid];
+    sb->prefix[tid] = pick.prefix[tid];
     if (DIGIT == 2 && tid == 0) {
-        const float a = __uint_as_float(sb->prefix[0]), c = __uint_as_float(sb->prefix[1]);
-        const float m = (n & 1) ? c : __fmul_rn(__fadd_rn(a, c), 0.5f);
+        const float m = median_of(n, pick.prefix[0], pick.prefix[1]);
         if (!DEV) {
             sb->med = m;
-            sb->vk = __uint_as_float(sb->prefix[2]);
+            sb->vk = __uint_as_float(pick.prefix[2]);
         } else {
-            // keep v >= max(T, v_(K')), K' = min(K, #{v >= T}): where fewer than K
-            // values reach T, v_(K) < T and the maximum is T itself, the same set
-            const float T = __fmul_rn(bud.lambda, __fdiv_rn(m, 0.6745f));
-            sb->thr = sb->none || T != T ? __int_as_float(0x7f800000) : fmaxf(T, sb->vk);
+            sb->thr = threshold(m, bud.lambda, sb->none, sb->vk);
         }
     }
 }
@@ -481,10 +609,12 @@ std::vector<Band> bands_of(const int dims[3], int levels)
     return out;
 }
 
-// Element offsets, marking chunks and selection blocks of the bands.  A
-// selection block takes at least 8192 elements of one band; beyond that the
-// blocks are two waves of the chip's resident ones, shared out by band size.
-BandTab band_table(const std::vector<Band> &bands)
+// Element offsets, marking chunks and selection blocks of the bands.  Bands of
+// at most kSmallBand elements have no blocks in the selection passes (one block
+// of the first launch takes all of theirs); of the others a block takes at least 8192
+// elements, and beyond that the blocks are two to an SM, shared out by band
+// size.
+BandTab band_table(const std::vector<Band> &bands, double beta_N)
 {
     BandTab t{};
     t.nb = (int)bands.size();
@@ -495,17 +625,18 @@ BandTab band_table(const std::vector<Band> &bands)
         const Band &B = bands[b];
         t.ox[b] = B.ox; t.oy[b] = B.oy; t.oz[b] = B.oz; t.mx[b] = B.mx; t.my[b] = B.my;
         t.n[b] = B.n;
+        t.n_beta[b] = std::pow((double)B.n, beta_N);
         t.voff[b] = off;
         off += (B.n + 31) / 32 * 32;
         t.chunk0[b + 1] = t.chunk0[b] + (int)((B.n + kChunk - 1) / kChunk);
-        t.blk0[b + 1] = t.blk0[b] + (int)((B.n + per - 1) / per);
+        t.blk0[b + 1] = t.blk0[b] + (B.n <= kSmallBand ? 0 : (int)((B.n + per - 1) / per));
     }
     return t;
 }
 
 // Device scratch of one build, in order; with ws = NULL only its size.
 struct BuildScratch {
-    float *A, *tmp;
+    float *A, *tmp, *v;
     uint32_t *mask, *count;
     int64_t *first;
     MapTab *map;
@@ -529,7 +660,8 @@ BuildScratch build_scratch(void *ws, const int dims[3])
     };
     const size_t chunks = n / kChunk + kMaxBands;
     s.A = (float *)take(4 * n * sizeof(float));                            // RF / pyramid
-    s.tmp = (float *)take(std::max((size_t)pyramid_tmp_floats(dims), padded) * sizeof(float));   // DWT, then magnitudes
+    s.tmp = (float *)take((size_t)pyramid_tmp_floats(dims) * sizeof(float));   // DWT temporaries
+    s.v = (float *)take(padded * sizeof(float));                           // joint magnitudes
     s.mask = (uint32_t *)take(padded / 32 * sizeof(uint32_t));
     s.count = (uint32_t *)take(chunks * sizeof(uint32_t));
     s.first = (int64_t *)take(chunks * sizeof(int64_t));
@@ -610,7 +742,7 @@ vbm_status vbm_build(const float *d_volume, const int dims[3], const vbm_tf *tf,
     cudaStream_t st = (cudaStream_t)stream;
     const int64_t n = (int64_t)dims[0] * dims[1] * dims[2];
     const BuildScratch w = build_scratch(d_ws, dims);
-    float *A = w.A, *v = w.tmp;
+    float *A = w.A, *v = w.v;
     std::vector<Band> bands = bands_of(dims, levels);
     const int nb = (int)bands.size();
     MapTab map{};
@@ -628,21 +760,23 @@ vbm_status vbm_build(const float *d_volume, const int dims[3], const vbm_tf *tf,
         me.j = B.j;
         me.s = sel->energy_comp ? (float)std::pow(2.0, -1.5 * B.j) : 1.f;
     }
-    const BandTab t = band_table(bands);
-    const Budget bud{sel->alpha_E, sel->beta_N, (double)sel->K_tot, sel->min_per_band, (float)sel->lambda_mad};
+    const BandTab t = band_table(bands, sel->beta_N);
+    const Budget bud{sel->alpha_E, (double)sel->K_tot, sel->min_per_band, (float)sel->lambda_mad};
 
     VBM_CUDA(cudaMemcpyAsync(w.map, &map, sizeof(map), cudaMemcpyHostToDevice, st));
     VBM_CUDA(cudaMemsetAsync(w.zeroed, 0, w.zero_bytes, st));
-    s = pyramid_from_volume(d_volume, dims, tf, levels, bank->wavelet, A, w.tmp, st);
+    s = pyramid_from_volume(d_volume, dims, tf, levels, bank->wavelet, A, w.tmp, v, t.voff, w.E, st);
     if (s != VBM_OK) return s;
     const int chunks = t.chunk0[nb], blocks = t.blk0[nb];
-    k_joint_mag<<<chunks, kMarkThreads, 0, st>>>(A, n, dims[0], dims[1], t, v, w.E);
-    k_select_pass<0, false><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
-    k_select_pass<1, false><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
-    k_select_pass<2, false><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
-    k_select_pass<0, true><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
-    k_select_pass<1, true><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
-    k_select_pass<2, true><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
+    // the first pass's last nb blocks do all of the small bands' selection
+    k_select_pass<0, false><<<blocks + nb, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
+    if (blocks > 0) {
+        k_select_pass<1, false><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
+        k_select_pass<2, false><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
+        k_select_pass<0, true><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
+        k_select_pass<1, true><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
+        k_select_pass<2, true><<<blocks, kSelThreads, 0, st>>>(v, t, bud, w.E, w.st, w.hist);
+    }
     VBM_LAUNCH("select");
     k_mark<<<chunks, kMarkThreads, 0, st>>>(v, t, dims[0], dims[1], w.st, w.mask, w.count, w.first, w.total, w.ticket,
                                             d_keep);

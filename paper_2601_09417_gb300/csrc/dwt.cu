@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kXYThreads, 2) k_dwt_xy(const __grid_constant_
     }
 }
 
-// z pass: a thread takes V neighbouring columns of one channel and `pairs`
+// z pass: a thread takes V neighbouring columns of NC channels and `pairs`
 // plane pairs, with the 10 planes the filter spans in a register ring and the
 // next pair's loads in flight.  Bound by memory: each value is read and
 // written once (plus the 8 planes of overlap between chunks, from L2).
@@ -297,6 +297,20 @@ struct ZArgs {
     int k_begin, k_end, pairs;           // output pairs of this launch, and of a thread
 };
 
+// What vbm_build selects by, written where the level's coefficients are formed
+// (NC = 4, V = 1): the joint magnitude of each, at its place in its subband,
+// and the subband's opacity energy.  Octant c = o_x + 2 o_y + 4 o_z is subband
+// band[c] (-1: the low octant of a level that is not the last) and its
+// magnitudes start at voff[c].  A pass of its own read the four channels again
+// (732 us of a 512^3 build; the fused stores and the energies' double
+// precision sums add 185 us).
+struct Magnitudes {
+    float *v;
+    double *E;
+    int64_t voff[8];
+    int band[8];
+};
+
 template <int V>
 struct Vec;
 template <>
@@ -304,29 +318,55 @@ struct Vec<1> { using T = float; };
 template <>
 struct Vec<4> { using T = float4; };
 
-constexpr int kZThreads = 256;
+// Threads a block: with four channels a thread takes up to 102 registers, and
+// blocks of 128 then leave 20 warps on an SM (of 256: 16).
+__host__ __device__ constexpr int z_threads(int channels) { return channels == 4 ? 128 : 256; }
 
-template <int WAVELET, int V>
-__global__ void __launch_bounds__(kZThreads) k_dwt_z(const __grid_constant__ ZArgs a, const __grid_constant__ Taps w)
+template <int WAVELET, int V, int NC>
+__global__ void __launch_bounds__(z_threads(NC), NC == 4 ? 5 : 3) k_dwt_z(const __grid_constant__ ZArgs a, const __grid_constant__ Taps w,
+                                                     const __grid_constant__ Magnitudes mag)
 {
     using Wv = Wavelet<WAVELET>;
     using T = typename Vec<V>::T;
     constexpr int R = Wv::PAIRS;
+    constexpr bool MAG = NC == 4;
+    constexpr int THREADS = z_threads(NC);
     const int64_t plane = (int64_t)a.sx * a.sy;
-    const int64_t at = ((int64_t)blockIdx.x * kZThreads + threadIdx.x) * V;
-    if (at >= plane) return;
+    int64_t at = ((int64_t)blockIdx.x * THREADS + threadIdx.x) * V;
+    const bool on = at < plane;
+    if (!MAG && !on) return;             // with MAG every lane stays for the energies' sum
+    if (!on) at = 0;
     const int k0 = a.k_begin + blockIdx.y * a.pairs, k1 = min(a.k_end, k0 + a.pairs);
     const int y = (int)(at / a.sx), x = (int)(at - (int64_t)y * a.sx);
     const float *src = a.src + blockIdx.z * a.src_chan + at;
     float *dst = a.dst + blockIdx.z * a.dst_chan + (int64_t)y * a.dst_row + x;
+    const int hx = a.sx >> 1, hy = a.sy >> 1;
+    const int code = (x >= hx) + 2 * (y >= hy);                  // MAG: octants code and code + 4
+    float *v_lo = nullptr, *v_hi = nullptr;
+    double e_lo = 0.0, e_hi = 0.0;
+    if (MAG && on) {
+        const int64_t in_plane = (int64_t)(y - (y >= hy ? hy : 0)) * hx + (x - (x >= hx ? hx : 0));
+        if (mag.band[code] >= 0) v_lo = mag.v + mag.voff[code] + in_plane;
+        v_hi = mag.v + mag.voff[code + 4] + in_plane;
+    }
     int t = wrap(2 * k0 + Wv::FIRST - a.z_first, a.planes);
-    float ring[R][2][V], next[2][V];
+    float ring[R][2][NC * V], next[2][NC * V];
     auto fetch = [&]() {
 #pragma unroll
         for (int r = 0; r < 2; r++) {
-            *reinterpret_cast<T *>(next[r]) = *reinterpret_cast<const T *>(src + (int64_t)t * plane);
+#pragma unroll
+            for (int n = 0; n < NC; n++)
+                *reinterpret_cast<T *>(&next[r][n * V]) =
+                    *reinterpret_cast<const T *>(src + n * a.src_chan + (int64_t)t * plane);
             t = t + 1 == a.planes ? 0 : t + 1;
         }
+    };
+    // sqrt(((a0 a0 + a1 a1) + a2 a2) + a3 a3), rounded op by op
+    auto magnitude = [](const float *c) {
+        float acc = __fmul_rn(c[0], c[0]);
+        acc = __fadd_rn(acc, __fmul_rn(c[1], c[1]));
+        acc = __fadd_rn(acc, __fmul_rn(c[2], c[2]));
+        return __fsqrt_rn(__fadd_rn(acc, __fmul_rn(c[3], c[3])));
     };
     const int steps = k1 - k0 + R - 1;
     fetch();
@@ -338,27 +378,60 @@ __global__ void __launch_bounds__(kZThreads) k_dwt_z(const __grid_constant__ ZAr
 #pragma unroll
             for (int r = 0; r < 2; r++)
 #pragma unroll
-                for (int c = 0; c < V; c++) ring[u][r][c] = next[r][c];
+                for (int c = 0; c < NC * V; c++) ring[u][r][c] = next[r][c];
             if (step + 1 < steps) fetch();
             if (step < R - 1) continue;
             const int k = k0 + step - (R - 1);
-            float lo[V], hi[V];
+            float lo[NC * V], hi[NC * V];
 #pragma unroll
-            for (int c = 0; c < V; c++) lo[c] = hi[c] = 0.f;
+            for (int c = 0; c < NC * V; c++) lo[c] = hi[c] = 0.f;
 #pragma unroll
             for (int i = 0; i < Wv::LO_LEN; i++) {
                 const int j = Wv::LO - Wv::FIRST + i;
 #pragma unroll
-                for (int c = 0; c < V; c++) lo[c] = __fmaf_rn(w.lo[i], ring[(u + 1 + j / 2) % R][j & 1][c], lo[c]);
+                for (int c = 0; c < NC * V; c++)
+                    lo[c] = __fmaf_rn(w.lo[i], ring[(u + 1 + j / 2) % R][j & 1][c], lo[c]);
             }
 #pragma unroll
             for (int i = 0; i < Wv::HI_LEN; i++) {
                 const int j = Wv::HI - Wv::FIRST + i;
 #pragma unroll
-                for (int c = 0; c < V; c++) hi[c] = __fmaf_rn(w.hi[i], ring[(u + 1 + j / 2) % R][j & 1][c], hi[c]);
+                for (int c = 0; c < NC * V; c++)
+                    hi[c] = __fmaf_rn(w.hi[i], ring[(u + 1 + j / 2) % R][j & 1][c], hi[c]);
             }
-            *reinterpret_cast<T *>(dst + (int64_t)k * a.dst_plane) = *reinterpret_cast<const T *>(lo);
-            *reinterpret_cast<T *>(dst + (int64_t)(a.sz / 2 + k) * a.dst_plane) = *reinterpret_cast<const T *>(hi);
+            if (MAG && !on) continue;
+            float *d_lo = dst + (int64_t)k * a.dst_plane, *d_hi = dst + (int64_t)(a.sz / 2 + k) * a.dst_plane;
+#pragma unroll
+            for (int n = 0; n < NC; n++) {
+                *reinterpret_cast<T *>(d_lo + n * a.dst_chan) = *reinterpret_cast<const T *>(&lo[n * V]);
+                *reinterpret_cast<T *>(d_hi + n * a.dst_chan) = *reinterpret_cast<const T *>(&hi[n * V]);
+            }
+            if constexpr (MAG) {
+                const int64_t in_band = (int64_t)k * hx * hy;
+                if (v_lo) {
+                    v_lo[in_band] = magnitude(lo);
+                    e_lo += (double)lo[3] * (double)lo[3];
+                }
+                v_hi[in_band] = magnitude(hi);
+                e_hi += (double)hi[3] * (double)hi[3];
+            }
+        }
+    }
+    if constexpr (MAG) {
+        const int lane = threadIdx.x & 31;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            if (!__any_sync(0xffffffffu, on && code == c)) continue;
+            double lo = on && code == c ? e_lo : 0.0, hi = on && code == c ? e_hi : 0.0;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                lo += __shfl_xor_sync(0xffffffffu, lo, off);
+                hi += __shfl_xor_sync(0xffffffffu, hi, off);
+            }
+            if (lane == 0) {
+                if (mag.band[c] >= 0) atomicAdd(mag.E + mag.band[c], lo);
+                atomicAdd(mag.E + mag.band[c + 4], hi);
+            }
         }
     }
 }
@@ -433,18 +506,22 @@ vbm_status launch_xy(XYArgs a, int channels, const Taps &w, const TFDev &tf, cud
     return VBM_OK;
 }
 
+// mag: the magnitudes of a level of four channels (NULL: none).
 template <int WAVELET>
-vbm_status launch_z(ZArgs a, int channels, const Taps &w, cudaStream_t st)
+vbm_status launch_z(ZArgs a, int channels, const Taps &w, const Magnitudes *mag, cudaStream_t st)
 {
     const int64_t plane = (int64_t)a.sx * a.sy;
-    const bool vec = a.sx % 4 == 0 && aligned(a.src, 16) && aligned(a.dst, 16) && a.src_chan % 4 == 0 &&
+    const bool vec = !mag && a.sx % 4 == 0 && aligned(a.src, 16) && aligned(a.dst, 16) && a.src_chan % 4 == 0 &&
                      a.dst_chan % 4 == 0 && a.dst_plane % 4 == 0 && a.dst_row % 4 == 0;
     const int64_t lanes = vec ? plane / 4 : plane;
-    a.pairs = pairs_per(a.k_end - a.k_begin, lanes * channels, 64);
-    dim3 grid((unsigned)((lanes + kZThreads - 1) / kZThreads),
-              (unsigned)((a.k_end - a.k_begin + a.pairs - 1) / a.pairs), (unsigned)channels);
-    if (vec) k_dwt_z<WAVELET, 4><<<grid, kZThreads, 0, st>>>(a, w);
-    else k_dwt_z<WAVELET, 1><<<grid, kZThreads, 0, st>>>(a, w);
+    const int split = mag ? 1 : channels;                        // channels of different threads
+    a.pairs = pairs_per(a.k_end - a.k_begin, lanes * split, 64);
+    const int threads = z_threads(mag ? 4 : 1);
+    dim3 grid((unsigned)((lanes + threads - 1) / threads),
+              (unsigned)((a.k_end - a.k_begin + a.pairs - 1) / a.pairs), (unsigned)split);
+    if (mag) k_dwt_z<WAVELET, 1, 4><<<grid, threads, 0, st>>>(a, w, *mag);
+    else if (vec) k_dwt_z<WAVELET, 4, 1><<<grid, threads, 0, st>>>(a, w, Magnitudes{});
+    else k_dwt_z<WAVELET, 1, 1><<<grid, threads, 0, st>>>(a, w, Magnitudes{});
     VBM_LAUNCH("dwt_z");
     return VBM_OK;
 }
@@ -453,7 +530,7 @@ vbm_status launch_z(ZArgs a, int channels, const Taps &w, cudaStream_t st)
 // them.
 template <int WAVELET>
 vbm_status dwt_level(float *data, int channels, const int dims[3], int level, float *tmp, const Taps &w,
-                     cudaStream_t st)
+                     const Magnitudes *mag, cudaStream_t st)
 {
     const int64_t n = (int64_t)dims[0] * dims[1] * dims[2], plane = (int64_t)dims[0] * dims[1];
     const int sx = dims[0] >> (level - 1), sy = dims[1] >> (level - 1), sz = dims[2] >> (level - 1);
@@ -478,37 +555,50 @@ vbm_status dwt_level(float *data, int channels, const int dims[3], int level, fl
     z.dst_row = dims[0];
     z.sx = sx; z.sy = sy; z.sz = sz;
     z.k_end = sz / 2;
-    return launch_z<WAVELET>(z, channels, w, st);
+    return launch_z<WAVELET>(z, channels, w, mag, st);
 }
 
 template <int WAVELET>
-vbm_status dwt_levels(float *data, int n_channels, const int dims[3], int first, int levels, float *tmp,
-                      int64_t tmp_floats, const Taps &w, cudaStream_t st)
+vbm_status dwt_levels(float *data, int n_channels, const int dims[3], int levels, float *tmp, int64_t tmp_floats,
+                      const Taps &w, cudaStream_t st)
 {
     const int64_t n = (int64_t)dims[0] * dims[1] * dims[2];
-    for (int j = first; j <= levels; j++) {
+    for (int j = 1; j <= levels; j++) {
         const int64_t region = n >> (3 * (j - 1));
         const int most = (int)std::min<int64_t>(n_channels, std::min<int64_t>(tmp_floats / region, 32768));
         for (int c = 0; c < n_channels; c += most) {
-            vbm_status s = dwt_level<WAVELET>(data + c * n, std::min(most, n_channels - c), dims, j, tmp, w, st);
+            vbm_status s = dwt_level<WAVELET>(data + c * n, std::min(most, n_channels - c), dims, j, tmp, w, nullptr,
+                                              st);
             if (s != VBM_OK) return s;
         }
     }
     return VBM_OK;
 }
 
-// The first level of the RGBA channels straight from the scalar volume, in
-// slabs of planes where tmp does not hold the four channels whole.
+// The RGBA pyramid of a scalar volume with the magnitudes of its subbands.
+// The first level reads the volume through the transfer function, in slabs of
+// planes where tmp does not hold the four channels whole.
 template <int WAVELET>
-vbm_status first_level_tf(const float *volume, const int dims[3], const TFDev &tf, float *A, float *tmp,
-                          int64_t tmp_floats, const Taps &w, cudaStream_t st)
+vbm_status pyramid_levels(const float *volume, const int dims[3], const TFDev &tf, int levels, float *A, float *tmp,
+                          int64_t tmp_floats, const Taps &w, float *v, const int64_t *voff, double *E, cudaStream_t st)
 {
     using Wv = Wavelet<WAVELET>;
+    // the subbands of level j: seven octants, and at the last level the low one first
+    auto level_magnitudes = [&](int j) {
+        Magnitudes m{v, E, {}, {}};
+        for (int c = 0; c < 8; c++) {
+            const int b = 7 * (j - 1) + c - (j == levels ? 0 : 1);
+            m.band[c] = c == 0 && j != levels ? -1 : b;
+            m.voff[c] = m.band[c] < 0 ? 0 : voff[b];
+        }
+        return m;
+    };
     const int64_t plane = (int64_t)dims[0] * dims[1], n = plane * dims[2];
     const int overlap = 2 * (Wv::PAIRS - 1);
-    const int64_t room = tmp_floats / (4 * plane);                   // planes of four channels
+    const int64_t room = tmp_floats / (4 * plane);                        // planes of four channels
     const bool whole = room >= dims[2];
     const int slab = whole ? dims[2] / 2 : (int)((room - overlap) / 2);   // output pairs
+    const Magnitudes first = level_magnitudes(1);
     for (int k = 0; k < dims[2] / 2; k += slab) {
         const int k1 = std::min(dims[2] / 2, k + slab);
         XYArgs a{};
@@ -534,7 +624,12 @@ vbm_status first_level_tf(const float *volume, const int dims[3], const TFDev &t
         z.sx = dims[0]; z.sy = dims[1]; z.sz = dims[2];
         z.k_begin = k;
         z.k_end = k1;
-        s = launch_z<WAVELET>(z, 4, w, st);
+        s = launch_z<WAVELET>(z, 4, w, &first, st);
+        if (s != VBM_OK) return s;
+    }
+    for (int j = 2; j <= levels; j++) {
+        const Magnitudes m = level_magnitudes(j);
+        vbm_status s = dwt_level<WAVELET>(A, 4, dims, j, tmp, w, &m, st);
         if (s != VBM_OK) return s;
     }
     return VBM_OK;
@@ -559,29 +654,29 @@ vbm_status dwt_channels(float *data, int n_channels, const int dims[3], int leve
 {
     const int64_t room = 2 * (int64_t)dims[0] * dims[1] * dims[2];
     const Taps w = make_taps(wavelet);
-    return wavelet == 1 ? dwt_levels<1>(data, n_channels, dims, 1, levels, tmp, room, w, st)
-                        : dwt_levels<0>(data, n_channels, dims, 1, levels, tmp, room, w, st);
+    return wavelet == 1 ? dwt_levels<1>(data, n_channels, dims, levels, tmp, room, w, st)
+                        : dwt_levels<0>(data, n_channels, dims, levels, tmp, room, w, st);
 }
 
 // Floats of tmp for pyramid_from_volume: the four channels whole up to 2^26
-// floats (256^3 volumes), beyond that two volumes' worth, worked in slabs.
+// floats (256^3 volumes); beyond that 1.2 volumes, worked in slabs, which with
+// the magnitudes keeps vbm_build's scratch at 25 bytes a voxel.  At least
+// half of the volume (the second level's four channels) and 16 planes.
 int64_t pyramid_tmp_floats(const int dims[3])
 {
     const int64_t n = (int64_t)dims[0] * dims[1] * dims[2], plane = (int64_t)dims[0] * dims[1];
-    return std::max(std::max(2 * n, std::min<int64_t>(4 * n, 1 << 26)), std::min(4 * n, 4 * plane * 16));
+    const int64_t whole = 4 * n;
+    return std::min(whole, std::max({n + n / 5, (int64_t)1 << 26, 4 * plane * 16}));
 }
 
 vbm_status pyramid_from_volume(const float *volume, const int dims[3], const vbm_tf *tf, int levels, int wavelet,
-                               float *A, float *tmp, cudaStream_t st)
+                               float *A, float *tmp, float *v, const int64_t *voff, double *E, cudaStream_t st)
 {
     const int64_t room = pyramid_tmp_floats(dims);
     const Taps w = make_taps(wavelet);
     const TFDev t = to_dev(tf);
-    vbm_status s = wavelet == 1 ? first_level_tf<1>(volume, dims, t, A, tmp, room, w, st)
-                                : first_level_tf<0>(volume, dims, t, A, tmp, room, w, st);
-    if (s != VBM_OK) return s;
-    return wavelet == 1 ? dwt_levels<1>(A, 4, dims, 2, levels, tmp, room, w, st)
-                        : dwt_levels<0>(A, 4, dims, 2, levels, tmp, room, w, st);
+    return wavelet == 1 ? pyramid_levels<1>(volume, dims, t, levels, A, tmp, room, w, v, voff, E, st)
+                        : pyramid_levels<0>(volume, dims, t, levels, A, tmp, room, w, v, voff, E, st);
 }
 
 }  // namespace vbm

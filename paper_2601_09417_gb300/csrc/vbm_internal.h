@@ -423,8 +423,10 @@ vbm_status tf_apply(const float *volume, int64_t n, const vbm_tf *tf, float *rf,
 vbm_status dwt_channels(float *data, int n_channels, const int dims[3], int levels, int wavelet, float *tmp,
                         cudaStream_t st);
 int64_t pyramid_tmp_floats(const int dims[3]);
+// The pyramid A[4][n] of a volume, with the joint magnitudes of every subband
+// b (raster order) at v + voff[b] and its opacity energy added to E[b].
 vbm_status pyramid_from_volume(const float *volume, const int dims[3], const vbm_tf *tf, int levels, int wavelet,
-                               float *A, float *tmp, cudaStream_t st);
+                               float *A, float *tmp, float *v, const int64_t *voff, double *E, cudaStream_t st);
 
 // ---------------------------------------------------------------- binning
 // Work-queue counters of the compositing kernels (2), tile-group sizes and
