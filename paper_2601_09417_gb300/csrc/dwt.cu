@@ -55,9 +55,9 @@ __device__ __forceinline__ int wrap(int i, int n)
     return i < 0 ? i + n : i;
 }
 
-constexpr int kXYThreads = 256;
+constexpr int kXYThreads = 128;
 constexpr int kXPer = 4;                 // x positions (two output pairs) a thread
-constexpr int kMaxSlot = 64;             // threads of a slot: 256 positions
+constexpr int kMaxSlot = 32;             // threads of a slot: 128 positions
 constexpr int kMinSlot = 8;
 
 // Where the rows of the x and y passes come from: an array read one value or
@@ -77,7 +77,9 @@ enum Source { kScalar, kQuads, kTransfer };
 // thread's columns in pairs (FP32x2) and rows of whole 16-byte words are
 // staged four values at a time: the kernel is bound by instruction issue, not
 // by the arithmetic itself (4 x 256^3, all levels: 200 -> 170 us; with the
-// transfer function on 512^3, first level: 2.76 -> 1.63 ms).
+// transfer function on 512^3, first level: 2.76 -> 1.63 ms).  A slot lies in
+// one warp, so that only the transfer function's four need a block barrier
+// (slots of 64 threads and barriers for all: 4 x 256^3 pyramid 395 -> 367 us).
 //
 // kTransfer: the source is the scalar volume; four neighbouring slots take the
 // four channels of one strip, whose threads share the loads and the transfer
@@ -97,7 +99,7 @@ struct XYArgs {
 };
 
 template <int WAVELET, int SOURCE>
-__global__ void __launch_bounds__(kXYThreads, 2) k_dwt_xy(const __grid_constant__ XYArgs a,
+__global__ void __launch_bounds__(kXYThreads, 5) k_dwt_xy(const __grid_constant__ XYArgs a,
                                                           const __grid_constant__ Taps w,
                                                           const __grid_constant__ TFDev tf)
 {
@@ -253,7 +255,8 @@ __global__ void __launch_bounds__(kXYThreads, 2) k_dwt_xy(const __grid_constant_
             if (step >= steps) break;
             stage(step & 1);
             if (step + 1 < steps) fetch();
-            __syncthreads();
+            if (TF) __syncthreads();
+            else __syncwarp();                                   // a slot lies in one warp
             x_filter(step & 1, ring[u]);
             if (step < R - 1 || k0 + step - (R - 1) >= k1) continue;
             // sample pair i of the window is ring slot (u + 1 + i) mod R
@@ -284,7 +287,7 @@ __global__ void __launch_bounds__(kXYThreads, 2) k_dwt_xy(const __grid_constant_
 
 // z pass: a thread takes V neighbouring columns of NC channels and `pairs`
 // plane pairs, with the 10 planes the filter spans in a register ring and the
-// next pair's loads in flight.  Bound by memory: each value is read and
+// next pairs' loads in flight.  Bound by memory: each value is read and
 // written once (plus the 8 planes of overlap between chunks, from L2).
 struct ZArgs {
     const float *src;                    // [channel][plane][sy][sx]
@@ -318,6 +321,30 @@ struct Vec<1> { using T = float; };
 template <>
 struct Vec<4> { using T = float4; };
 
+constexpr int kZDepth = 4;               // plane pairs in flight, a power of two
+
+// Asynchronous copies of 4 or 16 bytes into shared memory.
+__device__ __forceinline__ void copy_async(float *to, const float *from)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from)
+                 : "memory");
+}
+
+__device__ __forceinline__ void copy_async(float4 *to, const float *from)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from)
+                 : "memory");
+}
+
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+
+// At most N of the thread's groups still in flight.
+template <int N>
+__device__ __forceinline__ void copy_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // Threads a block: with four channels a thread takes up to 102 registers, and
 // blocks of 128 then leave 20 warps on an SM (of 256: 16).
 __host__ __device__ constexpr int z_threads(int channels) { return channels == 4 ? 128 : 256; }
@@ -349,15 +376,19 @@ __global__ void __launch_bounds__(z_threads(NC), NC == 4 ? 5 : 3) k_dwt_z(const 
         if (mag.band[code] >= 0) v_lo = mag.v + mag.voff[code] + in_plane;
         v_hi = mag.v + mag.voff[code + 4] + in_plane;
     }
+    // plane pairs on their way: copied asynchronously into the thread's own
+    // shared-memory words, so that the depth costs no registers (one pair ahead
+    // in registers left too few bytes in flight: 4 x 256^3 pyramid 395 -> 354
+    // us, vbm_build of 512^3 4.27 -> 4.07 ms)
+    __shared__ T stage[kZDepth][2][NC][THREADS];
     int t = wrap(2 * k0 + Wv::FIRST - a.z_first, a.planes);
-    float ring[R][2][NC * V], next[2][NC * V];
-    auto fetch = [&]() {
+    float ring[R][2][NC * V];
+    auto fetch = [&](int slot) {
 #pragma unroll
         for (int r = 0; r < 2; r++) {
 #pragma unroll
             for (int n = 0; n < NC; n++)
-                *reinterpret_cast<T *>(&next[r][n * V]) =
-                    *reinterpret_cast<const T *>(src + n * a.src_chan + (int64_t)t * plane);
+                copy_async(&stage[slot][r][n][threadIdx.x], src + n * a.src_chan + (int64_t)t * plane);
             t = t + 1 == a.planes ? 0 : t + 1;
         }
     };
@@ -369,17 +400,24 @@ __global__ void __launch_bounds__(z_threads(NC), NC == 4 ? 5 : 3) k_dwt_z(const 
         return __fsqrt_rn(__fadd_rn(acc, __fmul_rn(c[3], c[3])));
     };
     const int steps = k1 - k0 + R - 1;
-    fetch();
+#pragma unroll
+    for (int s = 0; s < kZDepth - 1; s++) {
+        if (s < steps) fetch(s);
+        copy_commit();
+    }
     for (int s0 = 0; s0 < steps; s0 += R) {
 #pragma unroll
         for (int u = 0; u < R; u++) {
             const int step = s0 + u;
             if (step >= steps) break;
+            if (step + kZDepth - 1 < steps) fetch((step + kZDepth - 1) % kZDepth);
+            copy_commit();
+            copy_wait<kZDepth - 1>();
 #pragma unroll
             for (int r = 0; r < 2; r++)
 #pragma unroll
-                for (int c = 0; c < NC * V; c++) ring[u][r][c] = next[r][c];
-            if (step + 1 < steps) fetch();
+                for (int n = 0; n < NC; n++)
+                    *reinterpret_cast<T *>(&ring[u][r][n * V]) = stage[step % kZDepth][r][n][threadIdx.x];
             if (step < R - 1) continue;
             const int k = k0 + step - (R - 1);
             float lo[NC * V], hi[NC * V];
