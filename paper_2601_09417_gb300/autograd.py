@@ -16,7 +16,9 @@ class SplatRender(torch.autograd.Function):
     @staticmethod
     def forward(ctx, params, plan, cams_dev, bg=(0.0, 0.0, 0.0), view_begin=0, view_count=None):
         vc = plan.n_views - view_begin if view_count is None else view_count
-        img = torch.zeros((plan.n_views, 3, plan.height, plan.width), dtype=torch.float32, device=params.device)
+        # a call over all views writes every pixel; of a part of them, the other views' images are zero
+        new = torch.empty if vc == plan.n_views else torch.zeros
+        img = new((plan.n_views, 3, plan.height, plan.width), dtype=torch.float32, device=params.device)
         plan.forward(params, cams_dev, img, view_begin=view_begin, view_count=vc, bg=bg)
         ctx.plan, ctx.cams, ctx.bg, ctx.vb, ctx.vc = plan, cams_dev, bg, view_begin, vc
         ctx.save_for_backward(params)
@@ -25,7 +27,9 @@ class SplatRender(torch.autograd.Function):
     @staticmethod
     def backward(ctx, dimg):
         (params,) = ctx.saved_tensors
-        grad = torch.zeros_like(params)
+        # likewise the gradient's columns, where every column belongs to a set that some view sees
+        whole = ctx.vc == ctx.plan.n_views and ctx.plan.seen_by_all_views == params.shape[1]
+        grad = torch.empty_like(params) if whole else torch.zeros_like(params)
         ctx.plan.backward(params, ctx.cams, dimg.contiguous(), grad, view_begin=ctx.vb, view_count=ctx.vc,
                           bg=ctx.bg)
         return grad, None, None, None, None, None

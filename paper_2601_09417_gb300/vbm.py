@@ -139,8 +139,8 @@ def _ptr(t):
 
 
 def _stream():
-    import torch
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    import torch      # the raw handle: a Stream object costs 6 us a call
+    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def _dims(dims):
@@ -318,6 +318,9 @@ class Plan:
         h = ctypes.c_void_p()
         _check(lib.vbm_plan_create(ctypes.byref(d), ctypes.byref(h)))
         self.handle = h
+        # Gaussians that a call over all views gives a gradient: all of them, unless some set has no view
+        seen = {0} if vs is None else set(vs.tolist())
+        self.seen_by_all_views = int(so[-1]) if len(seen) == so.size - 1 else -1
 
     def close(self):
         if getattr(self, "handle", None) is not None and self.handle.value:
