@@ -5,16 +5,14 @@
 // Two tiled passes over each plane, each staging a 32 x 32 output tile plus a
 // 5-pixel halo in shared memory and applying the separable window as a
 // horizontal then a vertical pass:
-//   1. four windowed moments of x and y (the variances only as their sum) -> per-pixel SSIM and the three
+//   1. the five windowed moments of x and y -> per-pixel SSIM and the three
 //      maps its gradient needs (written to the workspace as a float2 and a
 //      float plane), plus per-block sums of |x - y| and SSIM;
 //   2. windowed sums of those maps -> dL/dx per pixel.
 // In both passes a thread slides the window along a row segment (horizontal)
 // or a column segment (vertical) held in registers, so each staged value is
-// read from shared memory once per pass; the moment pairs (x, y), (x^2 + y^2,
-// x y) and the map pair (g1, g2) are accumulated with packed FP32x2 FMAs.  Pass 1
-// is bound by instruction issue (five moments as two pairs and a single: step of
-// 32 uneven sets 2106 -> 2068 us, 8 x 512^2 789 -> 779 us).
+// read from shared memory once per pass; the moment pairs (x, y), (x^2, y^2)
+// and the map pair (g1, g2) are accumulated with packed FP32x2 FMAs.
 // The first block of pass 2 adds pass 1's per-block sums in double in a fixed
 // order (they are complete when pass 2 starts), so the loss value is
 // deterministic and needs no launch of its own.
@@ -103,12 +101,12 @@ __global__ void __launch_bounds__(kLossThreads) k_ssim_fwd(const float *__restri
                                                           float *__restrict__ g3, double *__restrict__ partial)
 {
     __shared__ __align__(16) float2 sxy[kSH][kSWP];
-    // horizontal sums of (x, y) and (x^2 + y^2, x y): SSIM and its gradient need
-    // the two variances only as their sum, so four moments do, as two pairs;
-    // rows padded by one element so the horizontal pass's lanes (11 rows at the
-    // same column) write to different banks
+    // horizontal sums of (x, y), (x^2, y^2) and x y; rows padded by one
+    // element so the horizontal pass's lanes (11 rows at the same column)
+    // write to different banks
     __shared__ __align__(16) float2 hm[kSH][kHP];
     __shared__ __align__(16) float2 hq[kSH][kHP];
+    __shared__ float hp[kSH][kHP];
     __shared__ float red[2][kLossThreads / 32];
     const int plane = blockIdx.z;
     const int ox = blockIdx.x * kTW, oy = blockIdx.y * kTH;
@@ -122,23 +120,28 @@ __global__ void __launch_bounds__(kLossThreads) k_ssim_fwd(const float *__restri
     if (t < kSH * kSegs) {
         const int r = t / kSegs, c0 = (t - r * kSegs) * kSeg;
         float2 v[kSeg + kWin - 1], sq[kSeg + kWin - 1];
+        float pr[kSeg + kWin - 1];
 #pragma unroll
         for (int j = 0; j < kSeg + kWin - 1; j++) {
             v[j] = sxy[r][c0 + j];
-            sq[j] = make_float2(fmaf(v[j].x, v[j].x, v[j].y * v[j].y), v[j].x * v[j].y);
+            sq[j] = __fmul2_rn(v[j], v[j]);
+            pr[j] = v[j].x * v[j].y;
         }
 #pragma unroll
         for (int o = 0; o < kSeg; o++) {
             float2 m = make_float2(0.f, 0.f), q = m;
+            float p = 0.f;
 #pragma unroll
             for (int k = 0; k < kWin; k++) {
                 const float w = c_win[k];
                 m = __ffma2_rn(f2(w), v[o + k], m);
                 q = __ffma2_rn(f2(w), sq[o + k], q);
+                p = fmaf(w, pr[o + k], p);
             }
             if (c0 + o < kTW) {
                 hm[r][c0 + o] = m;
                 hq[r][c0 + o] = q;
+                hp[r][c0 + o] = p;
             }
         }
     }
@@ -146,27 +149,31 @@ __global__ void __launch_bounds__(kLossThreads) k_ssim_fwd(const float *__restri
     const int c = t & 31, r0 = (t >> 5) * kVRows;
     float l1 = 0.f, ss = 0.f;
     float2 m_in[kVRows + kWin - 1], q_in[kVRows + kWin - 1];
+    float p_in[kVRows + kWin - 1];
 #pragma unroll
     for (int j = 0; j < kVRows + kWin - 1; j++) {
         m_in[j] = hm[r0 + j][c];
         q_in[j] = hq[r0 + j][c];
+        p_in[j] = hp[r0 + j][c];
     }
     const int gx = ox + c;
 #pragma unroll
     for (int o = 0; o < kVRows; o++) {
         float2 m = make_float2(0.f, 0.f), q = m;
+        float p = 0.f;
 #pragma unroll
         for (int k = 0; k < kWin; k++) {
             const float w = c_win[k];
             m = __ffma2_rn(f2(w), m_in[o + k], m);
             q = __ffma2_rn(f2(w), q_in[o + k], q);
+            p = fmaf(w, p_in[o + k], p);
         }
         const int gy = oy + r0 + o;
         if (gy >= H || gx >= W) continue;
         const float mx = m.x, my = m.y;
-        const float mxy = mx * my, msq = fmaf(mx, mx, my * my), cxy = q.y - mxy;
-        const float A1 = 2.f * mxy + kC1, A2 = 2.f * cxy + kC2;
-        const float B1 = msq + kC1, B2 = (q.x - msq) + kC2;
+        const float vx = q.x - mx * mx, vy = q.y - my * my, cxy = p - mx * my;
+        const float A1 = 2.f * mx * my + kC1, A2 = 2.f * cxy + kC2;
+        const float B1 = mx * mx + my * my + kC1, B2 = vx + vy + kC2;
         const float iB1 = rcp_approx(B1), iB2 = rcp_approx(B2);
         const float ssim = A1 * A2 * iB1 * iB2;
         const int64_t e = base + (int64_t)gy * W + gx;
