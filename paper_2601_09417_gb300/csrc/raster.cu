@@ -61,6 +61,7 @@ constexpr float kNegLog2e = -kLog2e;           // scales B
 constexpr int kNV = 9;                         // gradient partials per (pixel, splat)
 constexpr int kWarps = 4;                      // warps per block
 constexpr int kRegionCols = 8, kRegionRows = 4;   // thread positions of a warp region
+constexpr int kFilledRegions = 32768;          // forward regions that keep every SM's warps busy several times over
 
 __device__ __forceinline__ float ex2_approx(float x)
 {
@@ -317,7 +318,8 @@ struct PixState {
 // stored.
 // The entries are prefetched in registers, or, with rs (the backward's replay),
 // through its asynchronous shared-memory stages.
-template <int PPT, int GL, bool COLOR = true, bool EVAL = false>
+// UNROLL: list entries composited at a time.
+template <int PPT, int GL, bool COLOR = true, bool EVAL = false, int UNROLL = 1>
 __device__ __forceinline__ void fwd_region(const WarpGeom &wg, const int2 *__restrict__ ranges,
                                            const uint32_t *__restrict__ pair_item, const SplatRec *__restrict__ rec, int W, int H, int vb, float bg0,
                                            float bg1, float bg2, float *__restrict__ img,
@@ -389,53 +391,68 @@ __device__ __forceinline__ void fwd_region(const WarpGeom &wg, const int2 *__res
             nxt = nxt2;
             it_next = it_after;
         }
+        // UNROLL entries at a time: their alphas do not depend on one another, only
+        // the transmittance does
         while (m) {                                    // no warp collectives inside
-            const int j = __ffs(m) - 1;
-            m &= m - 1;
-            const float4 g = s.geo[j];
-            const float2 cp = s.cp[j];
-            const float4 c = s.col[j];
-            const int pos1 = __float_as_int(cp.y);
-            const float dx = __fsub_rn(g.x, wg.pxc);
-            const float t0 = __fmul_rn(__fmul_rn(g.z, dx), dx);
-            const float bdx = __fmul_rn(g.w, dx);
+            float4 c[UNROLL];
+            int pos1[UNROLL];
+            float p2[UNROLL][PPT], raw[UNROLL][PPT];
 #pragma unroll
-            for (int k = 0; k < PPT; k += STEP) {
-                float p2[2], raw[2];
-                if (PPT == 1) {
-                    const float dy = __fsub_rn(g.y, pyc[k]);
-                    const float t = __fmaf_rn(__fmul_rn(cp.x, dy), dy, t0);
-                    p2[0] = __fmaf_rn(bdx, dy, t);
-                    raw[0] = __fmul_rn(c.w, ex2_approx(p2[0]));
-                } else {
-                    // a - b == a + (-b) exactly, so this matches __fsub_rn in the backward
-                    const float2 dy = __fadd2_rn(make_float2(g.y, g.y), make_float2(-pyc[k], -pyc[k + STEP - 1]));
-                    const float2 t = __ffma2_rn(__fmul2_rn(make_float2(cp.x, cp.x), dy), dy, make_float2(t0, t0));
-                    const float2 q = __ffma2_rn(make_float2(bdx, bdx), dy, t);
-                    p2[0] = q.x;
-                    p2[1] = q.y;
-                    const float2 r = __fmul2_rn(make_float2(c.w, c.w), make_float2(ex2_approx(q.x), ex2_approx(q.y)));
-                    raw[0] = r.x;
-                    raw[1] = r.y;
+            for (int e = 0; e < UNROLL; e++) {
+                const bool some = e == 0 || m != 0;    // past the group's last entry: never blends
+                const int j = e == 0 ? __ffs(m) - 1 : (__ffs(m) - 1) & 31;
+                m &= m - 1;
+                const float4 g = s.geo[j];
+                const float2 cp = s.cp[j];
+                c[e] = s.col[j];
+                pos1[e] = __float_as_int(cp.y);
+                const float dx = __fsub_rn(g.x, wg.pxc);
+                const float t0 = __fmul_rn(__fmul_rn(g.z, dx), dx);
+                const float bdx = __fmul_rn(g.w, dx);
+#pragma unroll
+                for (int k = 0; k < PPT; k += STEP) {
+                    if (PPT == 1) {
+                        const float dy = __fsub_rn(g.y, pyc[k]);
+                        const float t = __fmaf_rn(__fmul_rn(cp.x, dy), dy, t0);
+                        p2[e][0] = __fmaf_rn(bdx, dy, t);
+                        raw[e][0] = __fmul_rn(c[e].w, ex2_approx(p2[e][0]));
+                    } else {
+                        // a - b == a + (-b) exactly, so this matches __fsub_rn in the backward
+                        const float2 dy = __fadd2_rn(make_float2(g.y, g.y), make_float2(-pyc[k], -pyc[k + STEP - 1]));
+                        const float2 t = __ffma2_rn(__fmul2_rn(make_float2(cp.x, cp.x), dy), dy, make_float2(t0, t0));
+                        const float2 q = __ffma2_rn(make_float2(bdx, bdx), dy, t);
+                        p2[e][k] = q.x;
+                        p2[e][k + STEP - 1] = q.y;
+                        const float2 r =
+                            __fmul2_rn(make_float2(c[e].w, c[e].w), make_float2(ex2_approx(q.x), ex2_approx(q.y)));
+                        raw[e][k] = r.x;
+                        raw[e][k + STEP - 1] = r.y;
+                    }
                 }
+                if (e > 0) {
 #pragma unroll
-                for (int h = 0; h < STEP; h++) {
-                    const int kk = k + h;
-                    const float alpha = fminf(kAlphaMax, raw[h]);
-                    const bool cand = !done[kk] && p2[h] <= 0.f && alpha >= kAlphaMin;
+                    for (int k = 0; k < PPT; k++) raw[e][k] = some ? raw[e][k] : 0.f;
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < UNROLL; e++) {
+#pragma unroll
+                for (int kk = 0; kk < PPT; kk++) {
+                    const float alpha = fminf(kAlphaMax, raw[e][kk]);
+                    const bool cand = !done[kk] && p2[e][kk] <= 0.f && alpha >= kAlphaMin;
                     const float testT = __fmaf_rn(-alpha, T[kk], T[kk]);   // T (1 - alpha), one rounding
                     const bool term = cand && testT < kTMin;
                     const bool blend = cand && !term;
                     done[kk] = done[kk] || term;
-                    if (EVAL && term) evaluated[kk] = pos1;
+                    if (EVAL && term) evaluated[kk] = pos1[e];
                     if (COLOR && blend) {
                         const float wgt = __fmul_rn(alpha, T[kk]);
-                        C0[kk] = __fmaf_rn(c.x, wgt, C0[kk]);
-                        C1[kk] = __fmaf_rn(c.y, wgt, C1[kk]);
-                        C2[kk] = __fmaf_rn(c.z, wgt, C2[kk]);
+                        C0[kk] = __fmaf_rn(c[e].x, wgt, C0[kk]);
+                        C1[kk] = __fmaf_rn(c[e].y, wgt, C1[kk]);
+                        C2[kk] = __fmaf_rn(c[e].z, wgt, C2[kk]);
                     }
                     T[kk] = blend ? testT : T[kk];
-                    last[kk] = blend ? pos1 : last[kk];
+                    last[kk] = blend ? pos1[e] : last[kk];
                 }
             }
         }
@@ -855,7 +872,7 @@ __device__ __forceinline__ bool next_item(int &q, int w_global, int n_items_w, i
     return q < n_items_w;
 }
 
-template <int PPT, int GL, bool PERSIST, bool EVAL>
+template <int PPT, int GL, bool PERSIST, bool EVAL, int UNROLL>
 __global__ void __launch_bounds__(kWarps * 32)
     k_raster_fwd(const int *__restrict__ order, int *__restrict__ queue, int n_items_w, int n_regions,
                  const int2 *__restrict__ ranges, const uint32_t *__restrict__ pair_item,
@@ -874,7 +891,7 @@ __global__ void __launch_bounds__(kWarps * 32)
         const WarpGeom wg = warp_geom<PPT, GL>(tile, q % n_regions, tw, th, TX, TY, W, H);
         if (wg.x0 > wg.x1 || wg.y0 > wg.y1) continue;            // region outside the image
         const int cb = ckpt_base ? ckpt_base[tile] : -1;
-        fwd_region<PPT, GL, true, EVAL>(wg, ranges, pair_item, rec, W, H, vb, bg0, bg1, bg2, img, alpha_out,
+        fwd_region<PPT, GL, true, EVAL, UNROLL>(wg, ranges, pair_item, rec, W, H, vb, bg0, bg1, bg2, img, alpha_out,
                             T_final, n_contrib, n_eval, s, nullptr, nullptr,
                             cb >= 0 ? ckpt + (int64_t)cb * tile_px : nullptr, seg_len, tw, tile_px);
     }
@@ -994,8 +1011,15 @@ vbm_status launch_fwd(vbm_plan *p, int vb, int vc, const float bg[3], float *img
     // variants launched while that hook is set
     const bool eval = p->prof_n_eval != nullptr;
     int32_t *nc_out = p->n_contrib ? p->n_contrib : p->prof_n_contrib;
+    // two list entries at a time: their alphas are independent, which hides a
+    // step's latency where a thread has one pixel and the regions are too few
+    // to fill the chip (1 x 128^2: step 103 -> 98 us; 8 x 512^2, 65,536 regions:
+    // 786 -> 792), and pairs well with two pixels (1080p frame 619 -> 608 us)
+    constexpr int MORE = PPT <= 2 ? 2 : 1, FILLED = PPT == 2 ? 2 : 1;
+    const bool more = n_items_w < kFilledRegions;
     if (p->desc.flags & VBM_PLAN_PERSISTENT) {
-        auto kernel = eval ? k_raster_fwd<PPT, GL, true, true> : k_raster_fwd<PPT, GL, true, false>;
+        auto kernel = eval ? k_raster_fwd<PPT, GL, true, true, 1>
+                           : more ? k_raster_fwd<PPT, GL, true, false, MORE> : k_raster_fwd<PPT, GL, true, false, FILLED>;
         const int grid = persistent_grid(kernel, n_items_w);
         kernel<<<grid, kWarps * 32, 0, st>>>(p->tile_order, p->tile_queue, n_items_w, nr, p->ranges, p->pair_item,
                                              p->rec, p->desc.width, p->desc.height, p->desc.tile_w, p->desc.tile_h,
@@ -1003,7 +1027,9 @@ vbm_status launch_fwd(vbm_plan *p, int vb, int vc, const float bg[3], float *img
                                              p->prof_n_eval, p->ckpt, p->seg_len ? p->ckpt_base : nullptr,
                                              p->seg_len);
     } else {
-        auto kernel = eval ? k_raster_fwd<PPT, GL, false, true> : k_raster_fwd<PPT, GL, false, false>;
+        auto kernel = eval ? k_raster_fwd<PPT, GL, false, true, 1>
+                           : more ? k_raster_fwd<PPT, GL, false, false, MORE>
+                                  : k_raster_fwd<PPT, GL, false, false, FILLED>;
         kernel<<<(n_items_w + kWarps - 1) / kWarps, kWarps * 32, 0, st>>>(
             nullptr, nullptr, n_items_w, nr, p->ranges, p->pair_item, p->rec, p->desc.width, p->desc.height,
             p->desc.tile_w, p->desc.tile_h, p->TX, p->TY, vb, bg[0], bg[1], bg[2], img, alpha, p->T_final, nc_out,
