@@ -15,7 +15,8 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("W,H,V,recompute,length", [
     (96, 72, 2, False, 64), (101, 67, 1, True, 64),        # small batches: segments of 64
     (1024, 1023, 1, False, 64), (1024, 1024, 1, True, 256),   # either side of 2^20 pixels
-    (512, 512, 4, False, 256)])
+    (512, 512, 4, False, 256),
+    (1040, 1024, 1, False, 256), (1040, 1024, 1, True, 256)])   # more than 4096 tiles: claims by the warp
 def test_default_plan_splits_lists(cuda_lib, W, H, V, recompute, length):
     """The forward is unchanged bit for bit and the gradients equal those of whole walks
     (segment_len -1, 32-lane groups) up to FP32 rounding, also when the splats crowd a small
