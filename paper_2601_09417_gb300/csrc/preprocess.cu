@@ -272,8 +272,11 @@ __global__ void __launch_bounds__(32, 20) k_preprocess_bwd(const float *P, int64
                                  const int32_t *__restrict__ scene_view_ptr, const int32_t *__restrict__ scene_views,
                                  const int64_t *__restrict__ view_item_offset, int vb, int vc,
                                  const float *__restrict__ gs, float *__restrict__ grad, int accumulate,
-                                 int64_t g_begin, int64_t g_end, AdamArgs a)
+                                 int64_t g_begin, int64_t g_end, AdamArgs a, int *__restrict__ bwd_queue)
 {
+    // the backward compositing kernel has spent its work queue: ready for the next
+    // backward of the same forward (also when a captured backward is replayed)
+    if (blockIdx.x == 0 && threadIdx.x == 0) *bwd_queue = 0;
     const int64_t g = (ADAM ? 0 : g_begin) + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (ADAM ? g >= a.n : g >= g_end) return;
     if (ADAM && (g < g_begin || g >= g_end)) {   // no view of the call renders g's scene
@@ -452,13 +455,15 @@ vbm_status preprocess_bwd(vbm_plan *p, const float *params, int64_t stride, cons
         if (na == 0) return VBM_OK;
         k_preprocess_bwd<true><<<(unsigned)((na + 31) / 32), 32, 0, st>>>(
             params, stride, cams, p->d_scene_offset, p->desc.n_scenes, p->d_scene_view_ptr, p->d_scene_views,
-            p->d_view_item_offset, vb, vc, p->g_splat, nullptr, 0, g_begin, std::min(g_end, na), *adam);
+            p->d_view_item_offset, vb, vc, p->g_splat, nullptr, 0, g_begin, std::min(g_end, na), *adam,
+            p->tile_queue + 1);
     } else {
         k_preprocess_bwd<false><<<(unsigned)((n + 31) / 32), 32, 0, st>>>(
             params, stride, cams, p->d_scene_offset, p->desc.n_scenes, p->d_scene_view_ptr, p->d_scene_views,
-            p->d_view_item_offset, vb, vc, p->g_splat, grad, accumulate, g_begin, g_end, AdamArgs{});
+            p->d_view_item_offset, vb, vc, p->g_splat, grad, accumulate, g_begin, g_end, AdamArgs{}, p->tile_queue + 1);
     }
     VBM_LAUNCH("preprocess_bwd");
+    p->bwd_queue_used = false;
     note_launches(1);
     return VBM_OK;
 }

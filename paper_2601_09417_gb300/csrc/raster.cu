@@ -1051,8 +1051,8 @@ vbm_status launch_bwd(vbm_plan *p, int vb, int vc, const float bg[3], const floa
     const int n_items_w = n_tiles * nr;
     record_event(p->prof_ev[2], st);
     if ((p->desc.flags & VBM_PLAN_PERSISTENT) || p->seg_len) {
-        // a second backward of the same forward finds the backward's queue
-        // counter spent: clear it (the binning clears it for the first)
+        // the projection backward clears the queue counter behind every backward;
+        // where none ran (no columns), it is cleared here
         if (p->bwd_queue_used) VBM_CUDA(cudaMemsetAsync(p->tile_queue + 1, 0, sizeof(int), st));
         p->bwd_queue_used = true;
         const int grid = persistent_grid(k_raster_bwd<PPT, GL, true>, n_items_w);

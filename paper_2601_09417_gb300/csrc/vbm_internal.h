@@ -497,8 +497,8 @@ struct vbm_plan {
     float *g_splat = nullptr;               // [items][kGradStride]
     bool g_splat_clear = false;             // host: zeroed by the last forward, no backward since
     bool bwd_seen = false;                  // host: a backward has run on this plan
-    bool bwd_queue_used = false;            // host: a persistent backward has taken its work queue since
-                                            // the last binning zeroed the counters
+    bool bwd_queue_used = false;            // host: a backward has taken its work queue and no projection
+                                            // backward (or binning) has cleared the counter since
 
     // pairs
     uint64_t *pair_key = nullptr;            // [pairs] (depth bits << 32 | item), bucketed by tile

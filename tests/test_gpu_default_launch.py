@@ -61,3 +61,34 @@ def test_default_plan_splits_lists(cuda_lib, W, H, V, recompute, length):
         for lo, hi in [(0, 3), (3, 6), (6, 10), (10, 11), (11, 14)]:
             nrm, elt = rel_group_error(g[lo:hi], ref[lo:hi])
             assert nrm < 1e-4 and elt < 1e-4, (lo, nrm, elt)
+
+
+@pytest.mark.parametrize("flags,seg", [(0, 0), (0, -1), (2, 0)])
+def test_captured_backward_replays_after_one_forward(cuda_lib, flags, seg):
+    """A backward captured by itself gives the same gradient at every replay: its splat
+    gradients and its work queue are cleared each time."""
+    vbm = cuda_lib
+    W, H, V, G = 96, 72, 2, 32
+    P = random_gaussians(3000, 12.0, 20.0, seed=3, scale_range=(0.3, 1.2),
+                         opacity_logit_range=(-4.5, -2.5)).astype(np.float32)
+    params, cams_dev = to_device(P, orbit_cameras((G, G, G), V, W, H))
+    w = torch.from_numpy(np.random.default_rng(V).standard_normal((V, 3, H, W)).astype(np.float32)).cuda()
+    plan = vbm.Plan([0, P.shape[1]], V, W, H, pair_capacity=1 << 22, segment_len=seg, flags=flags)
+    img, grad = torch.zeros((V, 3, H, W), device="cuda"), torch.zeros_like(params)
+    plan.forward(params, cams_dev, img)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        plan.backward(params, cams_dev, w, grad)
+    got = []
+    for _ in range(3):
+        grad.fill_(float("nan"))
+        graph.replay()
+        got.append(grad.cpu().numpy())
+    ref = torch.zeros_like(params)
+    plan.forward(params, cams_dev, img)
+    plan.backward(params, cams_dev, w, ref)
+    for g in got:
+        for lo, hi in [(0, 3), (3, 6), (6, 10), (10, 11), (11, 14)]:
+            nrm, elt = rel_group_error(g[lo:hi], ref.cpu().numpy()[lo:hi])
+            assert nrm < 1e-5 and elt < 1e-4, (lo, nrm, elt)
