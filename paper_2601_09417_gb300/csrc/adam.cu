@@ -17,6 +17,15 @@ __global__ void k_step_inc(int32_t *step)
     if (threadIdx.x == 0 && blockIdx.x == 0) *step += 1;
 }
 
+// For the step fused into the projection backward: also the bias corrections.
+__global__ void k_step_count(int32_t *step, float beta1, float beta2, float2 *bias)
+{
+    if (threadIdx.x != 0) return;
+    const int t = *step + 1;
+    *step = t;
+    *bias = adam_bias_corrections(t, beta1, beta2);
+}
+
 // the bias corrections are the same for every scalar: one thread of the block
 // evaluates them
 __device__ __forceinline__ void bias_corrections(float *s_bc, const int32_t *step, float beta1, float beta2)
@@ -109,6 +118,14 @@ __global__ void k_adam_rows(float *__restrict__ P, const float *__restrict__ G, 
 }
 
 }  // namespace
+
+vbm_status adam_step_count(const AdamArgs &a, cudaStream_t st)
+{
+    k_step_count<<<1, 32, 0, st>>>(a.step, a.beta1, a.beta2, a.bias);
+    VBM_LAUNCH("adam_step_count");
+    note_launches(1);
+    return VBM_OK;
+}
 
 vbm_status adam_step(float *P, const float *G, float *M, float *V, int64_t n, int64_t stride, int32_t *step,
                      const float lrs[5], float beta1, float beta2, float eps, uint32_t *nonfinite, cudaStream_t st)

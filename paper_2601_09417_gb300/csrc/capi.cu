@@ -324,7 +324,7 @@ vbm_status vbm_raster_bwd(vbm_plan *p, const float *params, int64_t stride, cons
     VBM_ARG(vb == p->last_view_begin && vc == p->last_view_count,
             "backward views differ from the last forward call on this plan");
     cudaStream_t st = (cudaStream_t)stream;
-    s = raster_bwd(p, vb, vc, bg, dimg, dalpha, nullptr, st);
+    s = raster_bwd(p, vb, vc, bg, dimg, dalpha, st);
     if (s == VBM_OK) s = preprocess_bwd(p, params, stride, cams, vb, vc, grad, accumulate, st);
     record_event(p->prof_ev[6], st);
     return s;
@@ -354,7 +354,8 @@ vbm_status vbm_raster_bwd_adam(vbm_plan *p, float *params, int64_t stride, const
     a.eps = eps;
     a.nonfinite = nonfinite;
     a.bias = p->d_bias;
-    s = raster_bwd(p, vb, vc, bg, dimg, dalpha, &a, st);
+    s = raster_bwd(p, vb, vc, bg, dimg, dalpha, st);
+    if (s == VBM_OK) s = adam_step_count(a, st);
     if (s == VBM_OK) s = preprocess_bwd(p, params, stride, cams, vb, vc, nullptr, 0, st, &a);
     record_event(p->prof_ev[6], st);
     return s;

@@ -692,7 +692,7 @@ __device__ __forceinline__ void bwd_region(const WarpGeom &wg, const int2 *__res
     int my_max = 0;
     PixState<PPT> replay;
     if (!T_final && seg < 0)   // recompute mode, whole list: replay the forward decisions of this region
-        fwd_region<PPT, GL, false>(wg, ranges, pair_item, rec, W, H, vb, bg0, bg1, bg2, nullptr,
+        fwd_region<PPT, GL, false, false, PPT == 2 ? 2 : 1>(wg, ranges, pair_item, rec, W, H, vb, bg0, bg1, bg2, nullptr,
                                    nullptr, nullptr, nullptr, nullptr, s, &replay, &rs);
 #pragma unroll
     for (int k = 0; k < PPT; k++) {
@@ -897,14 +897,6 @@ __global__ void __launch_bounds__(kWarps * 32)
     }
 }
 
-// What the backward does for an Adam step fused behind it (step NULL: none):
-// count the step and evaluate its bias corrections.
-struct StepCount {
-    int32_t *step;
-    float beta1, beta2;
-    float2 *bias;
-};
-
 template <int PPT, int GL, bool PERSIST>
 __global__ void __launch_bounds__(kWarps * 32)
     k_raster_bwd(const int *__restrict__ order, int *__restrict__ queue, int n_items_w, int n_regions,
@@ -913,13 +905,8 @@ __global__ void __launch_bounds__(kWarps * 32)
                  float bg1, float bg2, const float *__restrict__ dimg, const float *__restrict__ dalpha,
                  const float *__restrict__ T_final, const int32_t *__restrict__ n_contrib, float *__restrict__ gs,
                  const int *__restrict__ seg_count, const int2 *__restrict__ seg_units,
-                 const float4 *__restrict__ ckpt, const int *__restrict__ ckpt_base, int seg_len, StepCount sc)
+                 const float4 *__restrict__ ckpt, const int *__restrict__ ckpt_base, int seg_len)
 {
-    if (sc.step && blockIdx.x == 0 && threadIdx.x == 0) {
-        const int t = *sc.step + 1;
-        *sc.step = t;
-        *sc.bias = adam_bias_corrections(t, sc.beta1, sc.beta2);
-    }
     __shared__ WarpSlots slots[kWarps];
     __shared__ RawStages raw[kWarps];
     __shared__ float acc_s[kWarps][32][kNV];
@@ -1043,9 +1030,8 @@ vbm_status launch_fwd(vbm_plan *p, int vb, int vc, const float bg[3], float *img
 
 template <int PPT, int GL>
 vbm_status launch_bwd(vbm_plan *p, int vb, int vc, const float bg[3], const float *dimg, const float *dalpha,
-                      const AdamArgs *adam, cudaStream_t st)
+                      cudaStream_t st)
 {
-    const StepCount sc = adam ? StepCount{adam->step, adam->beta1, adam->beta2, adam->bias} : StepCount{};
     const int n_tiles = vc * p->TX * p->TY;
     const int nr = regions_per_tile(p, PPT);
     const int n_items_w = n_tiles * nr;
@@ -1059,11 +1045,11 @@ vbm_status launch_bwd(vbm_plan *p, int vb, int vc, const float bg[3], const floa
         k_raster_bwd<PPT, GL, true><<<grid, kWarps * 32, 0, st>>>(
             p->tile_order, p->tile_queue + 1, n_items_w, nr, p->ranges, p->pair_item, p->rec, p->desc.width, p->desc.height, p->desc.tile_w, p->desc.tile_h, p->TX, p->TY, vb,
             bg[0], bg[1], bg[2], dimg, dalpha, p->T_final, p->n_contrib, p->g_splat, p->tile_queue,
-            p->seg_len ? p->seg_units : nullptr, p->ckpt, p->ckpt_base, p->seg_len, sc);
+            p->seg_len ? p->seg_units : nullptr, p->ckpt, p->ckpt_base, p->seg_len);
     } else {
         k_raster_bwd<PPT, GL, false><<<(n_items_w + kWarps - 1) / kWarps, kWarps * 32, 0, st>>>(
             nullptr, nullptr, n_items_w, nr, p->ranges, p->pair_item, p->rec, p->desc.width, p->desc.height, p->desc.tile_w, p->desc.tile_h, p->TX, p->TY, vb, bg[0], bg[1],
-            bg[2], dimg, dalpha, p->T_final, p->n_contrib, p->g_splat, nullptr, nullptr, nullptr, nullptr, 0, sc);
+            bg[2], dimg, dalpha, p->T_final, p->n_contrib, p->g_splat, nullptr, nullptr, nullptr, nullptr, 0);
     }
     VBM_LAUNCH("raster_bwd");
     record_event(p->prof_ev[3], st);
@@ -1097,7 +1083,7 @@ vbm_status raster_fwd(vbm_plan *p, int vb, int vc, const float bg[3], float *img
 }
 
 vbm_status raster_bwd(vbm_plan *p, int vb, int vc, const float bg[3], const float *dimg, const float *dalpha,
-                      const AdamArgs *adam, cudaStream_t st)
+                      cudaStream_t st)
 {
     // the forward's projection zeroed the splat-gradient records (once the
     // plan has run a backward); otherwise, and for a second backward of the
@@ -1105,7 +1091,7 @@ vbm_status raster_bwd(vbm_plan *p, int vb, int vc, const float bg[3], const floa
     if (!p->g_splat_clear) VBM_CUDA(cudaMemsetAsync(p->g_splat, 0, sizeof(float) * kGradStride * p->last_items, st));
     p->g_splat_clear = false;
     p->bwd_seen = true;
-    VBM_RASTER_DISPATCH(launch_bwd, true, p, vb, vc, bg, dimg, dalpha, adam, st)
+    VBM_RASTER_DISPATCH(launch_bwd, true, p, vb, vc, bg, dimg, dalpha, st)
 }
 
 }  // namespace vbm
