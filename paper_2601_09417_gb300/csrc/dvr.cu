@@ -31,7 +31,8 @@ constexpr int kOccupancyThreads = kOccupancyCols + 32;
 
 // Scalars f <= lo and f >= hi have no opacity: the transfer function's alpha is
 // 0 (or less) from its first knot up to a knot at lo, and from a knot at hi to
-// its last.  The margins cover the rounding of the interpolated value, so that
+// its last.  An absent bound is NaN, which no scalar compares with, infinite
+// ones included; lo is +infinity where no scalar has opacity.  The margins cover the rounding of the interpolated value, so that
 // a block all of whose corners lie beyond one of them holds no sample with
 // opacity; with lo = 0 (alpha rises from the first knot) corners of at most 0
 // interpolate to at most 0 exactly.
@@ -42,11 +43,12 @@ struct NoOpacity {
 NoOpacity no_opacity(const vbm_tf *tf)
 {
     const float inf = std::numeric_limits<float>::infinity();
-    NoOpacity r{-inf, inf};
+    const float absent = std::numeric_limits<float>::quiet_NaN();
+    NoOpacity r{absent, absent};
     const int n = tf->n_knots;
     int k = 0;
     while (k < n && tf->rgba[k][3] <= 0.f) k++;
-    if (k == n) return NoOpacity{inf, inf};                  // no opacity anywhere
+    if (k == n) return NoOpacity{inf, absent};               // no opacity anywhere
     if (k > 0 && tf->x[k - 1] >= 0.f) r.lo = tf->x[k - 1] * (1.f - 1e-5f);
     k = n - 1;
     while (k >= 0 && tf->rgba[k][3] <= 0.f) k--;
@@ -57,7 +59,12 @@ NoOpacity no_opacity(const vbm_tf *tf)
 // Occupancy words: bit b of word (bz, by, w) is block (32 w + b, by, bz).  One
 // thread a column of x, over the 9 x 9 rows whose voxels are corners of the
 // blocks' cells; a block then takes its 9 columns.  A voxel that is not
-// comparable (NaN) counts as occupied.
+// comparable (NaN) counts as occupied, and so does one at or above kMarkMax, from
+// which an interpolation can overflow: infinity times a weight of 0 is NaN and
+// reads as the scalar 0.  (Below lo nothing need be excluded: a bound there
+// means that 0 has no opacity either.)
+constexpr float kMarkMax = 1e38f;
+
 __global__ void __launch_bounds__(kOccupancyThreads) k_occupancy(const float *__restrict__ F, int nx, int ny, int nz,
                                                                  NoOpacity none, uint32_t *__restrict__ words)
 {
@@ -75,7 +82,7 @@ __global__ void __launch_bounds__(kOccupancyThreads) k_occupancy(const float *__
 #pragma unroll
                 for (int k = 0; k <= kCell; k++) {
                     lo &= v[k] <= none.lo;
-                    hi &= v[k] >= none.hi;
+                    hi &= v[k] >= none.hi && v[k] < kMarkMax;
                 }
             }
         }
