@@ -217,10 +217,16 @@ __global__ void __launch_bounds__(kDvrThreads) k_dvr(const float *__restrict__ F
     const float box[3] = {(float)nx, (float)ny, (float)nz};
     float t0 = 0.f, t1 = 3.4e38f;
     bool miss = false;
-    float inv_d[3];
+    // Steps per axis to a block's face: (8 c + face[k] - q[k]) inv_d[k] from the
+    // position q in block c.  A ray that does not move along an axis leaves the
+    // block through neither face: it looks at the one ahead of its q, infinitely
+    // far (a face at or behind q sent such a ray's empty space through the
+    // occupancy words sample by sample: 65536 x 16 x 16 at a step of 0.05, 200 ->
+    // 1.3 ms).
+    float inv_d[3], face[3];
 #pragma unroll
     for (int k = 0; k < 3; k++) {
-        inv_d[k] = 1e30f;
+        inv_d[k] = o[k] - 0.5f > fmaxf(box[k] - 2.f, 0.f) ? -1e30f : 1e30f;
         if (d[k] != 0.f) {
             const float inv = 1.f / d[k];
             inv_d[k] = inv;
@@ -230,6 +236,7 @@ __global__ void __launch_bounds__(kDvrThreads) k_dvr(const float *__restrict__ F
         } else if (o[k] < 0.f || o[k] > box[k]) {
             miss = true;
         }
+        face[k] = inv_d[k] > 0.f ? (float)kCell : 0.f;
     }
     float C0 = 0.f, C1 = 0.f, C2 = 0.f, T = 1.f;
     const bool hit = inside && !miss && t1 > t0;
@@ -269,7 +276,7 @@ __global__ void __launch_bounds__(kDvrThreads) k_dvr(const float *__restrict__ F
                 float leave = 1e6f;
 #pragma unroll
                 for (int k = 0; k < 3; k++)
-                    leave = fminf(leave, ((float)(kCell * (c[k] + (d[k] > 0.f))) - q[k]) * inv_d[k]);
+                    leave = fminf(leave, (__fmaf_rn((float)kCell, (float)c[k], face[k]) - q[k]) * inv_d[k]);
                 m_end = m + min(nseg - m, 1 + max(0, (int)fminf(leave * inv_step - 0.01f, 1e6f)));
                 const uint32_t word = words[((int64_t)c[2] * block_rows + c[1]) * word_cols + (c[0] >> 5)];
                 if (!((word >> (c[0] & 31)) & 1u)) m = m_end;
