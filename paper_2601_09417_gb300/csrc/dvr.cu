@@ -238,6 +238,17 @@ __global__ void __launch_bounds__(kDvrThreads) k_dvr(const float *__restrict__ F
         }
         face[k] = inv_d[k] > 0.f ? (float)kCell : 0.f;
     }
+    // The face is taken this much too near, so that the samples up to it lie in
+    // the block as their positions round.  A position is the float32 of o + tm d
+    // - 1/2 with tm the float32 of t0 + (m + 1/2) step: two samples' positions
+    // differ from the exact multiple of the step by at most 6 2^-24 (t1 + n)
+    // together (three roundings up to t1 and two up to n voxels for each), and
+    // 1e-5 covers the distance's own.  Towards the face they come in order, so
+    // none falls back behind the block's other faces.
+    const float margin = __fmaf_rn(0x1p-21f, t1 + fmaxf(fmaxf(box[0], box[1]), box[2]), 1e-5f);
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+        if (d[k] != 0.f) face[k] -= copysignf(margin, d[k]);
     float C0 = 0.f, C1 = 0.f, C2 = 0.f, T = 1.f;
     const bool hit = inside && !miss && t1 > t0;
     const int nseg = hit ? (int)ceilf((t1 - t0) / step) : 0;
@@ -271,13 +282,12 @@ __global__ void __launch_bounds__(kDvrThreads) k_dvr(const float *__restrict__ F
                     q[k] = __fadd_rn(__fmaf_rn(tm, d[k], o[k]), -0.5f);
                     c[k] = cell_of(q[k], last[k], top[k], f) >> kCellShift;
                 }
-                // samples from m on that lie in this block for certain (0.01
-                // of a step short of the ray's exit covers the rounding)
+                // samples from m on that lie in this block for certain
                 float leave = 1e6f;
 #pragma unroll
                 for (int k = 0; k < 3; k++)
                     leave = fminf(leave, (__fmaf_rn((float)kCell, (float)c[k], face[k]) - q[k]) * inv_d[k]);
-                m_end = m + min(nseg - m, 1 + max(0, (int)fminf(leave * inv_step - 0.01f, 1e6f)));
+                m_end = m + min(nseg - m, 1 + max(0, (int)fminf(leave * inv_step, 1e6f)));
                 const uint32_t word = words[((int64_t)c[2] * block_rows + c[1]) * word_cols + (c[0] >> 5)];
                 if (!((word >> (c[0] & 31)) & 1u)) m = m_end;
             }
