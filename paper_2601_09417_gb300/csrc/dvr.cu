@@ -199,8 +199,11 @@ __global__ void __launch_bounds__(kDvrThreads) k_dvr(const float *__restrict__ F
     __syncthreads();
     const int v = blockIdx.z;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int px = blockIdx.x * 16 + (warp & 1) * 8 + (lane & 7);
-    const int py = blockIdx.y * (kDvrThreads / 16) + (warp >> 1) * 4 + (lane >> 3);
+    // the image's blocks row by row along the grid's first axis, whose extent no
+    // image reaches (the second holds 65535)
+    const int block_cols = (W + 15) / 16, by = blockIdx.x / block_cols, bx = blockIdx.x - by * block_cols;
+    const int px = bx * 16 + (warp & 1) * 8 + (lane & 7);
+    const int py = by * (kDvrThreads / 16) + (warp >> 1) * 4 + (lane >> 3);
     const bool inside = px < W && py < H;                // every lane stays for the warp's votes
     const vbm_camera cam = cams[v];
     const float dcx = (px + 0.5f - cam.cx) / cam.fx, dcy = (py + 0.5f - cam.cy) / cam.fy;   // and 1 along z
@@ -387,7 +390,9 @@ vbm_status render_dvr(const float *F, const int dims[3], const vbm_tf *tf, const
     const dim3 marks = occupancy_grid(dims);
     uint32_t *words = (uint32_t *)ws;
     if (marks.y > 65535 || marks.z > 65535) words = nullptr;     // beyond a grid's extent
-    dim3 grid((W + 15) / 16, (H + kDvrThreads / 16 - 1) / (kDvrThreads / 16), n_views);
+    const int64_t blocks = (int64_t)((W + 15) / 16) * ((H + kDvrThreads / 16 - 1) / (kDvrThreads / 16));
+    VBM_ARG(blocks <= INT_MAX, "image too large");
+    dim3 grid((unsigned)blocks, 1, n_views);
     const bool general = std::min({dims[0], dims[1], dims[2]}) < 2 ||
                          (int64_t)dims[0] * dims[1] * dims[2] >= (int64_t)1 << 30;
     if (words) {
