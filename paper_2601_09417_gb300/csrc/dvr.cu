@@ -101,15 +101,23 @@ __global__ void __launch_bounds__(kOccupancyThreads) k_occupancy(const float *__
     if (threadIdx.x == 0) words[((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = word;
 }
 
-// Lower cell corner and fraction of a clamped coordinate q (n voxels): adding
-// 2^23 rounding down leaves floor(q) in the low mantissa bits, without
-// conversions.
-constexpr float kFloorMagic = 8388608.f;
+// Lower cell corner and fraction of a clamped coordinate q (n voxels, last = n -
+// 1).  Up to 2^23 voxels adding 2^23 rounding down leaves floor(q) in the low
+// mantissa bits, without conversions (top: 2^23 + the last lower corner); the
+// GENERAL march converts.
+constexpr int kFloorMax = 1 << 23;
+constexpr float kFloorMagic = (float)kFloorMax;
 constexpr int kFloorBits = 0x4B000000;
 
-__device__ __forceinline__ int cell_of(float q, float last, float top, float &frac)
+template <bool GENERAL>
+__device__ __forceinline__ int cell_of(float q, int n, float last, float top, float &frac)
 {
     q = fminf(fmaxf(q, 0.f), last);
+    if constexpr (GENERAL) {
+        const int i = min((int)floorf(q), max(n - 2, 0));
+        frac = q - (float)i;
+        return i;
+    }
     const float f = fminf(__fadd_rd(q, kFloorMagic), top);
     frac = q - (f - kFloorMagic);
     return __float_as_int(f) - kFloorBits;
@@ -186,8 +194,8 @@ __device__ __forceinline__ float4 march_tf(const TFDev &tf, const MarchTable &ta
                        __fmaf_rn(t, c.w, a.w));
 }
 
-// SKIP: use the occupancy words.  GENERAL: any volume; otherwise every edge has
-// at least two voxels and the volume less than 2^30 (32-bit byte offsets).
+// SKIP: use the occupancy words.  GENERAL: any volume; otherwise every edge has 2
+// to kFloorMax voxels and the volume less than 2^30 (32-bit byte offsets).
 template <bool SKIP, bool GENERAL>
 __global__ void __launch_bounds__(kDvrThreads) k_dvr(const float *__restrict__ F, int nx, int ny, int nz,
                                              const __grid_constant__ TFDev tf, NoOpacity none,
@@ -217,6 +225,7 @@ __global__ void __launch_bounds__(kDvrThreads) k_dvr(const float *__restrict__ F
         d[k] *= inv_len;
         o[k] = -dot3(R[k], cam.t[0], R[3 + k], cam.t[1], R[6 + k], cam.t[2]);   // -R^T t
     }
+    const int n[3] = {nx, ny, nz};
     const float box[3] = {(float)nx, (float)ny, (float)nz};
     float t0 = 0.f, t1 = 3.4e38f;
     bool miss = false;
@@ -283,7 +292,7 @@ __global__ void __launch_bounds__(kDvrThreads) k_dvr(const float *__restrict__ F
 #pragma unroll
                 for (int k = 0; k < 3; k++) {
                     q[k] = __fadd_rn(__fmaf_rn(tm, d[k], o[k]), -0.5f);
-                    c[k] = cell_of(q[k], last[k], top[k], f) >> kCellShift;
+                    c[k] = cell_of<GENERAL>(q[k], n[k], last[k], top[k], f) >> kCellShift;
                 }
                 // samples from m on that lie in this block for certain
                 float leave = 1e6f;
@@ -307,9 +316,9 @@ __global__ void __launch_bounds__(kDvrThreads) k_dvr(const float *__restrict__ F
                 if (seg > 0.f) {
                     const float tm = __fmaf_rn(0.5f, seg, a0);
                     float fx, fy, fz;
-                    const int x = cell_of(__fadd_rn(__fmaf_rn(tm, d[0], o[0]), -0.5f), last[0], top[0], fx);
-                    const int y = cell_of(__fadd_rn(__fmaf_rn(tm, d[1], o[1]), -0.5f), last[1], top[1], fy);
-                    const int z = cell_of(__fadd_rn(__fmaf_rn(tm, d[2], o[2]), -0.5f), last[2], top[2], fz);
+                    const int x = cell_of<GENERAL>(__fadd_rn(__fmaf_rn(tm, d[0], o[0]), -0.5f), n[0], last[0], top[0], fx);
+                    const int y = cell_of<GENERAL>(__fadd_rn(__fmaf_rn(tm, d[1], o[1]), -0.5f), n[1], last[1], top[1], fy);
+                    const int z = cell_of<GENERAL>(__fadd_rn(__fmaf_rn(tm, d[2], o[2]), -0.5f), n[2], last[2], top[2], fz);
                     const float gx = 1.f - fx, gy = 1.f - fy;
                     float c00, c10, c01, c11;
                     if constexpr (GENERAL) {
@@ -394,6 +403,7 @@ vbm_status render_dvr(const float *F, const int dims[3], const vbm_tf *tf, const
     VBM_ARG(blocks <= INT_MAX, "image too large");
     dim3 grid((unsigned)blocks, 1, n_views);
     const bool general = std::min({dims[0], dims[1], dims[2]}) < 2 ||
+                         std::max({dims[0], dims[1], dims[2]}) > kFloorMax ||
                          (int64_t)dims[0] * dims[1] * dims[2] >= (int64_t)1 << 30;
     if (words) {
         k_occupancy<<<marks, kOccupancyThreads, 0, st>>>(F, dims[0], dims[1], dims[2], none, words);
