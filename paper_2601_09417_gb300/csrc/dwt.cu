@@ -553,7 +553,9 @@ vbm_status launch_z(ZArgs a, int channels, const Taps &w, const Magnitudes *mag,
                      a.dst_chan % 4 == 0 && a.dst_plane % 4 == 0 && a.dst_row % 4 == 0;
     const int64_t lanes = vec ? plane / 4 : plane;
     const int split = mag ? 1 : channels;                        // channels of different threads
-    a.pairs = pairs_per(a.k_end - a.k_begin, lanes * split, 64);
+    // a grid's second axis holds 65535 chunks: a volume long beyond that in z
+    // takes longer ones
+    a.pairs = std::max(pairs_per(a.k_end - a.k_begin, lanes * split, 64), (a.k_end - a.k_begin + 65534) / 65535);
     const int threads = z_threads(mag ? 4 : 1);
     dim3 grid((unsigned)((lanes + threads - 1) / threads),
               (unsigned)((a.k_end - a.k_begin + a.pairs - 1) / a.pairs), (unsigned)split);
