@@ -305,6 +305,8 @@ vbm_status vbm_raster_fwd(vbm_plan *p, const float *params, int64_t stride, cons
     p->last_view_count = vc;
     p->last_items = p->view_item_offset[vb + vc] - p->view_item_offset[vb];
     p->g_splat_clear = p->bwd_seen;   // the projection zeroes the items' splat-gradient records
+    s = capture_id(st, p->g_splat_capture);
+    if (s != VBM_OK) return s;
     p->bwd_queue_used = false;        // the binning zeroes the work-queue counters
     record_event(p->prof_ev[4], st);
     s = preprocess_fwd(p, params, stride, cams, vb, vc, st);

@@ -1085,10 +1085,19 @@ vbm_status raster_fwd(vbm_plan *p, int vb, int vc, const float bg[3], float *img
 vbm_status raster_bwd(vbm_plan *p, int vb, int vc, const float bg[3], const float *dimg, const float *dalpha,
                       cudaStream_t st)
 {
-    // the forward's projection zeroed the splat-gradient records (once the
-    // plan has run a backward); otherwise, and for a second backward of the
-    // same forward, they are cleared here
-    if (!p->g_splat_clear) VBM_CUDA(cudaMemsetAsync(p->g_splat, 0, sizeof(float) * kGradStride * p->last_items, st));
+    // The forward's projection zeroed the splat-gradient records (once the plan
+    // has run a backward); otherwise, and for a second backward of the same
+    // forward, they are cleared here.  So they are wherever the two need not run
+    // one after the other, once each: a captured backward without its forward in
+    // the same capture, an eager one after a captured forward, or on a plan whose
+    // captured backward may have been replayed in between.
+    unsigned long long capture;
+    const vbm_status s = capture_id(st, capture);
+    if (s != VBM_OK) return s;
+    const bool paired = capture == p->g_splat_capture && (capture != 0 || !p->bwd_captured);
+    if (!p->g_splat_clear || !paired)
+        VBM_CUDA(cudaMemsetAsync(p->g_splat, 0, sizeof(float) * kGradStride * p->last_items, st));
+    p->bwd_captured |= capture != 0;
     p->g_splat_clear = false;
     p->bwd_seen = true;
     VBM_RASTER_DISPATCH(launch_bwd, true, p, vb, vc, bg, dimg, dalpha, st)

@@ -425,6 +425,16 @@ int64_t pyramid_tmp_floats(const int dims[3]);
 vbm_status pyramid_from_volume(const float *volume, const int dims[3], const vbm_tf *tf, int levels, int wavelet,
                                float *A, float *tmp, float *v, const int64_t *voff, double *E, cudaStream_t st);
 
+// The stream capture that a call on st becomes part of (0: none).
+inline vbm_status capture_id(cudaStream_t st, unsigned long long &id)
+{
+    cudaStreamCaptureStatus status;
+    id = 0;
+    VBM_CUDA(cudaStreamGetCaptureInfo(st, &status, &id));
+    if (status == cudaStreamCaptureStatusNone) id = 0;
+    return VBM_OK;
+}
+
 // ---------------------------------------------------------------- binning
 // Work-queue counters of the compositing kernels (2), tile-group sizes and
 // cursors of the longest-first order (32 + 32), then the list-segment
@@ -493,7 +503,9 @@ struct vbm_plan {
     uint4 *place = nullptr;                  // [items] tile rectangle, listed-tile word, depth (placement record)
     float *g_splat = nullptr;               // [items][kGradStride]
     bool g_splat_clear = false;             // host: zeroed by the last forward, no backward since
+    unsigned long long g_splat_capture = 0; // host: that forward's stream capture (0: none, it ran at once)
     bool bwd_seen = false;                  // host: a backward has run on this plan
+    bool bwd_captured = false;              // host: a backward of this plan was recorded in a stream capture
     bool bwd_queue_used = false;            // host: a backward has taken its work queue and no projection
                                             // backward (or binning) has cleared the counter since
 
