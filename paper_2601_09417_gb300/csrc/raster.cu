@@ -61,7 +61,6 @@ constexpr float kNegLog2e = -kLog2e;           // scales B
 constexpr int kNV = 9;                         // gradient partials per (pixel, splat)
 constexpr int kWarps = 4;                      // warps per block
 constexpr int kRegionCols = 8, kRegionRows = 4;   // thread positions of a warp region
-constexpr int kFilledRegions = 32768;          // forward regions that keep every SM's warps busy several times over
 
 __device__ __forceinline__ float ex2_approx(float x)
 {
@@ -998,15 +997,15 @@ vbm_status launch_fwd(vbm_plan *p, int vb, int vc, const float bg[3], float *img
     // variants launched while that hook is set
     const bool eval = p->prof_n_eval != nullptr;
     int32_t *nc_out = p->n_contrib ? p->n_contrib : p->prof_n_contrib;
-    // two list entries at a time: their alphas are independent, which hides a
-    // step's latency where a thread has one pixel and the regions are too few
-    // to fill the chip (1 x 128^2: step 103 -> 98 us; 8 x 512^2, 65,536 regions:
-    // 786 -> 792), and pairs well with two pixels (1080p frame 619 -> 608 us)
-    constexpr int MORE = PPT <= 2 ? 2 : 1, FILLED = PPT == 2 ? 2 : 1;
-    const bool more = n_items_w < kFilledRegions;
+    // two list entries at a time, except with four pixels a thread: their alphas
+    // are independent, which hides a step's latency.  With one pixel a thread,
+    // step of one entry at a time against two: 1 x 256^2 264 -> 247, 4 x 512^2
+    // 497 -> 490, 8 x 512^2 790 -> 774 us (100,000 splats; of 20,000 and 300,000
+    // 1 to 9% less or the same at 2048 to 65,536 regions); with two, 1080p frame
+    // 619 -> 608 us.  Four at a time: 1 x 128^2 step 97 -> 104 us.
+    constexpr int UNROLL = PPT <= 2 ? 2 : 1;
     if (p->desc.flags & VBM_PLAN_PERSISTENT) {
-        auto kernel = eval ? k_raster_fwd<PPT, GL, true, true, 1>
-                           : more ? k_raster_fwd<PPT, GL, true, false, MORE> : k_raster_fwd<PPT, GL, true, false, FILLED>;
+        auto kernel = eval ? k_raster_fwd<PPT, GL, true, true, 1> : k_raster_fwd<PPT, GL, true, false, UNROLL>;
         const int grid = persistent_grid(kernel, n_items_w);
         kernel<<<grid, kWarps * 32, 0, st>>>(p->tile_order, p->tile_queue, n_items_w, nr, p->ranges, p->pair_item,
                                              p->rec, p->desc.width, p->desc.height, p->desc.tile_w, p->desc.tile_h,
@@ -1014,9 +1013,7 @@ vbm_status launch_fwd(vbm_plan *p, int vb, int vc, const float bg[3], float *img
                                              p->prof_n_eval, p->ckpt, p->seg_len ? p->ckpt_base : nullptr,
                                              p->seg_len);
     } else {
-        auto kernel = eval ? k_raster_fwd<PPT, GL, false, true, 1>
-                           : more ? k_raster_fwd<PPT, GL, false, false, MORE>
-                                  : k_raster_fwd<PPT, GL, false, false, FILLED>;
+        auto kernel = eval ? k_raster_fwd<PPT, GL, false, true, 1> : k_raster_fwd<PPT, GL, false, false, UNROLL>;
         kernel<<<(n_items_w + kWarps - 1) / kWarps, kWarps * 32, 0, st>>>(
             nullptr, nullptr, n_items_w, nr, p->ranges, p->pair_item, p->rec, p->desc.width, p->desc.height,
             p->desc.tile_w, p->desc.tile_h, p->TX, p->TY, vb, bg[0], bg[1], bg[2], img, alpha, p->T_final, nc_out,
