@@ -249,7 +249,8 @@ typedef struct {
     int32_t flags;
     int32_t pixels_per_thread;     /* 1, 2 or 4; 0 = the library's choice (2; 1 in the forward of a batch
                                       below 2^20 pixels) */
-    int32_t group_lanes;           /* 4, 8, 16 or 32 lanes per compositing group; 0 = the library's choice (8) */
+    int32_t group_lanes;           /* 4, 8, 16 or 32 lanes per compositing group; 0 = the library's choice (8;
+                                      16 in the backward of a batch with fewer than one item to four pixels) */
     int32_t segment_len;           /* the backward walks a tile list longer than
                                       this many entries as segments that different warps take at
                                       once (the forward stores each pixel's transmittance and

@@ -952,9 +952,19 @@ __global__ void __launch_bounds__(kWarps * 32)
 // the entries that miss their pixels (forward call of 1 x 128^2 / 8 x 512^2 /
 // 4 x 800^2 with 32 lanes 116 / 493 / 1008, with 8 105 / 431 / 880, with 4 105
 // / 434 / 874 us; segmented backward 48 / 419 / 842, 48 / 378 / 728, 51 / 414
-// / 788 us), and a thread two pixels, or one in the forward of a batch below
-// 2^20 pixels, which two would leave with too few warps (105 -> 96 us on 1 x
-// 128^2; 431 -> 460 us on 8 x 512^2).
+// / 788 us).  In the backward of a sparse batch, of fewer than one item to four
+// pixels, they have 16: its splats are wide, few entries miss a group, and each
+// group adds its own sums.  Step with 8 / 16 / 32 backward lanes: 0.003 items a
+// pixel (1 x 1024 x 1040, 3000 splats) 231 / 211 / 207, 0.05 (1 x 1000^2) 376 /
+// 351 / 353, 0.10 (8 x 1024^2) 1710 / 1690 / 1709, 0.19 (8 x 512^2) 602 / 600 /
+// 613, 0.29 (8 x 1024^2) 2619 / 2632 / 2726, 0.95 (the same) 5245 / 5368 / 5700
+// us; 8 throughout left the sparsest slower than whole walks by 32-lane groups
+// (217 us).
+//
+// A thread has two pixels, or one in the forward of a batch below 2^20 pixels,
+// which two would leave with too few warps (step with one / two: 1 x 128^2 96 /
+// 105, 2 x 512^2 of 300,000 splats 707 / 756, 1 x 1000^2 519 / 537, 4 x 512 x
+// 514 1084 / 1108, 5 x 512^2 1254 / 1241, 8 x 512^2 1793 / 1747 us).
 int pixels_per_thread(const vbm_plan *p, bool bwd = false)
 {
     const int th = p->desc.tile_h;
@@ -969,7 +979,8 @@ int pixels_per_thread(const vbm_plan *p, bool bwd = false)
 int group_lanes(const vbm_plan *p, bool bwd = false)
 {
     const int want = bwd && p->desc.bwd_group_lanes > 0 ? p->desc.bwd_group_lanes : p->desc.group_lanes;
-    return want > 0 ? want : 8;
+    const int64_t pixels = (int64_t)p->desc.n_views * p->desc.width * p->desc.height;
+    return want > 0 ? want : bwd && 4 * p->items_cap < pixels ? 16 : 8;
 }
 
 int regions_per_tile(const vbm_plan *p, int ppt)
