@@ -6,6 +6,7 @@
 #include <cstring>
 #include <string>
 
+#include "checkpoints.h"
 #include "vbm_internal.h"
 
 namespace vbm {
@@ -211,22 +212,21 @@ vbm_status vbm_plan_create(const vbm_plan_desc *d, vbm_plan **out)
     if (d->segment_len >= 0) {
         p->seg_len = d->segment_len ? d->segment_len : default_segment_len(pixels);
         const int64_t tile_px = (int64_t)d->tile_w * d->tile_h;
-        // boundary slots for about kCheckpointPairsPerItem pairs per item (the
-        // workloads list about two per item before fine-tuning shrinks the
-        // splats, fewer after), one final-state slot per tile in recompute
-        // plans; never more than the pair capacity can use or kCheckpointBytes
-        const bool rc = (d->flags & VBM_PLAN_RECOMPUTE) != 0;
-        const int64_t want = (kCheckpointPairsPerItem * items + p->seg_len - 1) / p->seg_len + (rc ? tiles : 0);
-        const int64_t usable = (pairs + p->seg_len - 1) / p->seg_len * (rc ? 2 : 1);
-        p->ckpt_cap = std::max<int64_t>(1, std::min({want, usable,
-                                                     kCheckpointBytes / (tile_px * (int64_t)sizeof(float4))}));
-        ALLOC(p->ckpt_base, tiles);
-        ALLOC(p->seg_units, 2 * p->ckpt_cap);
+        const bool persistent = (d->flags & VBM_PLAN_PERSISTENT) != 0;
+        size_t free_bytes = 0, total_bytes = 0;
+        if (s == VBM_OK && !persistent) {
+            const cudaError_t e = cudaMemGetInfo(&free_bytes, &total_bytes);
+            if (e != cudaSuccess) s = cuda_fail(e, "plan allocation");
+        }
+        p->ckpt_cap = checkpoint_slots(items, tiles, pairs, tile_px, p->seg_len, (d->flags & VBM_PLAN_RECOMPUTE) != 0,
+                                       checkpoint_bytes(persistent, (int64_t)free_bytes));
         const vbm_status before = s;
         ALLOC(p->ckpt, p->ckpt_cap * tile_px);
+        ALLOC(p->ckpt_base, tiles);
+        ALLOC(p->seg_units, 2 * p->ckpt_cap);
         // a plan that did not ask for persistence does without segments rather
         // than fail for their memory
-        if (before == VBM_OK && s == VBM_ERR_NOMEM && !(d->flags & VBM_PLAN_PERSISTENT)) {
+        if (before == VBM_OK && s == VBM_ERR_NOMEM && !persistent) {
             cudaGetLastError();
             s = VBM_OK;
             p->seg_len = 0;

@@ -460,8 +460,6 @@ constexpr int kQSegUnits = 66, kQSegTiles = 67, kQSegSlots = 68, kQSegCursor = 6
 // 116 / 126 us; of 8 x 512^2 and 4 x 800^2: 385 and 801 against 378 and 728
 // us, and their forward, which writes the checkpoints, 10% slower.
 inline int default_segment_len(int64_t pixels) { return pixels < (1 << 20) ? 64 : 256; }
-constexpr int64_t kCheckpointPairsPerItem = 2;
-constexpr int64_t kCheckpointBytes = 1ll << 30;
 
 // Scratch of the binning: per-chunk sums of the tile counts and the lists of
 // tiles too long for one warp's sort (mid-size from the front, the longest
