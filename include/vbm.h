@@ -164,7 +164,9 @@ VBM_API vbm_status vbm_tf_apply(const float *d_volume, int64_t n, const vbm_tf *
 VBM_API vbm_status vbm_dwt3d(float *d_data, int n_channels, const int dims[3], int levels, int wavelet,
                      float *d_tmp, void *stream);
 
-/* Workspace bytes vbm_build needs for a volume of dims and levels. */
+/* Workspace bytes vbm_build needs for a volume of dims and levels: 25 a voxel
+ * above 2^24 voxels (more of volumes with fewer than 54 planes), up to 36 a
+ * voxel below (604 MB at 256^3), and about 2 MB. */
 VBM_API vbm_status vbm_build_workspace_size(const int dims[3], int levels, size_t *bytes);
 
 /* Volume -> Gaussians (Sec. 4.1: F -> RF -> Phi -> G): TF, J-level DWT,
@@ -177,7 +179,7 @@ VBM_API vbm_status vbm_build_workspace_size(const int dims[3], int levels, size_
  * returned with *n_out = the required capacity.  If d_coef is not NULL the
  * coefficient pyramid is also copied there (float[4][nz][ny][nx]) and
  * d_keep (if not NULL) receives one byte per pyramid element (1 = kept).
- * Synchronises the stream (copies the subband energies and counts). */
+ * Synchronises the stream (copies the number kept). */
 VBM_API vbm_status vbm_build(const float *d_volume, const int dims[3], const vbm_tf *tf, const vbm_bank *bank,
                      const vbm_select *sel, float *d_params, int64_t capacity, int64_t *n_out,
                      float *d_coef, uint8_t *d_keep, void *d_ws, size_t ws_bytes, void *stream);
@@ -202,7 +204,7 @@ VBM_API vbm_status vbm_render_dvr_workspace_size(const int dims[3], size_t *byte
 
 /* vbm_render_dvr with scratch (d_ws, 4-byte aligned): the call first marks
  * the blocks of the volume that the transfer function leaves any opacity in
- * and its rays then pass over the others.  The images are the same; nothing
+ * and its rays then pass over the others.  The images are the same bits; nothing
  * is kept in d_ws between calls.  d_ws NULL: vbm_render_dvr. */
 VBM_API vbm_status vbm_render_dvr_ws(const float *d_volume, const int dims[3], const vbm_tf *tf,
                              const vbm_camera *d_cams, int n_views, int width, int height, float step,

@@ -11,13 +11,14 @@
 //   keep = v >= max(T, v_(K')) and v > 0.
 // Kept coefficients are marked in a bit mask (raster order of each subband),
 // whose counts are scanned, and mapped chunk by chunk to the P[14][capacity]
-// layout.  The host waits once, for the number kept.  One launch a pass over
-// all bands (10 launches) instead of about 50 a band, and a map over the whole
-// chip instead of one block a band (which took 350 ms on a 512^3 volume):
-// vbm_build of 32^3 / 224 x 160 x 96 / 512^3 volumes 5.5 -> 0.33, 18.8 -> 1.38,
-// 390 -> 36.3 ms, the rest mostly the DWT.
+// layout.  The host waits for the number kept and for the end.  One launch a
+// pass over all bands (one where every band is small, else six, and two for the
+// marking and the map) instead of about 50 a band, and a map over the whole chip
+// instead of one block a band (which took 350 ms on a 512^3 volume): with the
+// DWT's kernels, vbm_build of 32^3 / 224 x 160 x 96 / 512^3 volumes 5.5 -> 0.13,
+// 18.9 -> 0.34, 390 -> 3.9 ms (selection passes 0.09 of the second, 0.63 of the
+// third).
 #include <cmath>
-#include <map>
 #include <vector>
 
 #include "vbm_internal.h"
@@ -610,9 +611,9 @@ std::vector<Band> bands_of(const int dims[3], int levels)
 }
 
 // Element offsets, marking chunks and selection blocks of the bands.  Bands of
-// at most kSmallBand elements have no blocks in the selection passes (one block
-// of the first launch takes all of theirs); of the others a block takes at least 8192
-// elements, and beyond that the blocks are two to an SM, shared out by band
+// at most kSmallBand elements have no blocks in the selection passes (a block of
+// the first launch runs all passes of one); of the others a block takes at least
+// 8192 elements, and beyond that the blocks are two to an SM, shared out by band
 // size.
 BandTab band_table(const std::vector<Band> &bands, double beta_N)
 {

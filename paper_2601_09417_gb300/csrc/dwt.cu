@@ -11,8 +11,8 @@
 // the transfer function where the rows are staged, so the four RGBA channels
 // are never stored untransformed.  Against one gather kernel an axis (a 64-bit
 // division and a modulo for every tap, three reads and writes of each value):
-// tf_apply + four-level dwt3d of 4 x 256^3, 4.30 -> 0.39 ms; vbm_build of a
-// 512^3 volume, 36.3 -> 4.6 ms.
+// tf_apply + four-level dwt3d of 4 x 256^3, 4.30 -> 0.32 ms; vbm_build of a
+// 512^3 volume, 36.3 -> 3.9 ms.
 #include "tf_dev.h"
 
 namespace vbm {
@@ -79,7 +79,8 @@ enum Source { kScalar, kQuads, kTransfer };
 // by the arithmetic itself (4 x 256^3, all levels: 200 -> 170 us; with the
 // transfer function on 512^3, first level: 2.76 -> 1.63 ms).  A slot lies in
 // one warp, so that only the transfer function's four need a block barrier
-// (slots of 64 threads and barriers for all: 4 x 256^3 pyramid 395 -> 367 us).
+// (with slots of 64 threads and barriers for all the 4 x 256^3 pyramid took 395
+// us instead of 367, before the z pass's asynchronous copies below).
 //
 // kTransfer: the source is the scalar volume; four neighbouring slots take the
 // four channels of one strip, whose threads share the loads and the transfer
@@ -379,7 +380,8 @@ __global__ void __launch_bounds__(z_threads(NC), NC == 4 ? 5 : 3) k_dwt_z(const 
     // plane pairs on their way: copied asynchronously into the thread's own
     // shared-memory words, so that the depth costs no registers (one pair ahead
     // in registers left too few bytes in flight: 4 x 256^3 pyramid 395 -> 354
-    // us, vbm_build of 512^3 4.27 -> 4.07 ms)
+    // us, with the slots within a warp above 327; vbm_build of 512^3 4.27 -> 4.07
+    // ms)
     __shared__ T stage[kZDepth][2][NC][THREADS];
     int t = wrap(2 * k0 + Wv::FIRST - a.z_first, a.planes);
     float ring[R][2][NC * V];
@@ -699,9 +701,12 @@ vbm_status dwt_channels(float *data, int n_channels, const int dims[3], int leve
 }
 
 // Floats of tmp for pyramid_from_volume: the four channels whole up to 2^26
-// floats (256^3 volumes); beyond that 1.2 volumes, worked in slabs, which with
-// the magnitudes keeps vbm_build's scratch at 25 bytes a voxel.  At least
-// half of the volume (the second level's four channels) and 16 planes.
+// floats (256^3 volumes), which makes vbm_build's scratch 36 bytes a voxel there
+// (604 MB at most); beyond that 1.2 volumes, worked in slabs, and 25 bytes.  Slabs
+// of 1.2 volumes throughout would keep 25 bytes everywhere and make vbm_build of
+// 128^3 / 224 x 160 x 96 / 256^3 take 336 / 460 / 750 us instead of 291 / 336 /
+// 645.  At least half of the volume (the second level's four channels) and 16
+// planes.
 int64_t pyramid_tmp_floats(const int dims[3])
 {
     const int64_t n = (int64_t)dims[0] * dims[1] * dims[2], plane = (int64_t)dims[0] * dims[1];

@@ -458,7 +458,12 @@ constexpr int kQSegUnits = 66, kQSegTiles = 67, kQSegSlots = 68, kQSegCursor = 6
 // lists, so it splits finer: backward of 1 x 128^2 / 3 x 509 x 347 / 4 x 256^2
 // at 16 x 16 tiles with segments of 64 against 256: 48 / 65 / 75 against 85 /
 // 116 / 126 us; of 8 x 512^2 and 4 x 800^2: 385 and 801 against 378 and 728
-// us, and their forward, which writes the checkpoints, 10% slower.
+// us, and their forward, which writes the checkpoints, 10% slower.  The line is
+// a compromise: with few splats 64 stays ahead beyond it and with many 256 is
+// ahead below it.  Step with 64 / 256: 20,000 splats on 1 x 512^2 146 / 200, 4 x
+// 512 x 510 288 / 316, 6 x 512^2 364 / 376; 100,000 on the same 230 / 262, 549 /
+// 547, 735 / 713; 1,000,000 1413 / 1287, 3216 / 2668, 4622 / 3740 us (whole
+// walks by 32-lane groups: 273, 455, 552; 648, 1116, 1276; 4041, 5650, 6817).
 inline int default_segment_len(int64_t pixels) { return pixels < (1 << 20) ? 64 : 256; }
 
 // Scratch of the binning: per-chunk sums of the tile counts and the lists of
