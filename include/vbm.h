@@ -259,11 +259,11 @@ typedef struct {
                                       colour still to come at every segment boundary, and with
                                       VBM_PLAN_RECOMPUTE the tile's final per-pixel state; the
                                       plan holds checkpoints for about 2 pairs per (view, Gaussian)
-                                      item, at most 1 GiB, and without VBM_PLAN_PERSISTENT at most
+                                      item (more where the library has chosen 64), at most 1 GiB, and without VBM_PLAN_PERSISTENT at most
                                       a 16th of the memory free at its creation; tiles beyond that
                                       are walked whole).  0 = the library's choice (256; 64 for a
-                                      batch below 2^20 pixels); a positive multiple of 32 up to
-                                      65536; -1 = never split, no such memory (a plan that only
+                                      batch below 2^20 pixels, fewer than eight items a pixel);
+                                      a positive multiple of 32 up to 65536; -1 = never split, no such memory (a plan that only
                                       renders needs none).  A plan that is not persistent does
                                       without segments when their memory cannot be had.  Results
                                       equal the unsplit walk's up to FP32 rounding of the

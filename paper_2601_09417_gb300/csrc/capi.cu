@@ -210,7 +210,7 @@ vbm_status vbm_plan_create(const vbm_plan_desc *d, vbm_plan **out)
     ALLOC(p->d_status, 2);
     ALLOC(p->d_bias, 1);
     if (d->segment_len >= 0) {
-        p->seg_len = d->segment_len ? d->segment_len : default_segment_len(pixels);
+        p->seg_len = d->segment_len ? d->segment_len : default_segment_len(pixels, items);
         const int64_t tile_px = (int64_t)d->tile_w * d->tile_h;
         const bool persistent = (d->flags & VBM_PLAN_PERSISTENT) != 0;
         size_t free_bytes = 0, total_bytes = 0;
@@ -219,7 +219,8 @@ vbm_status vbm_plan_create(const vbm_plan_desc *d, vbm_plan **out)
             if (e != cudaSuccess) s = cuda_fail(e, "plan allocation");
         }
         p->ckpt_cap = checkpoint_slots(items, tiles, pairs, tile_px, p->seg_len, (d->flags & VBM_PLAN_RECOMPUTE) != 0,
-                                       checkpoint_bytes(persistent, (int64_t)free_bytes));
+                                       checkpoint_bytes(persistent, (int64_t)free_bytes),
+                                       d->segment_len == 0 && fine_segments(pixels, items));
         const vbm_status before = s;
         ALLOC(p->ckpt, p->ckpt_cap * tile_px);
         ALLOC(p->ckpt_base, tiles);

@@ -452,19 +452,21 @@ constexpr int kQSegUnits = 66, kQSegTiles = 67, kQSegSlots = 68, kQSegCursor = 6
 // (transmittance, last contributor) in one more slot, so the backward replays
 // only the short lists.  Checkpoint memory is bounded; tiles that find no
 // free slot are walked whole.
-// Segment length of a plan that leaves it to the library, by the pixels of its
-// batch.  A batch of fewer than 2^20 pixels (16384 warp regions of 64, about
-// four to a resident warp of the backward) does not fill the chip with whole
-// lists, so it splits finer: backward of 1 x 128^2 / 3 x 509 x 347 / 4 x 256^2
-// at 16 x 16 tiles with segments of 64 against 256: 48 / 65 / 75 against 85 /
-// 116 / 126 us; of 8 x 512^2 and 4 x 800^2: 385 and 801 against 378 and 728
-// us, and their forward, which writes the checkpoints, 10% slower.  The line is
-// a compromise: with few splats 64 stays ahead beyond it and with many 256 is
-// ahead below it.  Step with 64 / 256: 20,000 splats on 1 x 512^2 146 / 200, 4 x
-// 512 x 510 288 / 316, 6 x 512^2 364 / 376; 100,000 on the same 230 / 262, 549 /
-// 547, 735 / 713; 1,000,000 1413 / 1287, 3216 / 2668, 4622 / 3740 us (whole
-// walks by 32-lane groups: 273, 455, 552; 648, 1116, 1276; 4041, 5650, 6817).
-inline int default_segment_len(int64_t pixels) { return pixels < (1 << 20) ? 64 : 256; }
+// Segment length of a plan that leaves it to the library.  A batch of fewer than
+// 2^20 pixels (16384 warp regions of 64, about four to a resident warp of the
+// backward) does not fill the chip with long units, so it splits finer: step
+// with segments of 64 / 256, 16 x 16 tiles: 3000 splats on 1 x 128^2 90 / 121, on
+// 1 x 512^2 112 / 147, 20,000 on 1 x 1000^2 228 / 275, on 4 x 512 x 510 285 / 314,
+// 100,000 on 1 x 512^2 230 / 261 us; 8 x 8 tiles 285 / 367 and 235 / 331 of the
+// last two.  More than eight items a pixel make every list long: 100,000 on 1 x
+// 100 x 80 1434 / 1263, 400,000 on 1 x 200 x 150 2322 / 2003 (8 x 8 tiles 1371 /
+// 1277), 2,000,000 on 1 x 64^2 33,300 / 27,400 us (17,400 / 15,600).  Between, 16 x
+// 16 tiles lose and 8 x 8 tiles gain (250,000 on 3 x 512^2 850 / 796 and 603 /
+// 639; 20,000 on 1 x 64^2 396 / 380 and 305 / 323).  Beyond 2^20 pixels few splats would still gain (20,000 on 8 x 512^2 430
+// / 442), many lose, and the forward, which writes the checkpoints, takes 10%
+// longer (8 x 512^2, 4 x 800^2).
+inline bool fine_segments(int64_t pixels, int64_t items) { return pixels < (1 << 20) && items < 8 * pixels; }
+inline int default_segment_len(int64_t pixels, int64_t items) { return fine_segments(pixels, items) ? 64 : 256; }
 
 // Scratch of the binning: per-chunk sums of the tile counts and the lists of
 // tiles too long for one warp's sort (mid-size from the front, the longest
