@@ -62,8 +62,13 @@ NoOpacity no_opacity(const vbm_tf *tf)
 // which an interpolation can overflow: infinity times a weight of 0 is NaN and
 // reads as the scalar 0.  (Below lo nothing need be excluded: a bound there
 // means that 0 has no opacity either.)
+//
+// HIGH: the transfer function has an upper bound.  One that is opaque at its last
+// knot has none, and its voxels take one comparison: the kernel is bound by
+// their issue (image of 512^2 of 512^3 at a step of 1, 608 -> 592 us in all).
 constexpr float kMarkMax = 1e38f;
 
+template <bool HIGH>
 __global__ void __launch_bounds__(kOccupancyThreads) k_occupancy(const float *__restrict__ F, int nx, int ny, int nz,
                                                                  NoOpacity none, uint32_t *__restrict__ words)
 {
@@ -71,7 +76,7 @@ __global__ void __launch_bounds__(kOccupancyThreads) k_occupancy(const float *__
     const int x = blockIdx.x * kOccupancyCols + threadIdx.x;
     const int y0 = blockIdx.y * kCell, z0 = blockIdx.z * kCell;
     if (threadIdx.x <= kOccupancyCols) {
-        bool lo = true, hi = true;
+        bool lo = true, hi = HIGH;
         if (x < nx) {
             for (int z = z0; z <= min(z0 + kCell, nz - 1); z++) {
                 const float *row = F + ((int64_t)z * ny + y0) * nx + x;
@@ -81,7 +86,7 @@ __global__ void __launch_bounds__(kOccupancyThreads) k_occupancy(const float *__
 #pragma unroll
                 for (int k = 0; k <= kCell; k++) {
                     lo &= v[k] <= none.lo;
-                    hi &= v[k] >= none.hi && v[k] < kMarkMax;
+                    if (HIGH) hi &= v[k] >= none.hi && v[k] < kMarkMax;
                 }
             }
         }
@@ -407,7 +412,8 @@ vbm_status render_dvr(const float *F, const int dims[3], const vbm_tf *tf, const
                          std::max({dims[0], dims[1], dims[2]}) > kFloorMax ||
                          (int64_t)dims[0] * dims[1] * dims[2] >= (int64_t)1 << 30;
     if (words) {
-        k_occupancy<<<marks, kOccupancyThreads, 0, st>>>(F, dims[0], dims[1], dims[2], none, words);
+        auto occupancy = none.hi == none.hi ? k_occupancy<true> : k_occupancy<false>;
+        occupancy<<<marks, kOccupancyThreads, 0, st>>>(F, dims[0], dims[1], dims[2], none, words);
         VBM_LAUNCH("occupancy");
         note_launches(1);
     }
