@@ -205,7 +205,9 @@ VBM_API vbm_status vbm_render_dvr_workspace_size(const int dims[3], size_t *byte
 /* vbm_render_dvr with scratch (d_ws, 4-byte aligned): the call first marks
  * the blocks of the volume that the transfer function leaves any opacity in
  * and its rays then pass over the others.  The images are the same bits; nothing
- * is kept in d_ws between calls.  d_ws NULL: vbm_render_dvr. */
+ * is kept in d_ws between calls.  d_ws NULL: vbm_render_dvr, which is faster for
+ * calls of few samples (below about 40 M: 1 x 100^2 of 256^3 164 us against 249;
+ * 8 x 512^2 of 128^3 767 against 425). */
 VBM_API vbm_status vbm_render_dvr_ws(const float *d_volume, const int dims[3], const vbm_tf *tf,
                              const vbm_camera *d_cams, int n_views, int width, int height, float step,
                              float *d_rgba, void *d_ws, size_t ws_bytes, void *stream);

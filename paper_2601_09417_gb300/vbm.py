@@ -254,12 +254,26 @@ def build(volume, dims, tf, bank, sel, capacity, coef=None, keep=None):
     return params, n.value
 
 
+def dvr_marks_pay(dims, n_views, width, height, step):
+    """Whether the occupancy marks save a call's rays more than they cost: from about 40 M samples on
+    (rays times the volume's mean chord), in volumes of more than 2^16 voxels, or where a ray alone has
+    thousands.  With / without: 1 x 100^2 of 256^3 249 / 164 us, 5 x 326 x 247 of 45 x 121 x 53 91 / 64,
+    5 x 265 x 190 of 38 x 149 x 156 184 / 166 (26 M samples); 2 x 300 x 200 of 512^3 670 / 712 (41 M),
+    1 x 512^2 of 128^3 157 / 178 (45 M), 2 x 400^2 of 350^3 380 / 717 (75 M); 8 x 512^2 of 32^3 190 / 155."""
+    nx, ny, nz = (int(d) for d in dims)
+    if min(nx, ny, nz) <= 0 or not step > 0 or nx + ny + nz > 4096 * step:
+        return True
+    chord = 2.0 * nx * ny * nz / (nx * ny + ny * nz + nz * nx)
+    return nx * ny * nz > 1 << 16 and n_views * width * height * chord >= 40e6 * step
+
+
 def render_dvr(volume, dims, tf, cams_dev, n_views, width, height, step, out):
-    import torch
     lib = load()
-    size = ctypes.c_size_t()
-    _check(lib.vbm_render_dvr_workspace_size(_dims(dims), ctypes.byref(size)))
-    ws = torch.empty(size.value, dtype=torch.uint8, device="cuda")
+    ws, size = None, ctypes.c_size_t()
+    if dvr_marks_pay(dims, n_views, width, height, step):
+        import torch
+        _check(lib.vbm_render_dvr_workspace_size(_dims(dims), ctypes.byref(size)))
+        ws = torch.empty(size.value, dtype=torch.uint8, device="cuda")
     _check(lib.vbm_render_dvr_ws(_ptr(volume), _dims(dims), ctypes.byref(tf), _ptr(cams_dev), n_views, width,
                                  height, float(step), _ptr(out), _ptr(ws), size.value, _stream()))
 
