@@ -235,16 +235,10 @@ __global__ void __launch_bounds__(kDvrThreads) k_dvr(const float *__restrict__ F
     const float box[3] = {(float)nx, (float)ny, (float)nz};
     float t0 = 0.f, t1 = 3.4e38f;
     bool miss = false;
-    // Steps per axis to a block's face: (8 c + face[k] - q[k]) inv_d[k] from the
-    // position q in block c.  A ray that does not move along an axis leaves the
-    // block through neither face: it looks at the one ahead of its q, infinitely
-    // far (a face at or behind q sent such a ray's empty space through the
-    // occupancy words sample by sample: 65536 x 16 x 16 at a step of 0.05, 200 ->
-    // 1.3 ms).
-    float inv_d[3], face[3];
+    float inv_d[3];
 #pragma unroll
     for (int k = 0; k < 3; k++) {
-        inv_d[k] = o[k] - 0.5f > fmaxf(box[k] - 2.f, 0.f) ? -1e30f : 1e30f;
+        inv_d[k] = 0.f;
         if (d[k] != 0.f) {
             const float inv = 1.f / d[k];
             inv_d[k] = inv;
@@ -254,22 +248,36 @@ __global__ void __launch_bounds__(kDvrThreads) k_dvr(const float *__restrict__ F
         } else if (o[k] < 0.f || o[k] > box[k]) {
             miss = true;
         }
-        face[k] = inv_d[k] > 0.f ? (float)kCell : 0.f;
     }
-    // The face is taken this much too near, so that the samples up to it lie in
-    // the block as their positions round.  A position is the float32 of o + tm d
-    // - 1/2 with tm the float32 of t0 + (m + 1/2) step: two samples' positions
-    // differ from the exact multiple of the step by at most 6 2^-24 (t1 + n)
-    // together (three roundings up to t1 and two up to n voxels for each), and
-    // 1e-5 covers the distance's own.  Towards the face they come in order, so
-    // none falls back behind the block's other faces.
-    const float margin = __fmaf_rn(0x1p-21f, t1 + fmaxf(fmaxf(box[0], box[1]), box[2]), 1e-5f);
-#pragma unroll
-    for (int k = 0; k < 3; k++)
-        if (d[k] != 0.f) face[k] -= copysignf(margin, d[k]);
     float C0 = 0.f, C1 = 0.f, C2 = 0.f, T = 1.f;
     const bool hit = inside && !miss && t1 > t0;
     const int nseg = hit ? (int)ceilf((t1 - t0) / step) : 0;
+    // Distance along the ray to a block's face: (8 c + face[k] - q[k]) inv_d[k] from
+    // the position q in block c.  The face is taken `margin` too near, so that the
+    // samples up to it lie in the block as their positions round.  A position is
+    // the float32 of o + tm d - 1/2 with tm the float32 of t0 + (m + 1/2) step: two
+    // samples' positions differ from the exact multiple of the step by at most 6
+    // 2^-24 (t1 + n) together (three roundings up to t1 and two up to n voxels for
+    // each), and 1e-5 covers the distance's own.  Towards the face they come in
+    // order, so none falls back behind the block's other faces.
+    // A ray that does not move along an axis leaves the block through neither
+    // face: it looks at the one ahead of its q, infinitely far (a face at or behind
+    // q sent such a ray's empty space through the occupancy words sample by
+    // sample: 65536 x 16 x 16 at a step of 0.05, 200 -> 1.3 ms).
+    float face[3] = {0.f, 0.f, 0.f};
+    if (SKIP && nseg > 0) {
+        const float margin = __fmaf_rn(0x1p-21f, t1 + fmaxf(fmaxf(box[0], box[1]), box[2]), 1e-5f);
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            if (d[k] != 0.f) {
+                face[k] = d[k] > 0.f ? (float)kCell - margin : margin;
+            } else {
+                const bool up = o[k] - 0.5f <= fmaxf(box[k] - 2.f, 0.f);
+                inv_d[k] = up ? 1e30f : -1e30f;
+                face[k] = up ? (float)kCell : 0.f;
+            }
+        }
+    }
     const float last[3] = {(float)(nx - 1), (float)(ny - 1), (float)(nz - 1)};
     // a cell's upper corner exists: the lower one is at most n - 2 (0 where n = 1)
     const float top[3] = {kFloorMagic + (float)max(nx - 2, 0), kFloorMagic + (float)max(ny - 2, 0),

@@ -256,12 +256,14 @@ def build(volume, dims, tf, bank, sel, capacity, coef=None, keep=None):
 
 def dvr_marks_pay(dims, n_views, width, height, step):
     """Whether the occupancy marks save a call's rays more than they cost: from about 40 M samples on
-    (rays times the volume's mean chord), in volumes of more than 2^16 voxels, or where a ray alone has
-    thousands.  With / without: 1 x 100^2 of 256^3 249 / 164 us, 5 x 326 x 247 of 45 x 121 x 53 91 / 64,
-    5 x 265 x 190 of 38 x 149 x 156 184 / 166 (26 M samples); 2 x 300 x 200 of 512^3 670 / 712 (41 M),
-    1 x 512^2 of 128^3 157 / 178 (45 M), 2 x 400^2 of 350^3 380 / 717 (75 M); 8 x 512^2 of 32^3 190 / 155."""
+    (rays times the volume's mean chord) in volumes of more than 2^16 voxels, and where an edge alone
+    has more than 512 samples, whose latency a few rays do not hide.  With / without: 1 x 100^2 of 256^3
+    249 / 164 us, 5 x 326 x 247 of 45 x 121 x 53 91 / 64, 5 x 265 x 190 of 38 x 149 x 156 184 / 166 (26 M
+    samples); 2 x 300 x 200 of 512^3 670 / 712 (41 M), 1 x 512^2 of 128^3 157 / 178 (45 M), 2 x 400^2 of
+    350^3 380 / 717 (75 M); 8 x 512^2 of 32^3 190 / 155; 6 x 136 x 65 of 39 x 433 x 291 at a step of 0.5
+    383 / 425."""
     nx, ny, nz = (int(d) for d in dims)
-    if min(nx, ny, nz) <= 0 or not step > 0 or nx + ny + nz > 4096 * step:
+    if min(nx, ny, nz) <= 0 or not step > 0 or max(nx, ny, nz) > 512 * step:
         return True
     chord = 2.0 * nx * ny * nz / (nx * ny + ny * nz + nz * nx)
     return nx * ny * nz > 1 << 16 and n_views * width * height * chord >= 40e6 * step
