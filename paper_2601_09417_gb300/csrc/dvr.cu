@@ -18,7 +18,7 @@
 // bit for bit.  The marks cost one read of the volume (98 us of 512^3).  Blocks of
 // 8^3: with 4^3 a ray asks twice as often for a sixth fewer samples (8 x 1024^2
 // of 512^3 8.07 -> 8.83 ms, 8 x 512^2 of 128^3 489 -> 553 us).  All together
-// against the full march in 16 x 16 blocks: 21.6 -> 6.4 ms and 1144 -> 413 us.
+// against the full march in 16 x 16 blocks: 21.3 -> 6.0 ms and 1152 -> 410 us.
 #include "tf_dev.h"
 
 namespace vbm {

@@ -955,8 +955,8 @@ __global__ void __launch_bounds__(kWarps * 32)
 // / 788 us).  In the backward of a sparse batch, of fewer than one item to four
 // pixels, they have 16: its splats are wide, few entries miss a group, and each
 // group adds its own sums.  Step with 8 / 16 / 32 backward lanes: 0.003 items a
-// pixel (1 x 1024 x 1040, 3000 splats) 231 / 211 / 207, 0.05 (1 x 1000^2) 376 /
-// 351 / 353, 0.10 (8 x 1024^2) 1710 / 1690 / 1709, 0.19 (8 x 512^2) 602 / 600 /
+// pixel (1 x 1024 x 1040, 3000 splats) 231 / 211 / 207, 0.05 (1 x 1000^2) 277 /
+// 272 / 271, 0.10 (8 x 1024^2) 1710 / 1690 / 1709, 0.19 (8 x 512^2) 602 / 600 /
 // 613, 0.29 (8 x 1024^2) 2619 / 2632 / 2726, 0.95 (the same) 5245 / 5368 / 5700
 // us; 8 throughout left the sparsest slower than whole walks by 32-lane groups
 // (217 us).
